@@ -22,6 +22,8 @@
 #include <vector>
 
 #include "flups_gpu.h"
+#include "fx64.cuh"
+#include "fx_plan.cuh"
 #include "green.cuh"
 #include "passes.cuh"
 
@@ -144,7 +146,9 @@ struct flups_solver_s {
   void* W1 = nullptr;
   void* W2 = nullptr;
   void* green_dev = nullptr;
+  int* green_exp = nullptr;     // fixed-point spectrum: exponent of each pencil's slice
   int green_pitch = 0;          // x pitch (elements) of the stored spectrum
+  bool fx = false;              // passes in 64-bit fixed point (FP64-class Poisson solves)
   bool share_green = false;     // look the stored spectrum up in (and add it to) the process-wide cache
   std::string green_key;        // its cache key when shared
   void* gmaps_dev = nullptr;    // TMA tensor maps of the stored spectrum (fused column pass)
@@ -206,6 +210,26 @@ static int make_twiddles_uncached(int P, int prec, void** out) {
   return FLUPS_OK;
 }
 
+// Twiddles of the fixed-point passes, exp(-2 pi i m/(2P)) 2^60 in signed 32-bit halves (fx64.cuh).
+constexpr int kFxTables = 3;  // their key beside the precisions
+int make_twiddles_fx(int P, void** out) {
+  const int M = 2 * P;
+  std::vector<int> h((size_t)4 * M);
+  for (int m = 0; m < M; ++m) {
+    const long double a = 3.141592653589793238462643383279502884L * (long double)m / (long double)P;
+    const long long c = llroundl(ldexpl(cosl(a), kFxTwBits)), sn = llroundl(ldexpl(-sinl(a), kFxTwBits));
+    h[4 * m] = fx_hi(c);
+    h[4 * m + 1] = fx_lo(c);
+    h[4 * m + 2] = fx_hi(sn);
+    h[4 * m + 3] = fx_lo(sn);
+  }
+  void* d = nullptr;
+  CK(cudaMalloc(&d, (size_t)M * 16));
+  CK(cudaMemcpy(d, h.data(), (size_t)M * 16, cudaMemcpyHostToDevice));
+  *out = d;
+  return FLUPS_OK;
+}
+
 // Twiddle tables are shared by every plan of a process: one table per (device,
 // P, precision), created on first use and kept until exit (a few KB each), so
 // that plan setup and teardown allocate and free no twiddles.
@@ -223,7 +247,7 @@ int make_twiddles(int P, int prec, void** out) {
     return FLUPS_OK;
   }
   void* d = nullptr;
-  const int rc = make_twiddles_uncached(P, prec, &d);
+  const int rc = prec == kFxTables ? make_twiddles_fx(P, &d) : make_twiddles_uncached(P, prec, &d);
   if (rc) return rc;
   g_tw_cache[key] = d;
   *out = d;
@@ -409,6 +433,43 @@ void fill_geom(Launch& L, const DirPlan& dp, int axis, const int* din, const int
   }
 }
 
+// Tile of a fixed-point pass (after fill_geom): about 2048 complex values per CTA (32 KB, 128-192 threads of
+// up to 128 registers, so that four CTAs share an SM), 4096 in the fused complex pass, whose code is the
+// longest: warps of one CTA run the same stretch of it and share its instruction fetches (unbounded 128^3
+// 197 -> 186 us, 192^3 895 -> 840; the other passes 0-8% slower with 4096, all 10-30% slower with 8192).  At
+// least 4 lanes (64 contiguous bytes along x) up to P = 1024; narrower when the grid would leave SMs idle.
+void fx_geom(Launch& L, int axis, bool packed) {
+  PassParams& p = L.p;
+  const int P = p.P, target = L.kind == K_FUSED_C2C ? 4096 : 2048;
+  int W = 1;
+  while (W < 32 && 2 * W * P <= target) W *= 2;
+  const int wmin = P <= 1024 ? 4 : (P <= 2048 ? 2 : 1);
+  if (W < wmin) W = wmin;
+  const int need = packed ? (p.npen + 1) / 2 : p.npen;
+  while (W > 1 && W / 2 >= need) W /= 2;
+  auto ctas = [&](int w) { return (long long)((need + w - 1) / w) * L.grid.y * L.grid.z; };
+  while (W > 1 && ctas(W) < 2 * 152 && W * P >= 512) W /= 2;
+  // every stage's butterflies and every item loop fit: P W / ept threads, ept <= 18; a small grid takes a thread
+  // per four values instead, one butterfly each
+  const int ept = fx_ept(P);
+  int nt = (P * W + ept - 1) / ept;
+  if (ctas(W) * nt < 152 * 256) nt = std::max(nt, std::min(256, P * W / 4));
+  nt = std::max(32, (nt + 31) / 32 * 32);
+  p.W = W;
+  p.lw = ilog2(W);
+  p.LS = W == 1 ? 1 : W + 1;
+  p.fx = 1;
+  p.ct = 0;
+  p.hz = 0;
+  p.ept = 0;
+  L.grid.x = (unsigned)((need + W - 1) / W);
+  L.nthr = nt;
+  // alignment, mbarrier block, tile, Green offsets and exponents, lane exponents, renormalisation words
+  L.smem = 128 + 128 + (size_t)P * p.LS * 16 + (size_t)W * (2 * 8 + 4 + 2 * 4 + kFxSlots * 4);
+  p.rowx = (axis == 0 && p.center == C_CELL && (p.type == T_PER || p.type == T_UNB) &&
+            (L.kind == K_FWD_REAL || L.kind == K_INV_REAL)) ? 1 : 0;
+}
+
 // CTAs per SM the compile-time kernels are built for (their __launch_bounds__ minimum).
 int ct_min_blocks(const PassParams& p, int nthr, int prec) {
   nthr = std::max(nthr, 32);  // a CTA narrower than a warp holds a whole warp
@@ -444,6 +505,18 @@ cudaError_t sample_green(const flups_solver_s* s, const GreenSampleParams& q, do
   return (s->green == FLUPS_LGF2) ? launch_lgf(g64, q.gext, q.h, st) : launch_green_sample(g64, q, st);
 }
 
+// The spectrum g64 times scale into green_dev, in the passes' format.
+cudaError_t store_green(flups_solver_s* s, const double* g64, const int* gext, double scale, cudaStream_t st) {
+  const long long n = (long long)gext[0] * gext[1] * gext[2];
+  if (!s->fx) return launch_green_finalize(g64, s->green_dev, s->topo.prec, n, gext[0], s->green_pitch, scale, st);
+  const int ax = s->order[2];
+  const size_t bytes = (size_t)(n / gext[ax]) * sizeof(int);
+  cudaError_t e = cudaMallocAsync((void**)&s->green_exp, bytes, st);
+  if (e) return e;
+  s->ws_bytes += bytes;
+  return launch_green_finalize_fx(g64, s->green_dev, s->green_exp, gext, s->green_pitch, ax, scale, !s->cplx[2], st);
+}
+
 int setup_green_compute(flups_solver_s* s, cudaStream_t st) {
   const int prec = s->topo.prec;
   int du = 0;
@@ -476,8 +549,8 @@ int setup_green_compute(flups_solver_s* s, cudaStream_t st) {
       }
       s->ws_bytes += bytes;
     }
-    if (prec == FLUPS_F64E) {
-      // the double-float path reads a stored spectrum: evaluate the closed form in FP64 once
+    if (prec == FLUPS_F64E || s->fx) {
+      // these passes read a stored spectrum: evaluate the closed form in FP64 once
       int gext[3];
       long long n = 1;
       for (int d = 0; d < 3; ++d) {
@@ -491,7 +564,7 @@ int setup_green_compute(flups_solver_s* s, cudaStream_t st) {
       s->green_pitch = (gext[0] + 1) & ~1;  // 16-byte rows (8-byte elements)
       const size_t padded = (size_t)s->green_pitch * gext[1] * gext[2] * 8;
       if (!e) e = cudaMallocAsync(&s->green_dev, padded, st);
-      if (!e) e = launch_green_finalize(g64, s->green_dev, prec, n, gext[0], s->green_pitch, 1.0, st);
+      if (!e) e = store_green(s, g64, gext, 1.0, st);
       cudaFreeAsync(g64, st);
       cudaError_t e2 = cudaStreamSynchronize(st);
       if (e || e2) return cuda_fail(e ? e : e2, "green spectral");
@@ -543,7 +616,7 @@ int setup_green_compute(flups_solver_s* s, cudaStream_t st) {
   const size_t padded = (size_t)s->green_pitch * q.gext[1] * q.gext[2] * esize(prec);
   e = cudaMallocAsync(&s->green_dev, padded, st);
   if (e) { cudaFreeAsync(g64, st); return cuda_fail(e, "green alloc"); }
-  e = launch_green_finalize(g64, s->green_dev, prec, n, q.gext[0], s->green_pitch, scale, st);
+  e = store_green(s, g64, q.gext, scale, st);
   cudaFreeAsync(g64, st);
   cudaError_t e2 = cudaStreamSynchronize(st);
   if (e || e2) return cuda_fail(e ? e : e2, "green finalize");
@@ -560,6 +633,7 @@ int setup_green_compute(flups_solver_s* s, cudaStream_t st) {
 // serving runtime releases idle plans only).
 struct GreenEntry {
   void* dev;
+  int* gexp;
   int pitch;
   double bytes;
   size_t padded;
@@ -577,6 +651,9 @@ std::string green_cache_key(const flups_solver_s* s) {
   put(&s->topo.prec, sizeof s->topo.prec);
   put(&s->green, sizeof s->green);
   put(&s->eps, sizeof s->eps);
+  // fixed-point spectra depend on the fused direction and on whether its pass is real
+  const int fmt = s->fx ? 1 + s->order[2] + 3 * s->cplx[2] : 0;
+  put(&fmt, sizeof fmt);
   for (int d = 0; d < 3; ++d) {
     const DirPlan& dp = s->dir[d];
     put(&dp.unb, sizeof dp.unb);
@@ -594,7 +671,7 @@ std::string green_cache_key(const flups_solver_s* s) {
 int setup_green(flups_solver_s* s, cudaStream_t st) {
   int du = 0;
   for (int d = 0; d < 3; ++d) du += s->dir[d].unb;
-  const bool stored = du > 0 || s->topo.prec == FLUPS_F64E;
+  const bool stored = du > 0 || s->topo.prec == FLUPS_F64E || s->fx;
   if (!s->share_green || !stored) return setup_green_compute(s, st);
   const std::string key = green_cache_key(s);
   {
@@ -603,6 +680,7 @@ int setup_green(flups_solver_s* s, cudaStream_t st) {
     if (it != g_green_cache.end()) {
       it->second.refs++;
       s->green_dev = it->second.dev;
+      s->green_exp = it->second.gexp;
       s->green_pitch = it->second.pitch;
       s->green_bytes = it->second.bytes;
       s->green_key = key;
@@ -616,12 +694,14 @@ int setup_green(flups_solver_s* s, cudaStream_t st) {
   if (it != g_green_cache.end()) {
     // another solver stored the same spectrum meanwhile: use that copy
     cudaFreeAsync(s->green_dev, st);
+    if (s->green_exp) cudaFreeAsync(s->green_exp, st);
     it->second.refs++;
     s->green_dev = it->second.dev;
+    s->green_exp = it->second.gexp;
     s->green_pitch = it->second.pitch;
   } else {
     const size_t padded = (size_t)s->green_pitch * s->dir[1].gext * s->dir[2].gext * esize(s->topo.prec);
-    g_green_cache[key] = GreenEntry{s->green_dev, s->green_pitch, s->green_bytes, padded, 1};
+    g_green_cache[key] = GreenEntry{s->green_dev, s->green_exp, s->green_pitch, s->green_bytes, padded, 1};
   }
   s->green_key = key;
   return FLUPS_OK;
@@ -816,6 +896,7 @@ void encode_input_map(Launch& L, int prec) {
 // wavefronts on bank conflicts (unbounded 512x256x256 FP32 under ncu).
 void set_rowx(Launch& L, int prec) {
   PassParams& p = L.p;
+  if (p.fx) return;
   p.rowx = 0;
   if (!p.ct || p.axis != 0 || (prec != FLUPS_F32 && prec != FLUPS_F64E) || p.W != 4 || p.center != C_CELL) return;
   if (L.kind != K_FWD_REAL && L.kind != K_INV_REAL) return;
@@ -881,6 +962,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     L.kind = K_FWD_REAL;
     fill_geom(L, s->dir[o[0]], o[0], s->dims[0], s->dims[1], prec, true, center, nc, 1, s->pitch[0], s->pitch[1]);
     L.p.ctypes = pack3(s->tf[0][o[0]], s->tf[1][o[0]], s->tf[2][o[0]]);
+    if (s->fx) fx_geom(L, o[0], true);
     L.p.out = s->W1;
     L.out_buf = 1;
     L.user_in = 1;
@@ -897,6 +979,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     L.kind = real ? K_FWD_REAL : K_FWD_C2C;
     fill_geom(L, s->dir[o[1]], o[1], s->dims[1], s->dims[2], prec, real, center, nc, 1, s->pitch[1], s->pitch[2]);
     L.p.ctypes = pack3(s->tf[0][o[1]], s->tf[1][o[1]], s->tf[2][o[1]]);
+    if (s->fx) fx_geom(L, o[1], real);
     L.p.in = s->W1;
     L.p.out = s->W2;
     L.in_buf = 1;
@@ -916,6 +999,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     fill_geom(L, dp, o[2], s->dims[2], s->dims[2], prec, real, center, curl ? 1 : nc, curl ? 3 : 1, s->pitch[2],
               s->pitch[2]);
     L.p.ctypes = pack3(s->tf[0][o[2]], s->tf[1][o[2]], s->tf[2][o[2]]);
+    if (s->fx) fx_geom(L, o[2], real);
     L.p.in = s->W2;
     L.p.out = s->W2;
     L.in_buf = 2;
@@ -936,6 +1020,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
       }
     }
     g.stored = s->green_dev;
+    g.gexp = s->green_exp;
     for (int d = 0; d < 3; ++d) {
       g.tab[d] = s->tabs[d];
       g.gext[d] = s->dir[d].gext;
@@ -953,6 +1038,18 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
         // the slice by TMA when the lanes' x indices are contiguous in the spectrum (x not folded)
         if (g.fold[0] == 0 && green_tensor_maps(s, o[2], L.p.W, dp.P, prec, &L.p.gbox, st))
           L.p.gmap = s->gmaps_dev;
+      }
+    }
+    if (s->fx && !real && o[2] != 0 && dp.gext == dp.P / 2 + 1 && g.fold[0] == 0) {
+      // fixed-point fused column pass: the Green slice by TMA while the forward transform runs, where
+      // two CTAs still fit an SM with it
+      const size_t gbytes = 128 + (size_t)L.p.W * (dp.P / 2 + 1) * sizeof(long long);
+      // (the slice's last row is a copy of its own, which must start on 128 bytes)
+      if (2 * (L.smem + gbytes + 1024) <= 228 * 1024 && (size_t)(dp.P / 2) * L.p.W * sizeof(long long) % 128 == 0 &&
+          green_tensor_maps(s, o[2], L.p.W, dp.P, prec, &L.p.gbox, st)) {
+        L.smem += gbytes;
+        L.p.gpre = 1;
+        L.p.gmap = s->gmaps_dev;
       }
     }
     g.kernel = s->green;
@@ -973,6 +1070,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     L.kind = real ? K_INV_REAL : K_INV_C2C;
     fill_geom(L, s->dir[o[1]], o[1], s->dims[2], s->dims[1], prec, real, center, nc, 1, s->pitch[2], s->pitch[1]);
     L.p.ctypes = pack3(s->tu[0][o[1]], s->tu[1][o[1]], s->tu[2][o[1]]);
+    if (s->fx) fx_geom(L, o[1], real);
     L.p.in = s->W2;
     L.p.out = s->W1;
     L.in_buf = 2;
@@ -988,6 +1086,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     L.kind = K_INV_REAL;
     fill_geom(L, s->dir[o[0]], o[0], s->dims[1], s->dims[0], prec, true, center, nc, 1, s->pitch[1], s->pitch[0]);
     L.p.ctypes = pack3(s->tu[0][o[0]], s->tu[1][o[0]], s->tu[2][o[0]]);
+    if (s->fx) fx_geom(L, o[0], true);
     L.p.in = s->W1;
     L.in_buf = 1;
     L.user_out = 1;
@@ -1001,6 +1100,8 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
   for (Launch& L : s->passes) set_rowx(L, prec);  // before set_rows_bulk (flups_setup): the staged rows follow the tile
   for (const Launch& L : s->passes)
     if (L.smem > 227 * 1024 || L.nthr > 1024) return FLUPS_ESIZE;
+  if (s->fx)
+    for (const Launch& L : s->passes) CK(limit_fx(L.kind, L.p.P));
   return FLUPS_OK;
 }
 
@@ -1138,6 +1239,12 @@ int flups_init_solver(flups_topo t, const int* bc, const double h[3], const doub
     }
   }
   if (rc == FLUPS_OK) rc = build_plan(s);
+  // FP64-class Poisson solves run in 64-bit fixed point, except the smallest: up to 2^16 points of the extended
+  // box a pass is one warp's chain of instructions, and the short FP64 columns of the warp engine are
+  // faster (measured, us per solve, FP64 / fixed point: periodic 32^3 25.7 / 29.9, unbounded 16^3 25.1 / 29.0,
+  // against periodic 36^3 39.8 / 28.6, unbounded 24^3 55.4 / 33.2, unbounded 64^3 230 / 76)
+  s->fx = t->prec != FLUPS_F32 && op == FLUPS_POISSON &&
+          (long long)s->dir[0].P * s->dir[1].P * s->dir[2].P > 65536;
   if (rc == FLUPS_OK) {
     int du = 0;
     for (int d = 0; d < 3; ++d) du += s->dir[d].unb;
@@ -1174,7 +1281,7 @@ int flups_setup(flups_solver s, void* stream, size_t* workspace_bytes) {
     }
   }
   for (int d = 0; d < 3; ++d) {
-    int rc = make_twiddles(s->dir[d].P, prec, &s->dir[d].tw);
+    int rc = make_twiddles(s->dir[d].P, s->fx ? kFxTables : prec, &s->dir[d].tw);
     if (rc) return rc;
     s->ws_bytes += (size_t)4 * s->dir[d].P * es;
   }
@@ -1244,7 +1351,8 @@ static int solve_impl(flups_solver s, void* phi, const void* rhs, void* ws, void
       encode_input_map(Lw, prec);
       set_rows_bulk(Lw, prec);
     }
-    if (p.rowx && ((L.user_in && host_in) || (L.user_out && host_out))) {
+    if (p.fx) p.fx_host = p.axis == 0 && ((L.user_in && host_in) || (L.user_out && host_out));
+    else if (p.rowx && ((L.user_in && host_in) || (L.user_out && host_out))) {
       p.rowx = 0;
       Lw.nthr = L.gnthr;
       if (!p.rows_bulk) Lw.smem = L.gsmem;
@@ -1282,9 +1390,10 @@ int flups_solver_memory(flups_solver s, size_t* resident, size_t* transient, siz
     if ((size_t)s->dir[d].gext > gmax) gmax = s->dir[d].gext;
     if (s->op == FLUPS_BIOT_SAVART) res += (size_t)s->dir[d].P * es;
   }
-  if (du == 0) {
+  if (du == 0)
     for (int d = 0; d < 3; ++d) res += (size_t)s->dir[d].gext * es;
-  } else {
+  if (s->fx) res += gn / s->dir[s->order[2]].gext * sizeof(int);
+  if (du > 0 || s->fx) {
     res += gn * es;
     tr += gn * sizeof(double) + (size_t)8 * 2 * gmax * sizeof(double);
   }
@@ -1329,12 +1438,23 @@ int flups_debug_green(flups_solver s, double* samples, double* spectrum, long lo
   const size_t rows = (size_t)q.gext[1] * q.gext[2];
   std::vector<unsigned char> buf(rows * s->green_pitch * es);
   CK(cudaMemcpy(buf.data(), s->green_dev, buf.size(), cudaMemcpyDeviceToHost));
-  // element formats: FP32, FP64, or on the double-float path a pair of floats (hi, lo)
+  std::vector<int> gexp;
+  if (s->fx) {
+    gexp.resize((size_t)(cnt / q.gext[s->order[2]]));
+    CK(cudaMemcpy(gexp.data(), s->green_exp, gexp.size() * sizeof(int), cudaMemcpyDeviceToHost));
+  }
+  // element formats: FP32, fixed point with an exponent per pencil, FP64, or a pair of floats (hi, lo)
   for (size_t r = 0; r < rows; ++r)
     for (int x = 0; x < q.gext[0]; ++x) {
       const size_t i = r * s->green_pitch + x;
       double v;
       if (es == 4) v = (double)((const float*)buf.data())[i];
+      else if (s->fx) {
+        const int ax = s->order[2], y = (int)(r % q.gext[1]), z = (int)(r / q.gext[1]);
+        const int pen = ax == 0 ? y + q.gext[1] * z : x + q.gext[0] * (ax == 1 ? z : y);
+        const long long g = ((const long long*)buf.data())[i];
+        v = std::ldexp((double)((long long)(int)(g >> 32) * 4294967296LL + (int)g), gexp[pen]);
+      }
       else if (s->topo.prec == FLUPS_F64E) v = (double)((const float*)buf.data())[2 * i] + (double)((const float*)buf.data())[2 * i + 1];
       else v = ((const double*)buf.data())[i];
       spectrum[r * q.gext[0] + x] = v;
@@ -1486,12 +1606,15 @@ static void release(flups_solver s, cudaStream_t st, bool async) {
     auto it = g_green_cache.find(s->green_key);
     if (it != g_green_cache.end() && --it->second.refs == 0) {
       fr(it->second.dev);
+      fr(it->second.gexp);
       g_green_cache.erase(it);
     }
     s->green_dev = nullptr;
+    s->green_exp = nullptr;
     s->green_key.clear();
   }
   fr(s->green_dev);
+  fr(s->green_exp);
   fr(s->stage);
   fr(s->errflag);
   fr(s->gmaps_dev);

@@ -1,0 +1,707 @@
+// Passes of the FP64-class Poisson solves (FP64 arrays in and out) in 64-bit block fixed point
+// (fx64.cuh): one kernel per pass kind and length P = 2^a 3^b, for every axis and tile width.
+//
+// A CTA holds W lanes (pencils; two packed real pencils per lane for real data) x P complex values
+// in shared memory and transforms them in place: a thread takes whole butterflies of up to 18 values in
+// registers, the block synchronises, and the values go back.  Complex passes read the first stage's
+// inputs from HBM into registers and store the last stage's outputs from registers, as do the real
+// passes of periodic and unbounded directions; symmetric directions build their extension in shared
+// memory.  Each length has its plan of radices 16, 12, 9, 8, 6, 4, 3, 2 at compile time (fx_plan), so the
+// factor 3 costs no separate engine; the tile width stays a run-time value, one integer operation per access.
+#pragma once
+#include <cuda_runtime.h>
+
+#include "fx64.cuh"
+#include "fx_plan.cuh"
+#include "pass_common.cuh"
+#include "passes.cuh"
+
+namespace flups {
+
+namespace {
+
+// A tile's shared memory after the 128-byte block of its mbarrier: S, then lane exponents and Green
+// offsets, then the staged Green slice (128-byte aligned).
+// renormalisation slots: second to fourth stage forward (and before the Green product, one more), after the
+// product, second to fourth stage inverse
+constexpr int kFxSlotFwd = 0, kFxSlotGain = 4, kFxSlotInv = 5;
+
+struct FxSmem {
+  cfx* S;
+  int* emax;          // W lane exponents
+  int* gexp;          // 2 W exponents of the pencils' Green slices
+  unsigned* words;    // kFxSlots x W magnitudes (upper words ORed) behind the lanes' renormalisations
+  long long* goff;    // 2 W Green offsets
+  unsigned long long* mbar;
+  long long* G;       // staged slice, (P/2 + 1) x W
+};
+
+__device__ __forceinline__ FxSmem fx_smem(unsigned char* smraw, int P, int W, int LS) {
+  FxSmem m;
+  unsigned char* base = smraw + ((128u - (smem_u32(smraw) & 127u)) & 127u);
+  m.mbar = reinterpret_cast<unsigned long long*>(base);
+  m.S = reinterpret_cast<cfx*>(base + 128);
+  m.goff = reinterpret_cast<long long*>(base + 128 + (size_t)P * LS * sizeof(cfx));
+  m.emax = reinterpret_cast<int*>(m.goff + 2 * W);
+  m.gexp = m.emax + W;
+  m.words = reinterpret_cast<unsigned*>(m.gexp + 2 * W);
+  unsigned char* g = reinterpret_cast<unsigned char*>(m.words + kFxSlots * W);
+  m.G = reinterpret_cast<long long*>(g + ((128u - (smem_u32(g) & 127u)) & 127u));
+  return m;
+}
+
+__device__ __forceinline__ unsigned abs_hi(double d) { return (unsigned)__double2hiint(d) & 0x7fffffffu; }
+__device__ __forceinline__ long long dec(double d, int E, int up = kFxUp) {
+  return fx_decode((unsigned long long)__double_as_longlong(d), E, up);
+}
+// FP64 value of x 2^q rounded to nearest; `kind` (from fx_out_kind) tells NaN lanes and scales outside FP64's
+// normal range.  The conversion runs on the FP64 pipe (measured 1.9 per SM and clock), which is otherwise idle, and
+// the scale joins the exponent field; normalising in integers took 3 times the instructions.
+__device__ __forceinline__ double enc(long long x, int q, int kind) {
+  const double d = __ll2double_rn(x);
+  if (kind == 0) {
+    const int h = __double2hiint(d);
+    return __hiloint2double(h ? h + (q << 20) : 0, __double2loint(d));
+  }
+  return kind == 1 ? scalbn(d, q) : __longlong_as_double(0x7ff8000000000000ll);
+}
+// 0: every |x| < 2^63 scales to a normal number (or 0); 1: not so; 2: NaN lane
+__device__ __forceinline__ int fx_out_kind(int E, int q) { return E >= 2047 ? 2 : (q > -1020 && q < 950 ? 0 : 1); }
+
+// Largest magnitude (upper words) of the lane's inputs over the CTA, as a biased exponent; a thread's
+// inputs belong to lane `lane` = tid mod W.
+__device__ __forceinline__ void lane_max(int* emax, unsigned m, int W, int lane, int tid) {
+  for (int o = W; o < 32; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((tid & 31) < W) atomicMax(&emax[lane], (int)(m >> 20));
+}
+
+__device__ __forceinline__ fxw fx_twiddle(const fxw* tw, int i) {
+  const int4 q = __ldg(reinterpret_cast<const int4*>(tw + i));
+  fxw w;
+  w.xh = q.x;
+  w.xl = q.y;
+  w.yh = q.z;
+  w.yl = q.w;
+  return w;
+}
+
+struct FxTile {
+  cfx* S;
+  int W, lw, LS, tid, nt;
+  const fxw* tw;
+};
+
+// Lane renormalisation.  The fixed factor 2^-4 of a twiddled stage is what the worst case needs; a lane whose
+// values did not grow (a spectrum of a few modes) would lose those bits at every stage.  From the second stage
+// of a transform on, and after the Green product, the lane's values are therefore shifted up to the bound
+// again: the stage before ORs the magnitudes of its outputs' upper words per lane, the next one shifts by
+// the free bits, eight integer operations per value.  (Relative error against a 64-bit solution, mixed 256^3: 1e-13
+// to 1.7e-12 with the fixed factors alone, 4e-16 to 5e-15 with the shift from the third stage on.)
+enum FxSrc : int { FX_TILE = 0, FX_RAW = 1, FX_GAIN = 2 };
+__device__ __forceinline__ int fx_free_tw(unsigned w) { return max(__clz(w) - 3, 0); }    // parts below 2^61
+__device__ __forceinline__ int fx_free_in(unsigned w) { return max(__clz(w) - 7, 0); }    // parts below 2^57
+__device__ __forceinline__ unsigned fx_mag(long long x) {
+  const int h = (int)(x >> 32);
+  return (unsigned)(h ^ (h >> 31));
+}
+__device__ __forceinline__ void lane_or(unsigned* word, unsigned m, int W, int lane, int tid) {
+  for (int o = W; o < 32; o <<= 1) m |= __shfl_xor_sync(0xffffffffu, m, o);
+  if ((tid & 31) < W) atomicOr(&word[lane], m);
+}
+// Shift that the renormalisations of lane l added: forward and inverse transforms of the plan, gain.
+template <int P>
+__device__ __forceinline__ int fx_shifted(const unsigned* words, int W, int l, bool fwd, bool gain, bool inv) {
+  constexpr int n = fx_plan(P).n;
+  int e = gain ? fx_free_in(words[kFxSlotGain * W + l]) + fx_free_tw(words[(kFxSlotFwd + n - 1) * W + l]) : 0;
+#pragma unroll
+  for (int s = 1; s < n; ++s) {
+    if (fwd) e += fx_free_tw(words[(kFxSlotFwd + s - 1) * W + l]);
+    if (inv) e += fx_free_tw(words[(kFxSlotInv + s - 1) * W + l]);
+  }
+  return e;
+}
+
+// One stage of radix R after a product Ns of earlier radices.  SRC: FX_RAW, In gives FP64 bits, aligned to the
+// lane's exponent (maxima in `lanes`) here; FX_GAIN, In gives products to renormalise (words `lanes`).  words:
+// the transform's slots; every stage but the first is renormalised.  Out: receives position o of lane l.
+template <int P, int R, int Ns, bool INV, int SRC, bool TO_S, int s, bool SCAN_LAST = false, class In, class Out>
+__device__ __forceinline__ void fx_stage(const FxTile& t, unsigned* lanes, unsigned* words, In in, Out out) {
+  constexpr int NB = fx_nb(R), nbf = P / R;
+  constexpr bool TW = s > 0, SCAN = SCAN_LAST || s < fx_plan(P).n - 1;
+  static_assert((s > 0) == (Ns > 1), "stage and product of earlier radices");
+  const int total = nbf * t.W;
+  const int lane = t.tid & (t.W - 1);
+  cfx v[NB][R];
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    const int idx = t.tid + b * t.nt, j = idx >> t.lw;
+    if (idx < total) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[b][r] = in(j + r * nbf, lane);
+    } else {
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[b][r] = fx_make(0, 0);
+    }
+  }
+  if constexpr (SRC == FX_RAW) {
+    unsigned m = 0;
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        m = max(m, max((unsigned)(v[b][r].x >> 32) & 0x7fffffffu, (unsigned)(v[b][r].y >> 32) & 0x7fffffffu));
+    lane_max(reinterpret_cast<int*>(lanes), m, t.W, lane, t.tid);
+    __syncthreads();
+    const int E = max((int)lanes[lane], kFxMinE);
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[b][r] = fx_make(fx_decode(v[b][r].x, E), fx_decode(v[b][r].y, E));
+  } else if constexpr (SRC == FX_GAIN) {
+    unsigned m = 0;
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+      for (int r = 0; r < R; ++r) m |= fx_mag(v[b][r].x) | fx_mag(v[b][r].y);
+    lane_or(lanes, m, t.W, lane, t.tid);
+    __syncthreads();
+  } else if constexpr (TO_S) {
+    __syncthreads();  // every input is in registers before the tile is overwritten
+  }
+  if constexpr (TW || SRC == FX_GAIN) {
+    const int n = SRC == FX_GAIN ? fx_free_in(lanes[lane]) : fx_free_tw(words[(s - 1) * t.W + lane]);
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[b][r] = fx_make(v[b][r].x << n, v[b][r].y << n);
+  }
+  unsigned mo = 0;
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    const int idx = t.tid + b * t.nt, j = idx >> t.lw;
+    if (idx < total) {
+      const int k = TW ? j % Ns : 0;
+      if constexpr (TW) {
+        constexpr int tstep = (2 * P) / (Ns * R);
+        v[b][0] = fx_make(fx_shr(v[b][0].x, kFxTwShift), fx_shr(v[b][0].y, kFxTwShift));
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[b][r] = fx_cmul<INV>(v[b][r], fx_twiddle(t.tw, r * k * tstep));
+      }
+      fx_dft<R, INV>(v[b]);
+      const int o0 = (j - k) * R + k;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        out(o0 + r * Ns, lane, v[b][r]);
+        if constexpr (SCAN) mo |= fx_mag(v[b][r].x) | fx_mag(v[b][r].y);
+      }
+    }
+  }
+  if constexpr (SCAN) lane_or(words + s * t.W, mo, t.W, lane, t.tid);
+  if constexpr (TO_S) __syncthreads();
+}
+
+// Stages [s, s1) of the plan inside the tile (REV: radices in reverse order); words: the transform's slots.
+// SCAN_LAST: the last stage's outputs are scanned too.
+template <int P, bool INV, bool REV, int s, int s1, bool SCAN_LAST = false>
+__device__ __forceinline__ void fx_mid_stages(const FxTile& t, unsigned* words) {
+  if constexpr (s < s1) {
+    constexpr FxPlan pl = fx_plan(P);
+    constexpr int R = pl.r[REV ? pl.n - 1 - s : s], Ns = REV ? fx_prod(P, pl.n - s, pl.n) : fx_prod(P, 0, s);
+    cfx* S = t.S;
+    const int LS = t.LS;
+    fx_stage<P, R, Ns, INV, FX_TILE, true, s, SCAN_LAST>(
+        t, nullptr, words, [=](int i, int l) { return S[i * LS + l]; },
+        [=](int o, int l, const cfx& v) { S[o * LS + l] = v; });
+    fx_mid_stages<P, INV, REV, s + 1, s1, SCAN_LAST>(t, words);
+  }
+}
+
+// Green offset (axis term excluded) and exponent of pencil q; past the last pencil a zero offset and an
+// exponent that takes no part in a pair's common one.
+__device__ __forceinline__ void fx_green_base(const PassParams& p, int q, int o, long long* goff, int* gexp) {
+  const FusedGreen& g = p.g;
+  *goff = 0;
+  *gexp = -(1 << 20);
+  if (q >= p.npen) return;
+  int c[3];
+  if (p.axis == 0) { c[1] = q % g.dims1; c[2] = q / g.dims1; c[0] = 0; }
+  else if (p.axis == 1) { c[0] = q; c[2] = o; c[1] = 0; }
+  else { c[0] = q; c[1] = o; c[2] = 0; }
+  const long long st[3] = {1, (long long)g.gpitch, (long long)g.gpitch * g.gext[1]};
+  long long off = 0, e = 0, es = 1;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    if (d == p.axis) continue;
+    int gi = c[d];
+    if (g.fold[d]) gi = min(gi, g.fold[d] - gi);
+    off += gi * st[d];
+    e += gi * es;
+    es *= g.gext[d];
+  }
+  *goff = off;
+  *gexp = g.gexp[e];
+}
+
+// Load of real data pairs whose extension is built in the tile (symmetric and semi-unbounded directions, and
+// every real pass on pinned host arrays): items (lane, i < n_data), at most U per thread.
+template <int P, int U>
+__device__ __forceinline__ void fx_load_ext(const PassParams& p, const FxTile& t, int type, const double* in, int q0,
+                                            int* emax) {
+  const int W = t.W, LS = t.LS, N = p.N, nd = p.n_data, tot = nd * W;
+  const int bt = base_type(type);
+  const bool rev = is_reversed(type);
+  cfx* S = t.S;
+  double a[U], b[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int idx = t.tid + u * t.nt;
+    a[u] = b[u] = 0.0;
+    if (idx < tot) {
+      const int l = p.fx_host ? idx / nd : idx & (W - 1), i = p.fx_host ? idx % nd : idx >> t.lw;
+      const int qa = q0 + 2 * l;
+      const long long off = (long long)qa * p.ai.ls + (long long)i * p.ai.js;
+      if (qa < p.npen) a[u] = in[off];
+      if (qa + 1 < p.npen) b[u] = in[off + p.ai.ls];
+      if (p.type == T_PER && i >= N) a[u] = b[u] = 0.0;  // the duplicate node is not used
+      if (p.fx_host) atomicMax(&emax[l], (int)(max(abs_hi(a[u]), abs_hi(b[u])) >> 20));
+    }
+  }
+  // zero padding and odd faces
+  int lo[3], hi[3];
+  const int nz = zero_ranges(bt, p.center, N, lo, hi);
+  for (int z = 0; z < nz; ++z)
+    for (int idx = t.tid; idx < (min(hi[z], P) - lo[z]) * W; idx += t.nt)
+      S[(lo[z] + (idx >> t.lw)) * LS + (idx & (W - 1))] = fx_make(0, 0);
+  if (!p.fx_host) {
+    unsigned m = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) m = max(m, max(abs_hi(a[u]), abs_hi(b[u])));
+    lane_max(emax, m, W, t.tid & (W - 1), t.tid);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int idx = t.tid + u * t.nt;
+    if (idx >= tot) continue;
+    const int l = p.fx_host ? idx / nd : idx & (W - 1), i = p.fx_host ? idx % nd : idx >> t.lw;
+    const int E = max(emax[l], kFxMinE);
+    const cfx v = fx_make(dec(a[u], E), dec(b[u], E));
+    const int dix = rev ? nd - 1 - i : i;
+    int pos[4], sg[4];
+    const int n = images(bt, p.center, N, dix, pos, sg);
+    for (int k = 0; k < n; ++k) S[pos[k] * LS + l] = sg[k] > 0 ? v : fx_make(-v.x, -v.y);
+  }
+  __syncthreads();
+}
+
+// Forward transform of real data into the tile: pairs (row q0 + 2l, row q0 + 2l + 1).
+template <int P, bool SCAN_LAST>
+__device__ __forceinline__ void fx_forward_real(const PassParams& p, const FxTile& t, int type, const double* in,
+                                                int q0, int* emax, unsigned* words) {
+  cfx* S = t.S;
+  const int LS = t.LS;
+  constexpr FxPlan pl = fx_plan(P);
+  auto to_s = [=](int o, int l, const cfx& v) { S[o * LS + l] = v; };
+  if ((type == T_PER || type == T_UNB) && !p.fx_host) {
+    // no images: the first stage reads its positions from memory
+    const int nu = p.n_use, npen = p.npen;
+    const long long ls = p.ai.ls, js = p.ai.js;
+    fx_stage<P, pl.r[0], 1, false, FX_RAW, true, 0>(
+        t, reinterpret_cast<unsigned*>(emax), words,
+        [=](int i, int l) {
+          const int qa = q0 + 2 * l;
+          const double* r = in + (long long)qa * ls + (long long)i * js;
+          cfx v = fx_make(0, 0);
+          if (i < nu && qa < npen) v.x = __double_as_longlong(r[0]);
+          if (i < nu && qa + 1 < npen) v.y = __double_as_longlong(r[ls]);
+          return v;
+        },
+        to_s);
+  } else {
+    if (p.n_data * t.W <= 9 * t.nt) fx_load_ext<P, 9>(p, t, type, in, q0, emax);
+    else fx_load_ext<P, 19>(p, t, type, in, q0, emax);
+    fx_stage<P, pl.r[0], 1, false, FX_TILE, true, 0>(
+        t, nullptr, words, [=](int i, int l) { return S[i * LS + l]; }, to_s);
+  }
+  fx_mid_stages<P, false, false, 1, pl.n, SCAN_LAST>(t, words);
+}
+
+// Store of real data from the tile's last inverse stage; q: exponent of lane l's values.
+template <int P, class Q>
+__device__ __forceinline__ void fx_store_real(const PassParams& p, const FxTile& t, int type, double* out, int q0,
+                                              unsigned* words, Q lane_q) {
+  constexpr FxPlan pl = fx_plan(P);
+  constexpr int R = pl.r[pl.n - 1], Ns = P / R;
+  cfx* S = t.S;
+  const int LS = t.LS, nd = p.n_data, N = p.N;
+  const int bt = base_type(type);
+  const bool rev = is_reversed(type);
+  const bool node = p.center == C_NODE;
+  const bool odd0 = node && (bt == T_OO || bt == T_OE || bt == T_OU), oddN = node && (bt == T_OO || bt == T_EO);
+  const long long ls = p.ao.ls, js = p.ao.js;
+  const int npen = p.npen;
+  auto put = [&](int l, int pos, int i, const cfx& v) {
+    const int qa = q0 + 2 * l;
+    if (qa >= npen) return;
+    int q, kind;
+    lane_q(l, &q, &kind);
+    const bool zero = (odd0 && pos == 0) || (oddN && pos == N);
+    double* o = out + (long long)qa * ls + (long long)i * js;
+    o[0] = zero ? 0.0 : enc(v.x, q, kind);
+    if (qa + 1 < npen) o[ls] = zero ? 0.0 : enc(v.y, q, kind);
+  };
+  if (!p.fx_host) {
+    const bool dup = bt == T_PER && node && nd > N;
+    fx_stage<P, R, Ns, true, FX_TILE, false, pl.n - 1>(
+        t, nullptr, words, [=](int i, int l) { return S[i * LS + l]; },
+        [&](int o, int l, const cfx& v) {
+          if (o < nd && !(dup && o == N)) put(l, o, rev ? nd - 1 - o : o, v);
+          if (dup && o == 0) put(l, 0, N, v);
+        });
+    return;
+  }
+  fx_stage<P, R, Ns, true, FX_TILE, true, pl.n - 1>(
+      t, nullptr, words, [=](int i, int l) { return S[i * LS + l]; },
+      [=](int o, int l, const cfx& v) { S[o * LS + l] = v; });
+  for (int idx = t.tid; idx < nd * t.W; idx += t.nt) {
+    const int l = idx / nd, i = idx % nd;
+    const int pos = (bt == T_PER && node && i == N) ? 0 : (rev ? nd - 1 - i : i);
+    put(l, pos, i, S[pos * LS + l]);
+  }
+}
+
+template <int KIND, int P>
+__global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParams p) {
+  pass_entry(p);
+  extern __shared__ __align__(16) unsigned char smraw[];
+  constexpr bool REAL = KIND == K_FWD_REAL || KIND == K_INV_REAL || KIND == K_FUSED_REAL;
+  constexpr bool FUSED = KIND == K_FUSED_REAL || KIND == K_FUSED_C2C;
+  const FxSmem m = fx_smem(smraw, P, p.W, p.LS);
+  const int tid = threadIdx.x, nt = blockDim.x;
+  FxTile t;
+  t.S = m.S;
+  t.W = p.W;
+  t.lw = p.lw;
+  t.LS = p.LS;
+  t.tid = tid;
+  t.nt = nt;
+  t.tw = (const fxw*)p.tw;
+  constexpr FxPlan pl = fx_plan(P);
+  constexpr int ns = pl.n, half = P / 2, R0 = pl.r[0], RL = pl.r[ns - 1];
+  const int W = p.W, LS = p.LS;
+  cfx* S = m.S;
+  const int q0 = blockIdx.x * (REAL ? 2 * W : W);
+  // fused pass: rows o and n - o share a Green slice and run back to back
+  int o = blockIdx.y;
+  if (KIND == K_FUSED_C2C && o > 0) o = (blockIdx.y & 1) ? (o + 1) / 2 : (int)gridDim.y - o / 2;
+  const long long bi = (long long)o * p.ai.os + (long long)blockIdx.z * p.ai.cs;
+  const long long bo = (long long)o * p.ao.os + (long long)blockIdx.z * p.ao.cs;
+  const int type = comp_type(p, blockIdx.z);
+  if (tid < W) m.emax[tid] = 0;
+  for (int i = tid; i < kFxSlots * W; i += nt) m.words[i] = 0;
+  unsigned* wf = m.words + kFxSlotFwd * W;
+  unsigned* wi = m.words + kFxSlotInv * W;
+  unsigned* wg = m.words + kFxSlotGain * W;
+  unsigned* emax = reinterpret_cast<unsigned*>(m.emax);
+  const bool tma_g = FUSED && p.gpre && p.gmap;
+  if constexpr (FUSED) {
+    for (int l = tid; l < (REAL ? 2 * W : W); l += nt) fx_green_base(p, q0 + l, o, &m.goff[l], &m.gexp[l]);
+    if (tma_g && tid == 0) mbar_init(m.mbar, 1);
+  }
+  __syncthreads();
+  if (tma_g && tid == 0) {
+    const FusedGreen& g = p.g;
+    const int od = p.axis == 2 ? 1 : 2;  // the direction o runs along
+    const int go = g.fold[od] ? min(o, g.fold[od] - o) : o;
+    const char* maps = (const char*)p.gmap;
+    mbar_expect_tx(m.mbar, (unsigned)((half + 1) * W * sizeof(long long)));
+    for (int r0 = 0; r0 < half; r0 += p.gbox) {
+      if (p.axis == 2) tma_load_3d(m.G + (size_t)r0 * W, maps, q0, go, r0, m.mbar);
+      else tma_load_3d(m.G + (size_t)r0 * W, maps, q0, r0, go, m.mbar);
+    }
+    if (p.axis == 2) tma_load_3d(m.G + (size_t)half * W, maps + 128, q0, go, half, m.mbar);
+    else tma_load_3d(m.G + (size_t)half * W, maps + 128, q0, half, go, m.mbar);
+  }
+  // exponent of a fixed-point value of lane l after the forward (or a single inverse) transform
+  constexpr int shift = kFxTwShift * (ns - 1) - kFxBias;
+  auto from_s = [=](int i, int l) { return S[i * LS + l]; };
+  auto to_s = [=](int i, int l, const cfx& v) { S[i * LS + l] = v; };
+
+  if constexpr (KIND == K_FWD_REAL) {
+    fx_forward_real<P, false>(p, t, type, (const double*)p.in + bi, q0, m.emax, wf);
+    const int bt = base_type(type);
+    const bool cplx = bt == T_PER || bt == T_UNB, quarter = is_quarter(bt), oddo = is_odd_origin(bt);
+    const bool cell = p.center == C_CELL;
+    const int nm = p.n_modes, l = tid & (W - 1), qa = q0 + 2 * l;
+    const int E = max(m.emax[l], kFxMinE);
+    // the split leaves twice the modes; a phase costs 2^4, a quarter-wave type halves
+    const int q = E + shift - fx_shifted<P>(m.words, W, l, true, false, false) - 1 + (cplx || !cell ? 0 : kFxTwShift) - (quarter ? 1 : 0);
+    const int kind = fx_out_kind(E, q);
+    if (qa < p.npen) {
+      const bool two = qa + 1 < p.npen;
+      for (int k = tid >> p.lw; k < nm; k += nt >> p.lw) {
+        const int kk = quarter ? 2 * k + 1 : k, km = kk == 0 ? 0 : P - kk;
+        const cfx zk = S[kk * LS + l], zm = S[km * LS + l];
+        cfx A = fx_make(zk.x + zm.x, zk.y - zm.y), B = fx_make(zk.y + zm.y, zm.x - zk.x);
+        const long long off = bo + (long long)qa * p.ao.ls + (long long)k * p.ao.js;
+        if (cplx) {
+          double2* out = (double2*)p.out;
+          out[off] = make_double2(enc(A.x, q, kind), enc(A.y, q, kind));
+          if (two) out[off + p.ao.ls] = make_double2(enc(B.x, q, kind), enc(B.y, q, kind));
+        } else {
+          double* out = (double*)p.out;
+          if (cell) {
+            const fxw w = fx_twiddle(t.tw, kk);
+            A = fx_cmul<false>(A, w);
+            B = fx_cmul<false>(B, w);
+          }
+          out[off] = enc(oddo ? -A.y : A.x, q, kind);
+          if (two) out[off + p.ao.ls] = enc(oddo ? -B.y : B.x, q, kind);
+        }
+      }
+    }
+  } else if constexpr (KIND == K_INV_REAL) {
+    const int bt = base_type(type);
+    const bool cplx = bt == T_PER || bt == T_UNB, quarter = is_quarter(bt), oddo = is_odd_origin(bt);
+    const bool cell = p.center == C_CELL;
+    const int nm = p.n_modes, l = tid & (W - 1), qa = q0 + 2 * l;
+    const bool ra = qa < p.npen, rb = qa + 1 < p.npen;
+    // stored modes of both pencils: at most 10 per thread (the host sizes the block)
+    constexpr int U = 10;
+    double ax[U], ay[U], bx[U], by[U];
+    const long long offl = bi + (long long)qa * p.ai.ls;
+    unsigned mx = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int k = (tid + u * nt) >> p.lw;
+      ax[u] = ay[u] = bx[u] = by[u] = 0.0;
+      if (k < nm) {
+        const long long off = offl + (long long)k * p.ai.js;
+        if (cplx) {
+          const double2* in = (const double2*)p.in;
+          const bool real_mode = k == 0 || 2 * k == P;
+          if (ra) {
+            const double2 c = in[off];
+            ax[u] = c.x;
+            ay[u] = real_mode ? 0.0 : c.y;
+          }
+          if (rb) {
+            const double2 c = in[off + p.ai.ls];
+            bx[u] = c.x;
+            by[u] = real_mode ? 0.0 : c.y;
+          }
+        } else {
+          const double* in = (const double*)p.in;
+          if (ra) ax[u] = in[off];
+          if (rb) bx[u] = in[off + p.ai.ls];
+        }
+      }
+      mx = max(max(mx, max(abs_hi(ax[u]), abs_hi(ay[u]))), max(abs_hi(bx[u]), abs_hi(by[u])));
+    }
+    lane_max(m.emax, mx, W, l, tid);
+    if (quarter)  // even modes of the quarter-wave types are zero
+      for (int idx = tid; idx < half * W; idx += nt) S[2 * (idx >> p.lw) * LS + (idx & (W - 1))] = fx_make(0, 0);
+    __syncthreads();
+    const int E = max(m.emax[l], kFxMinE);
+    // the half-sample phase divides by 2^4: such coefficients keep 4 more bits
+    const int up = kFxUp + (cplx || !cell ? 0 : kFxTwShift);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int k = (tid + u * nt) >> p.lw;
+      if (k >= nm) continue;
+      const int kk = quarter ? 2 * k + 1 : k;
+      cfx A = fx_make(dec(ax[u], E, up), dec(ay[u], E, up)), B = fx_make(dec(bx[u], E, up), dec(by[u], E, up));
+      if (!cplx) {
+        if (oddo) {
+          A = fx_make(0, -A.x);
+          B = fx_make(0, -B.x);
+        }
+        if (cell) {
+          const fxw w = fx_twiddle(t.tw, kk);
+          A = fx_cmul<true>(A, w);
+          B = fx_cmul<true>(B, w);
+        }
+      }
+      S[kk * LS + l] = fx_make(A.x - B.y, A.y + B.x);
+      if (kk != 0 && 2 * kk != P) S[(P - kk) * LS + l] = fx_make(A.x + B.y, B.x - A.y);
+    }
+    __syncthreads();
+    fx_stage<P, R0, 1, true, FX_TILE, true, 0>(t, nullptr, wi, from_s, to_s);
+    fx_mid_stages<P, true, false, 1, ns - 1>(t, wi);
+    const int add = shift + (quarter ? 1 : 0);
+    fx_store_real<P>(p, t, type, (double*)p.out + bo, q0, wi, [&](int lane, int* q, int* kind) {
+      const int Ee = max(m.emax[lane], kFxMinE);
+      *q = Ee + add - fx_shifted<P>(m.words, W, lane, false, false, true);
+      *kind = fx_out_kind(Ee, *q);
+    });
+  } else if constexpr (KIND == K_FUSED_REAL) {
+    fx_forward_real<P, true>(p, t, type, (const double*)p.in + bi, q0, m.emax, wf);
+    const bool quarter = is_quarter(base_type(type));
+    unsigned mo = 0;
+    {
+      const int l = tid & (W - 1), upx = fx_free_tw(wf[(ns - 1) * W + l]);
+      const long long ga = m.goff[2 * l], gb = m.goff[2 * l + 1];
+      const int ea = m.gexp[2 * l], eb = m.gexp[2 * l + 1], e = max(ea, eb);
+      const int sa = min(e - ea, 62), sb = min(e - eb, 62);
+      const long long st3 = p.axis == 0 ? 1 : (p.axis == 1 ? (long long)p.g.gpitch : (long long)p.g.gpitch * p.g.gext[1]);
+      const long long* G = (const long long*)p.g.stored;
+      for (int k = tid >> p.lw; k <= half; k += nt >> p.lw) {
+        const int km = k == 0 ? 0 : P - k;
+        cfx zk = S[k * LS + l], zm = S[km * LS + l];
+        zk = fx_make(zk.x << upx, zk.y << upx);
+        zm = fx_make(zm.x << upx, zm.y << upx);
+        cfx A = fx_make(0, 0), B = A;
+        if (!quarter || (k & 1)) {
+          const int g3 = quarter ? (k - 1) >> 1 : k;
+          const long long va = __ldg(&G[ga + g3 * st3]), vb = __ldg(&G[gb + g3 * st3]);
+          const int ah = (int)(va >> 32), al = (int)va, bh = (int)(vb >> 32), bl = (int)vb;
+          A = fx_make(fx_shr(fx_mul(zk.x + zm.x, ah, al), sa), fx_shr(fx_mul(zk.y - zm.y, ah, al), sa));
+          B = fx_make(fx_shr(fx_mul(zk.y + zm.y, bh, bl), sb), fx_shr(fx_mul(zm.x - zk.x, bh, bl), sb));
+        }
+        const cfx zp = fx_make(A.x - B.y, A.y + B.x), zq = fx_make(A.x + B.y, B.x - A.y);
+        mo |= fx_mag(zp.x) | fx_mag(zp.y) | fx_mag(zq.x) | fx_mag(zq.y);
+        S[k * LS + l] = zp;
+        if (k != 0 && 2 * k != P) S[km * LS + l] = zq;
+      }
+      lane_or(wg, mo, W, l, tid);
+    }
+    __syncthreads();
+    const int up = fx_free_in(wg[tid & (W - 1)]);
+    fx_stage<P, R0, 1, true, FX_TILE, true, 0>(
+        t, nullptr, wi,
+        [=](int i, int l) {
+          const cfx z = S[i * LS + l];
+          return fx_make(z.x << up, z.y << up);
+        },
+        to_s);
+    fx_mid_stages<P, true, false, 1, ns - 1>(t, wi);
+    fx_store_real<P>(p, t, type, (double*)p.out + bo, q0, wi, [&](int lane, int* q, int* kind) {
+      const int Ee = max(m.emax[lane], kFxMinE);
+      *q = Ee - fx_shifted<P>(m.words, W, lane, true, true, true) + 2 * shift + kFxBias - 1 + 64 + max(m.gexp[2 * lane], m.gexp[2 * lane + 1]);
+      *kind = fx_out_kind(Ee, *q);
+    });
+  } else {
+    // complex passes
+    const double2* in = (const double2*)p.in + bi;
+    double2* out = (double2*)p.out + bo;
+    const int npen = p.npen, n_in = KIND == K_INV_C2C ? P : p.n_use;
+    const long long ils = p.ai.ls, ijs = p.ai.js, ols = p.ao.ls, ojs = p.ao.js;
+    auto load = [=](int i, int l) {
+      cfx v = fx_make(0, 0);
+      if (i < n_in && q0 + l < npen) {
+        const longlong2 c = *reinterpret_cast<const longlong2*>(&in[(long long)(q0 + l) * ils + (long long)i * ijs]);
+        v = fx_make(c.x, c.y);
+      }
+      return v;
+    };
+    const int l0 = tid & (W - 1);
+    const int n_out = KIND == K_FWD_C2C ? P : p.n_data;
+    const int dup = (KIND != K_FWD_C2C && p.type == T_PER && p.center == C_NODE && p.n_data > p.N) ? p.N : -1;
+    int q = 0, kind = 0;
+    bool store_ok = true;
+    auto store = [&](int i, int l, const cfx& v) {
+      if (q0 + l >= npen || !store_ok) return;
+      const double2 d = make_double2(enc(v.x, q, kind), enc(v.y, q, kind));
+      if (i < n_out && i != dup) out[(long long)(q0 + l) * ols + (long long)i * ojs] = d;
+      if (i == 0 && dup >= 0) out[(long long)(q0 + l) * ols + (long long)dup * ojs] = d;
+    };
+    if constexpr (KIND == K_FUSED_C2C) {
+      fx_stage<P, R0, 1, false, FX_RAW, true, 0>(t, emax, wf, load, to_s);
+      fx_mid_stages<P, false, false, 1, ns, true>(t, wf);
+      // u^ = G^ f^ in the first inverse stage (radices reversed)
+      if (tma_g) {
+        if (!mbar_wait_bounded(m.mbar, p.errflag, 1, p.dbg_wait & 1)) store_ok = false;
+      }
+      const long long go = m.goff[l0];
+      const long long st3 = p.axis == 0 ? 1 : (p.axis == 1 ? (long long)p.g.gpitch : (long long)p.g.gpitch * p.g.gext[1]);
+      const long long* G = (const long long*)p.g.stored + go;
+      const long long* Gs = m.G;
+      const int upx = fx_free_tw(wf[(ns - 1) * W + l0]);
+      auto gained = [=](int i, int l) {
+        const cfx z = S[i * LS + l];
+        const int g3 = min(i, P - i);
+        const long long g = tma_g ? Gs[g3 * W + l] : __ldg(&G[g3 * st3]);
+        const int gh = (int)(g >> 32), gl = (int)g;
+        return fx_make(fx_mul(z.x << upx, gh, gl), fx_mul(z.y << upx, gh, gl));
+      };
+      fx_stage<P, RL, 1, true, FX_GAIN, true, 0>(t, wg, wi, gained, to_s);
+      fx_mid_stages<P, true, true, 1, ns - 1>(t, wi);
+      const int E = max(m.emax[l0], kFxMinE);
+      q = E - fx_shifted<P>(m.words, W, l0, true, true, true) + 2 * shift + kFxBias + 64 + m.gexp[l0];
+      kind = fx_out_kind(E, q);
+      fx_stage<P, R0, P / R0, true, FX_TILE, false, ns - 1>(t, nullptr, wi, from_s, store);
+    } else {
+      constexpr bool INV = KIND == K_INV_C2C;
+      fx_stage<P, R0, 1, INV, FX_RAW, true, 0>(t, emax, wf, load, to_s);
+      fx_mid_stages<P, INV, false, 1, ns - 1>(t, wf);
+      const int E = max(m.emax[l0], kFxMinE);
+      q = E + shift - fx_shifted<P>(m.words, W, l0, true, false, false);
+      kind = fx_out_kind(E, q);
+      fx_stage<P, RL, P / RL, INV, FX_TILE, false, ns - 1>(t, nullptr, wf, from_s, store);
+    }
+  }
+}
+
+}  // namespace
+
+template <int KIND, int P>
+cudaError_t fx_launch(const PassParams& p, dim3 grid, int nthr, size_t smem, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)nthr);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = p.pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k_fx<KIND, P>, p);
+}
+
+template <int P>
+cudaError_t fx_launch_kind(int kind, const PassParams& p, dim3 grid, int nthr, size_t smem, cudaStream_t st) {
+  switch (kind) {
+    case K_FWD_REAL: return fx_launch<K_FWD_REAL, P>(p, grid, nthr, smem, st);
+    case K_INV_REAL: return fx_launch<K_INV_REAL, P>(p, grid, nthr, smem, st);
+    case K_FWD_C2C: return fx_launch<K_FWD_C2C, P>(p, grid, nthr, smem, st);
+    case K_INV_C2C: return fx_launch<K_INV_C2C, P>(p, grid, nthr, smem, st);
+    case K_FUSED_REAL: return fx_launch<K_FUSED_REAL, P>(p, grid, nthr, smem, st);
+    case K_FUSED_C2C: return fx_launch<K_FUSED_C2C, P>(p, grid, nthr, smem, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <int KIND, int P> cudaError_t fx_limit() {
+  return cudaFuncSetAttribute(k_fx<KIND, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+}
+template <int P> cudaError_t fx_limit_kind(int kind) {
+  switch (kind) {
+    case K_FWD_REAL: return fx_limit<K_FWD_REAL, P>();
+    case K_INV_REAL: return fx_limit<K_INV_REAL, P>();
+    case K_FWD_C2C: return fx_limit<K_FWD_C2C, P>();
+    case K_INV_C2C: return fx_limit<K_INV_C2C, P>();
+    case K_FUSED_REAL: return fx_limit<K_FUSED_REAL, P>();
+    case K_FUSED_C2C: return fx_limit<K_FUSED_C2C, P>();
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+#define FX_LAUNCH_CASE(P) \
+  case P: return fx_launch_kind<P>(kind, p, grid, nthr, smem, st);
+#define FX_LIMIT_CASE(P) \
+  case P: return fx_limit_kind<P>(kind);
+// Launcher and shared-memory limits of the lengths of FX_SHARD_<i>.
+#define FX_UNIT(i)                                                                                              \
+  namespace flups {                                                                                             \
+  cudaError_t launch_fx_##i(int kind, const PassParams& p, dim3 grid, int nthr, size_t smem, cudaStream_t st) { \
+    switch (p.P) { FX_SHARD_##i(FX_LAUNCH_CASE) }                                                               \
+    return cudaErrorInvalidValue;                                                                               \
+  }                                                                                                             \
+  cudaError_t limit_fx_##i(int kind, int P) {                                                                   \
+    switch (P) { FX_SHARD_##i(FX_LIMIT_CASE) }                                                                  \
+    return cudaErrorInvalidValue;                                                                               \
+  }                                                                                                             \
+  }
+
+}  // namespace flups

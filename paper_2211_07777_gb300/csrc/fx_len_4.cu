@@ -1,0 +1,4 @@
+// Fixed-point passes of the lengths of FX_SHARD_4.
+#include "fx_kernels.cuh"
+
+FX_UNIT(4)

@@ -1,0 +1,111 @@
+// Lengths of the fixed-point passes, their radices, and the translation units that compile them.
+#pragma once
+
+namespace flups {
+
+// Lengths and their radices, fewest stages first, then the cheapest split by operations per value and
+// threads left idle.
+#define FX_LENGTHS(X) \
+  X(4, 2, 2, 2, 1, 1) \
+  X(6, 2, 3, 2, 1, 1) \
+  X(8, 2, 4, 2, 1, 1) \
+  X(9, 2, 3, 3, 1, 1) \
+  X(12, 2, 4, 3, 1, 1) \
+  X(16, 2, 4, 4, 1, 1) \
+  X(18, 2, 6, 3, 1, 1) \
+  X(24, 2, 8, 3, 1, 1) \
+  X(27, 3, 3, 3, 3, 1) \
+  X(32, 2, 8, 4, 1, 1) \
+  X(36, 2, 6, 6, 1, 1) \
+  X(48, 2, 12, 4, 1, 1) \
+  X(54, 2, 9, 6, 1, 1) \
+  X(64, 2, 8, 8, 1, 1) \
+  X(72, 2, 12, 6, 1, 1) \
+  X(81, 2, 9, 9, 1, 1) \
+  X(96, 2, 12, 8, 1, 1) \
+  X(108, 3, 6, 6, 3, 1) \
+  X(128, 2, 16, 8, 1, 1) \
+  X(144, 2, 12, 12, 1, 1) \
+  X(162, 3, 9, 9, 2, 1) \
+  X(192, 2, 16, 12, 1, 1) \
+  X(216, 3, 6, 6, 6, 1) \
+  X(243, 4, 9, 3, 3, 3) \
+  X(256, 2, 16, 16, 1, 1) \
+  X(288, 3, 12, 12, 2, 1) \
+  X(324, 3, 9, 9, 4, 1) \
+  X(384, 3, 16, 8, 3, 1) \
+  X(432, 3, 12, 6, 6, 1) \
+  X(486, 4, 9, 9, 3, 2) \
+  X(512, 3, 8, 8, 8, 1) \
+  X(576, 3, 12, 12, 4, 1) \
+  X(648, 4, 6, 6, 6, 3) \
+  X(729, 3, 9, 9, 9, 1) \
+  X(768, 3, 16, 16, 3, 1) \
+  X(864, 3, 12, 12, 6, 1) \
+  X(972, 4, 9, 9, 4, 3) \
+  X(1024, 3, 16, 8, 8, 1) \
+  X(1152, 3, 12, 12, 8, 1) \
+  X(1296, 4, 6, 6, 6, 6) \
+  X(1458, 4, 9, 9, 9, 2) \
+  X(1536, 4, 8, 8, 8, 3) \
+  X(1728, 3, 12, 12, 12, 1) \
+  X(1944, 4, 9, 6, 6, 6) \
+  X(2048, 3, 16, 16, 8, 1) \
+  X(2187, 4, 9, 9, 9, 3) \
+  X(2304, 3, 16, 12, 12, 1) \
+  X(2592, 4, 12, 6, 6, 6) \
+  X(2916, 4, 9, 9, 9, 4) \
+  X(3072, 4, 16, 8, 8, 3) \
+  X(3456, 4, 12, 12, 12, 2) \
+  X(3888, 4, 12, 9, 6, 6) \
+  X(4096, 3, 16, 16, 16, 1)
+
+
+// The lengths by translation unit (fx_len_<i>.cu), balanced by compile time.
+#define FX_SHARD_0(X) X(4) X(12) X(27) X(256) X(1296) X(2187)
+#define FX_SHARD_1(X) X(6) X(8) X(81) X(972) X(4096)
+#define FX_SHARD_2(X) X(9) X(24) X(162) X(288) X(2304)
+#define FX_SHARD_3(X) X(16) X(18) X(384) X(512) X(3072)
+#define FX_SHARD_4(X) X(32) X(144) X(1152) X(1458)
+#define FX_SHARD_5(X) X(36) X(432) X(864) X(2916)
+#define FX_SHARD_6(X) X(48) X(96) X(1536) X(3456)
+#define FX_SHARD_7(X) X(54) X(128) X(192) X(3888)
+#define FX_SHARD_8(X) X(64) X(324) X(729) X(1728)
+#define FX_SHARD_9(X) X(72) X(243) X(1944) X(2048)
+#define FX_SHARD_10(X) X(108) X(486) X(1024) X(2592)
+#define FX_SHARD_11(X) X(216) X(576) X(648) X(768)
+
+// Words per lane behind the renormalisations: three per direction of a four-stage transform, before and after the
+// Green product.
+constexpr int kFxSlots = 8;
+
+struct FxPlan {
+  int n, r[4];
+};
+__host__ __device__ constexpr FxPlan fx_plan(int P) {
+  switch (P) {
+#define FX_ROW(P, n, a, b, c, d) \
+  case P: return FxPlan{n, {a, b, c, d}};
+    FX_LENGTHS(FX_ROW)
+#undef FX_ROW
+  }
+  return FxPlan{0, {1, 1, 1, 1}};
+}
+// butterflies of radix R a thread takes: up to 18 values in registers
+__host__ __device__ constexpr int fx_nb(int R) { return R == 9 || R == 6 ? 2 : (R == 3 ? 5 : (R > 8 ? 1 : 16 / R)); }
+// values per thread that every stage of the plan can take: a block has at least P W / fx_ept(P) threads
+__host__ __device__ constexpr int fx_ept(int P) {
+  int e = 18;
+  for (int s = 0; s < fx_plan(P).n; ++s) {
+    const int R = fx_plan(P).r[s], v = R * fx_nb(R);
+    if (v < e) e = v;
+  }
+  return e;
+}
+__host__ __device__ constexpr int fx_prod(int P, int s0, int s1) {
+  int n = 1;
+  for (int s = s0; s < s1; ++s) n *= fx_plan(P).r[s];
+  return n;
+}
+
+}  // namespace flups

@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "fx64.cuh"
 #include "green.cuh"
 
 namespace flups {
@@ -477,6 +478,27 @@ __global__ void k_green_finalize_df(const double* __restrict__ g, float2* __rest
   }
 }
 
+// Fixed-point storage for the FP64-class passes: every pencil along `axis` is aligned to its largest
+// value (|g| < 2^(53 + up)), its exponent kept beside (value = g 2^gexp); one thread per pencil.
+__global__ void k_green_finalize_fx(const double* __restrict__ g, long long* __restrict__ out, int* __restrict__ gexp,
+                                    int gx, int gy, int gz, int gp, int axis, double scale, int up) {
+  const int n0 = axis == 0 ? gy : gx, n1 = axis == 2 ? gy : gz, n = axis == 0 ? gx : (axis == 1 ? gy : gz);
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i >= (long long)n0 * n1) return;
+  const int a = (int)(i % n0), b = (int)(i / n0);
+  long long src, dst, ss, ds;
+  if (axis == 0) { src = (long long)gx * (a + (long long)gy * b); dst = (long long)gp * (a + (long long)gy * b); ss = ds = 1; }
+  else if (axis == 1) { src = a + (long long)gx * gy * b; dst = a + (long long)gp * gy * b; ss = gx; ds = gp; }
+  else { src = a + (long long)gx * b; dst = a + (long long)gp * b; ss = (long long)gx * gy; ds = (long long)gp * gy; }
+  unsigned m = 0;
+  for (int k = 0; k < n; ++k) m = max(m, (unsigned)__double2hiint(g[src + k * ss] * scale) & 0x7fffffffu);
+  const int E = max((int)(m >> 20), kFxMinE);
+  for (int k = 0; k < n; ++k)
+    out[dst + k * ds] =
+        fx_halves(fx_decode((unsigned long long)__double_as_longlong(g[src + k * ss] * scale), E, up));
+  gexp[i] = m ? E - 1075 - up : -(1 << 20);  // a pencil of zeros takes no part in a pair's common exponent
+}
+
 // Fully spectral kernels evaluated in FP64 (stored spectrum of the double-float path):
 // tab[d][g] holds |w_d|^2, or the 7-point symbol for LGF2; G = scale * f(sum_d tab[d][g_d]).
 __global__ void k_green_spectral(double* __restrict__ g, int gx, int gy, int gz, const double* __restrict__ t0,
@@ -542,6 +564,15 @@ cudaError_t launch_green_finalize(const double* g, void* out, int prec, long lon
   if (prec == 0) k_green_finalize<float><<<(unsigned)blocks, 256, 0, st>>>(g, (float*)out, n, gx, gp, scale);
   else if (prec == 2) k_green_finalize_df<<<(unsigned)blocks, 256, 0, st>>>(g, (float2*)out, n, gx, gp, scale);
   else k_green_finalize<double><<<(unsigned)blocks, 256, 0, st>>>(g, (double*)out, n, gx, gp, scale);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_green_finalize_fx(const double* g, void* out, int* gexp, const int* gext, int gp, int axis,
+                                     double scale, bool real_fused, cudaStream_t st) {
+  const long long n = (long long)gext[axis == 0 ? 1 : 0] * gext[axis == 2 ? 1 : 2];
+  k_green_finalize_fx<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(
+      g, (long long*)out, gexp, gext[0], gext[1], gext[2], gp, axis, scale,
+      (real_fused ? kFxGreenBitsReal : kFxGreenBits) - 53);
   return cudaGetLastError();
 }
 

@@ -36,6 +36,8 @@ struct FusedGreen {
   const void* stored;     // stored real spectrum (path precision) or nullptr for closed form
   const void* tab[3];     // closed form: per-direction |w|^2 (or FD symbol) tables, path precision
   int gext[3];            // Green index extents (x, y, z)
+  const int* gexp;        // fixed-point spectrum (FP64-class Poisson passes): exponent of each pencil's slice
+                          // along the fused axis, over the other two Green extents (lower direction fastest)
   int gpitch;             // x pitch of the stored spectrum (elements): gext[0] rounded up to 16 bytes
   int fold[3];            // green index = fold ? min(i, fold - i) : i, for the two non-axis dirs
   int kernel;             // closed-form kernel id (0 spectral, 2..10 HEJ order, 100 LGF2)
@@ -78,6 +80,8 @@ struct PassParams {
                           // copy into shared memory at byte offset rows_off (after the tile) instead of
                           // per-thread loads
   int rows_off;
+  int fx;                 // FP64-class pass in 64-bit fixed point (fx_passes.cu)
+  int fx_host;            // such an x pass reads or writes pinned host memory: whole row pieces per warp
   int pdl;                // launched as a programmatic dependent of the stream's previous kernel: each CTA
                           // waits for the previous grid (complete, memory visible) before touching memory
   // column passes of the compile-time engine: the input tile by TMA (0 rows: loads from registers)
@@ -114,6 +118,10 @@ cudaError_t set_limits_ct_df();
 cudaError_t launch_ct_df_large(int P, int kind, const PassParams& p, dim3 grid, int nthr, size_t smem,
                                cudaStream_t st);
 cudaError_t set_limits_ct_df_large();
+// FP64-class Poisson passes in 64-bit block fixed point
+cudaError_t launch_fx(int kind, const PassParams& p, dim3 grid, int nthr, size_t smem, cudaStream_t st);
+// shared-memory limit of the kernel of that kind and length (per device, set when a plan is made)
+cudaError_t limit_fx(int kind, int P);
 // narrow compile-time tiles for small grids: lanes per tile, 0 when not compiled
 int ct_small_width(int P, int prec);
 cudaError_t launch_ct_small(int prec, int P, int kind, const PassParams& p, dim3 grid, int nthr, size_t smem,

@@ -1,0 +1,76 @@
+// Host-side check of the fixed-point arithmetic (csrc/fx64.cuh, compiled for the CPU; no device code runs):
+// prints the largest errors, in units of the last place, of the register DFTs against long double sums of
+// their definition, of the products against long double products, and of the FP64 decoding; inputs reach the bounds
+// the header states.  One "name value" pair per line.
+#include <cmath>
+#include <complex>
+#include <cstdio>
+#include <cstring>
+#include <random>
+
+#include "fx64.cuh"
+#include "fx_plan.cuh"
+
+using namespace flups;
+using ld = long double;
+using C = std::complex<ld>;
+
+static std::mt19937_64 gen(11);
+static const ld kPi = 3.141592653589793238462643383279502884L;
+static ld uni() { return std::uniform_real_distribution<double>(-1.0, 1.0)(gen); }
+
+template <int R, bool INV> static ld dft_error() {
+  ld worst = 0;
+  for (int t = 0; t < 64; ++t) {
+    cfx v[16];
+    C x[16];
+    for (int i = 0; i < R; ++i) {
+      // bound of a decoded pair; t = 0: every part at it, t = 1: one value only
+      const ld a = t == 0 ? 1 : uni(), b = t == 0 ? -1 : uni();
+      const ld s = t == 1 && i != 1 ? 0 : 0x1.6ap57L;
+      v[i].x = (long long)(a * s);
+      v[i].y = (long long)(b * s);
+      x[i] = C(v[i].x, v[i].y);
+    }
+    fx_dft<R, INV>(v);
+    for (int k = 0; k < R; ++k) {
+      C s = 0;
+      for (int i = 0; i < R; ++i) s += x[i] * std::polar((ld)1, (INV ? 2 : -2) * kPi * (ld)(i * k % R) / R);
+      worst = std::fmax(worst, std::abs(s - C(v[k].x, v[k].y)));
+    }
+  }
+  return worst;
+}
+template <int R> static void dft_line() {
+  std::printf("dft%d %.3Lg\ndft%d_inv %.3Lg\n", R, dft_error<R, false>(), R, dft_error<R, true>());
+}
+
+int main() {
+  dft_line<2>(); dft_line<3>(); dft_line<4>(); dft_line<6>(); dft_line<8>(); dft_line<9>(); dft_line<12>(); dft_line<16>();
+  ld wc = 0, wm = 0, wd = 0;
+  for (int t = 0; t < 20000; ++t) {
+    const ld a = kPi * uni(), ph = kPi * uni(), r = std::pow((ld)2, t % 2 ? 62.5L : 40 + 20 * uni());
+    const long long wr = llroundl(ldexpl(cosl(a), kFxTwBits)), wi = llroundl(ldexpl(-sinl(a), kFxTwBits));
+    const fxw w = {fx_hi(wr), fx_lo(wr), fx_hi(wi), fx_lo(wi)};
+    const cfx x = fx_make((long long)(r * cosl(ph) * 0.999L), (long long)(r * sinl(ph) * 0.999L));
+    const cfx p = fx_cmul<false>(x, w), q = fx_cmul<true>(x, w);
+    wc = std::fmax(wc, std::abs(C(x.x, x.y) * C(wr, wi) / 0x1p64L - C(p.x, p.y)));
+    wc = std::fmax(wc, std::abs(C(x.x, x.y) * C(wr, -wi) / 0x1p64L - C(q.x, q.y)));
+    wm = std::fmax(wm, std::fabs((ld)x.x * wr / 0x1p64L - fx_mul(x.x, w.xh, w.xl)));
+    const double d = std::ldexp((double)uni(), (int)(70 * uni()));
+    const int E = 1023 + 70;
+    unsigned long long b;
+    std::memcpy(&b, &d, 8);
+    wd = std::fmax(wd, std::fabs(ldexpl(d, kFxBias - E) - (ld)fx_decode(b, E)));
+    if (fx_halves(x.x) != (long long)(((unsigned long long)(unsigned)fx_hi(x.x) << 32) | (unsigned)fx_lo(x.x))) return 1;
+    if ((ld)fx_hi(x.x) * 0x1p32L + fx_lo(x.x) != (ld)x.x) return 1;
+  }
+  std::printf("cmul %.3Lg\nmul %.3Lg\ndecode %.3Lg\n", wc, wm, wd);
+  std::printf("zero %lld\nsubnormal %lld\n", fx_decode(0, kFxMinE), fx_decode(0x800fffffffffffffull, kFxMinE));
+  std::printf("shr_even %lld\n", fx_shr(24, 4) * 100 + fx_shr(8, 4) * 10 + fx_shr(7, 0));  // 1.5 -> 2, 0.5 -> 0, 7
+  // every plan multiplies to its length within the block limits
+#define CHECK(P, N, r0, r1, r2, r3) \
+  if (r0 * r1 * r2 * r3 != P || fx_prod(P, 0, fx_plan(P).n) != P || N < 2 || fx_ept(P) < 12 || fx_ept(P) > 18) return 2;
+  FX_LENGTHS(CHECK)
+  return 0;
+}

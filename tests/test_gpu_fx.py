@@ -1,0 +1,84 @@
+"""FP64-class Poisson solves in 64-bit fixed point: every transform length on some axis and direction type
+against the oracle, ragged tiles, and lanes of extreme, zero, infinite and NaN values."""
+import numpy as np
+import pytest
+
+import oracle
+from oracle import CELL, NODE, EVEN as E, ODD as O, PER, UNB as U
+from paper_2211_07777_gb300 import flups as F
+from tests.gpu_util import cuda_solve, rel_linf
+
+pytestmark = pytest.mark.gpu
+
+LENGTHS = sorted({2 ** a * 3 ** b for a in range(13) for b in range(8) if 4 <= 2 ** a * 3 ** b <= 4096})
+# direction types by extension length over cells
+TYPES = {1: [(PER, PER)], 2: [(U, U), (E, E), (O, O)], 4: [(E, O), (O, E), (E, U), (U, O)]}
+
+
+def _cases():
+    out = []
+    for i, P in enumerate(LENGTHS):
+        for m in (1, 2, 4):
+            if P % m or P // m < 4:
+                continue
+            bc = TYPES[m][i % len(TYPES[m])]
+            axis = (i + m) % 3
+            # the other directions: enough points for the fixed-point passes, odd counts of pencils
+            need = 70000 // P
+            small = next(v for v in (8, 9, 12, 16, 18, 24, 27, 36, 54, 72, 96, 128, 162) if v * v >= need)
+            bcs, n = [(PER, PER), (PER, PER)], [small, small]
+            if i % 2:
+                bcs[i % 3 == 0] = (U, U)
+            bcs.insert(axis, bc)
+            n.insert(axis, P // m)
+            out.append((tuple(n), tuple(bcs), NODE if i % 3 == 1 else CELL, P, axis))
+    return out
+
+
+@pytest.mark.parametrize("n,bcs,center,P,axis", _cases(), ids=[f"{c[3]}-{'xyz'[c[4]]}-{c[0][c[4]]}" for c in _cases()])
+def test_every_length_matches_the_oracle(n, bcs, center, P, axis):
+    data = [v + (1 if center == NODE else 0) for v in n]
+    rng = np.random.default_rng(P + axis)
+    f = rng.standard_normal((data[2], data[1], data[0]))
+    h = (1.0 / max(n),) * 3
+    L = tuple(v * h[0] for v in n)
+    kernel = "hej2" if any(U in b for b in bcs) else "spectral"
+    ref = oracle.solve(f, oracle.Problem(bc=bcs, h=h, center=center, kernel=kernel))
+    out, _ = cuda_solve(f, bcs, center, F.F64, kernel, L=L, h=h)
+    assert rel_linf(out, ref) < 1e-13, rel_linf(out, ref)
+
+
+def _solve(f, prec=F.F64):
+    return cuda_solve(f, ((U, U), (E, O), (PER, PER)), CELL, prec, "hej2", h=(1 / 48,) * 3,
+                      L=tuple(v / 48 for v in (48, 32, 36)))[0]
+
+
+def _field(seed=0):
+    return np.random.default_rng(seed).standard_normal((36, 32, 48))
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -800, 2.0 ** -400, 2.0 ** 400, 2.0 ** 900])
+def test_power_of_two_scales_are_exact(scale):
+    a, b = _solve(_field()), _solve(_field() * scale)
+    assert np.array_equal(a * scale, b)
+
+
+def test_rows_of_very_different_size_keep_their_accuracy():
+    f = _field(1) * 10.0 ** np.random.default_rng(2).integers(-12, 1, size=(36, 32, 1))
+    ref = oracle.solve(f, oracle.Problem(bc=((U, U), (E, O), (PER, PER)), h=(1 / 48,) * 3, center=CELL, kernel="hej2"))
+    assert rel_linf(_solve(f), ref) < 1e-14
+
+
+def test_zero_field_gives_zero():
+    assert np.array_equal(_solve(np.zeros((36, 32, 48))), np.zeros((36, 32, 48)))
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_non_finite_input_makes_the_solution_nan(bad):
+    f = _field()
+    f[3, 4, 5] = bad
+    assert np.isnan(_solve(f)).all()
+
+
+def test_both_fp64_precisions_run_the_same_passes():
+    assert np.array_equal(_solve(_field(), F.F64), _solve(_field(), F.F64E))
