@@ -433,18 +433,13 @@ void fill_geom(Launch& L, const DirPlan& dp, int axis, const int* din, const int
   }
 }
 
-// Tile of a fixed-point pass (after fill_geom): about 2048 complex values per CTA (32 KB, 128-192 threads of
-// up to 128 registers, so that four CTAs share an SM), 4096 in the fused complex pass, whose code is the
-// longest: warps of one CTA run the same stretch of it and share its instruction fetches (unbounded 128^3
-// 197 -> 186 us, 192^3 895 -> 840; the other passes 0-8% slower with 4096, all 10-30% slower with 8192).  At
-// least 4 lanes (64 contiguous bytes along x) up to P = 1024; narrower when the grid would leave SMs idle.
+// Tile of a fixed-point pass (after fill_geom): the full width of fx_width, narrower when the grid would leave SMs
+// idle (rows keep their stride).
 void fx_geom(Launch& L, int axis, bool packed) {
   PassParams& p = L.p;
-  const int P = p.P, target = L.kind == K_FUSED_C2C ? 4096 : 2048;
-  int W = 1;
-  while (W < 32 && 2 * W * P <= target) W *= 2;
-  const int wmin = P <= 1024 ? 4 : (P <= 2048 ? 2 : 1);
-  if (W < wmin) W = wmin;
+  const int P = p.P;
+  const bool fused_c2c = L.kind == K_FUSED_C2C;
+  int W = fx_width(fused_c2c, P);
   const int need = packed ? (p.npen + 1) / 2 : p.npen;
   while (W > 1 && W / 2 >= need) W /= 2;
   auto ctas = [&](int w) { return (long long)((need + w - 1) / w) * L.grid.y * L.grid.z; };
@@ -457,7 +452,7 @@ void fx_geom(Launch& L, int axis, bool packed) {
   nt = std::max(32, (nt + 31) / 32 * 32);
   p.W = W;
   p.lw = ilog2(W);
-  p.LS = W == 1 ? 1 : W + 1;
+  p.LS = fx_ls(fused_c2c, P);
   p.fx = 1;
   p.ct = 0;
   p.hz = 0;

@@ -54,16 +54,20 @@ __device__ __forceinline__ unsigned abs_hi(double d) { return (unsigned)__double
 __device__ __forceinline__ long long dec(double d, int E, int up = kFxUp) {
   return fx_decode((unsigned long long)__double_as_longlong(d), E, up);
 }
-// FP64 value of x 2^q rounded to nearest; `kind` (from fx_out_kind) tells NaN lanes and scales outside FP64's
-// normal range.  The conversion runs on the FP64 pipe (measured 1.9 per SM and clock), which is otherwise idle, and
-// the scale joins the exponent field; normalising in integers took 3 times the instructions.
-__device__ __forceinline__ double enc(long long x, int q, int kind) {
+// FP64 value of x 2^q rounded to nearest, for results in FP64's normal range.  The conversion runs on the FP64
+// pipe (measured 1.9 per SM and clock), which is otherwise idle, and the scale joins the exponent field;
+// normalising in integers took 3 times the instructions.
+__device__ __forceinline__ double enc(long long x, int q) {
   const double d = __ll2double_rn(x);
-  if (kind == 0) {
-    const int h = __double2hiint(d);
-    return __hiloint2double(h ? h + (q << 20) : 0, __double2loint(d));
-  }
-  return kind == 1 ? scalbn(d, q) : __longlong_as_double(0x7ff8000000000000ll);
+  const int h = __double2hiint(d);
+  return __hiloint2double(h ? h + (q << 20) : 0, __double2loint(d));
+}
+// the same for any scale (kind 1), or NaN (kind 2); out of line, so that the passes' code stays short
+__device__ __noinline__ double enc_slow(long long x, int q, int kind) {
+  return kind == 1 ? scalbn(__ll2double_rn(x), q) : __longlong_as_double(0x7ff8000000000000ll);
+}
+__device__ __forceinline__ double enc_any(long long x, int q, int kind) {
+  return __builtin_expect(kind == 0, 1) ? enc(x, q) : enc_slow(x, q, kind);
 }
 // 0: every |x| < 2^63 scales to a normal number (or 0); 1: not so; 2: NaN lane
 __device__ __forceinline__ int fx_out_kind(int E, int q) { return E >= 2047 ? 2 : (q > -1020 && q < 950 ? 0 : 1); }
@@ -85,10 +89,31 @@ __device__ __forceinline__ fxw fx_twiddle(const fxw* tw, int i) {
   return w;
 }
 
+template <int N> using ic = std::integral_constant<int, N>;
+
 struct FxTile {
   cfx* S;
-  int W, lw, LS, tid, nt;
+  int W, lw, tid, nt;
   const fxw* tw;
+};
+// Rows of the tile are LS values apart at compile time (fx_ls), so that a butterfly's accesses are offsets
+// from one address; narrower tiles of small grids keep the stride.
+// Values j + r nbf of a butterfly from the tile, and its outputs o + r Ns into it
+template <int LS> struct FxFromS {
+  const cfx* S;
+  template <int R, int nbf> __device__ __forceinline__ void operator()(ic<R>, ic<nbf>, int j, int l, cfx* v) const {
+    const cfx* s = S + j * LS + l;
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = s[r * nbf * LS];
+  }
+};
+template <int LS> struct FxToS {
+  cfx* S;
+  template <int R, int Ns> __device__ __forceinline__ void operator()(ic<R>, ic<Ns>, int o, int l, const cfx* v) const {
+    cfx* s = S + o * LS + l;
+#pragma unroll
+    for (int r = 0; r < R; ++r) s[r * Ns * LS] = v[r];
+  }
 };
 
 // Lane renormalisation.  The fixed factor 2^-4 of a twiddled stage is what the worst case needs; a lane whose
@@ -123,7 +148,8 @@ __device__ __forceinline__ int fx_shifted(const unsigned* words, int W, int l, b
 
 // One stage of radix R after a product Ns of earlier radices.  SRC: FX_RAW, In gives FP64 bits, aligned to the
 // lane's exponent (maxima in `lanes`) here; FX_GAIN, In gives products to renormalise (words `lanes`).  words:
-// the transform's slots; every stage but the first is renormalised.  Out: receives position o of lane l.
+// the transform's slots; every stage but the first is renormalised.  In and Out move whole butterflies: values
+// at positions j + r P/R, outputs at o + r Ns.
 template <int P, int R, int Ns, bool INV, int SRC, bool TO_S, int s, bool SCAN_LAST = false, class In, class Out>
 __device__ __forceinline__ void fx_stage(const FxTile& t, unsigned* lanes, unsigned* words, In in, Out out) {
   constexpr int NB = fx_nb(R), nbf = P / R;
@@ -136,8 +162,7 @@ __device__ __forceinline__ void fx_stage(const FxTile& t, unsigned* lanes, unsig
   for (int b = 0; b < NB; ++b) {
     const int idx = t.tid + b * t.nt, j = idx >> t.lw;
     if (idx < total) {
-#pragma unroll
-      for (int r = 0; r < R; ++r) v[b][r] = in(j + r * nbf, lane);
+      in(ic<R>(), ic<nbf>(), j, lane, v[b]);
     } else {
 #pragma unroll
       for (int r = 0; r < R; ++r) v[b][r] = fx_make(0, 0);
@@ -188,11 +213,10 @@ __device__ __forceinline__ void fx_stage(const FxTile& t, unsigned* lanes, unsig
         for (int r = 1; r < R; ++r) v[b][r] = fx_cmul<INV>(v[b][r], fx_twiddle(t.tw, r * k * tstep));
       }
       fx_dft<R, INV>(v[b]);
-      const int o0 = (j - k) * R + k;
+      out(ic<R>(), ic<Ns>(), (j - k) * R + k, lane, v[b]);
+      if constexpr (SCAN) {
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        out(o0 + r * Ns, lane, v[b][r]);
-        if constexpr (SCAN) mo |= fx_mag(v[b][r].x) | fx_mag(v[b][r].y);
+        for (int r = 0; r < R; ++r) mo |= fx_mag(v[b][r].x) | fx_mag(v[b][r].y);
       }
     }
   }
@@ -202,17 +226,13 @@ __device__ __forceinline__ void fx_stage(const FxTile& t, unsigned* lanes, unsig
 
 // Stages [s, s1) of the plan inside the tile (REV: radices in reverse order); words: the transform's slots.
 // SCAN_LAST: the last stage's outputs are scanned too.
-template <int P, bool INV, bool REV, int s, int s1, bool SCAN_LAST = false>
+template <int P, int LS, bool INV, bool REV, int s, int s1, bool SCAN_LAST = false>
 __device__ __forceinline__ void fx_mid_stages(const FxTile& t, unsigned* words) {
   if constexpr (s < s1) {
     constexpr FxPlan pl = fx_plan(P);
     constexpr int R = pl.r[REV ? pl.n - 1 - s : s], Ns = REV ? fx_prod(P, pl.n - s, pl.n) : fx_prod(P, 0, s);
-    cfx* S = t.S;
-    const int LS = t.LS;
-    fx_stage<P, R, Ns, INV, FX_TILE, true, s, SCAN_LAST>(
-        t, nullptr, words, [=](int i, int l) { return S[i * LS + l]; },
-        [=](int o, int l, const cfx& v) { S[o * LS + l] = v; });
-    fx_mid_stages<P, INV, REV, s + 1, s1, SCAN_LAST>(t, words);
+    fx_stage<P, R, Ns, INV, FX_TILE, true, s, SCAN_LAST>(t, nullptr, words, FxFromS<LS>{t.S}, FxToS<LS>{t.S});
+    fx_mid_stages<P, LS, INV, REV, s + 1, s1, SCAN_LAST>(t, words);
   }
 }
 
@@ -244,10 +264,10 @@ __device__ __forceinline__ void fx_green_base(const PassParams& p, int q, int o,
 
 // Load of real data pairs whose extension is built in the tile (symmetric and semi-unbounded directions, and
 // every real pass on pinned host arrays): items (lane, i < n_data), at most U per thread.
-template <int P, int U>
+template <int P, int LS, int U>
 __device__ __forceinline__ void fx_load_ext(const PassParams& p, const FxTile& t, int type, const double* in, int q0,
                                             int* emax) {
-  const int W = t.W, LS = t.LS, N = p.N, nd = p.n_data, tot = nd * W;
+  const int W = t.W, N = p.N, nd = p.n_data, tot = nd * W;
   const int bt = base_type(type);
   const bool rev = is_reversed(type);
   cfx* S = t.S;
@@ -295,78 +315,98 @@ __device__ __forceinline__ void fx_load_ext(const PassParams& p, const FxTile& t
 }
 
 // Forward transform of real data into the tile: pairs (row q0 + 2l, row q0 + 2l + 1).
-template <int P, bool SCAN_LAST>
+template <int P, int LS, bool SCAN_LAST>
 __device__ __forceinline__ void fx_forward_real(const PassParams& p, const FxTile& t, int type, const double* in,
                                                 int q0, int* emax, unsigned* words) {
-  cfx* S = t.S;
-  const int LS = t.LS;
   constexpr FxPlan pl = fx_plan(P);
-  auto to_s = [=](int o, int l, const cfx& v) { S[o * LS + l] = v; };
   if ((type == T_PER || type == T_UNB) && !p.fx_host) {
     // no images: the first stage reads its positions from memory
     const int nu = p.n_use, npen = p.npen;
     const long long ls = p.ai.ls, js = p.ai.js;
     fx_stage<P, pl.r[0], 1, false, FX_RAW, true, 0>(
         t, reinterpret_cast<unsigned*>(emax), words,
-        [=](int i, int l) {
+        [=](auto R, auto nbf, int j, int l, cfx* v) {
           const int qa = q0 + 2 * l;
-          const double* r = in + (long long)qa * ls + (long long)i * js;
-          cfx v = fx_make(0, 0);
-          if (i < nu && qa < npen) v.x = __double_as_longlong(r[0]);
-          if (i < nu && qa + 1 < npen) v.y = __double_as_longlong(r[ls]);
-          return v;
+          const double* r = in + (long long)qa * ls + (long long)j * js;
+          const long long step = (long long)nbf.value * js;
+          const int la = qa < npen ? nu - j : 0, lb = qa + 1 < npen ? nu - j : 0;
+#pragma unroll
+          for (int k = 0; k < R.value; ++k, r += step)
+            v[k] = fx_make(k * nbf.value < la ? __double_as_longlong(r[0]) : 0,
+                           k * nbf.value < lb ? __double_as_longlong(r[ls]) : 0);
         },
-        to_s);
+        FxToS<LS>{t.S});
   } else {
-    if (p.n_data * t.W <= 9 * t.nt) fx_load_ext<P, 9>(p, t, type, in, q0, emax);
-    else fx_load_ext<P, 19>(p, t, type, in, q0, emax);
-    fx_stage<P, pl.r[0], 1, false, FX_TILE, true, 0>(
-        t, nullptr, words, [=](int i, int l) { return S[i * LS + l]; }, to_s);
+    if (p.n_data * t.W <= 9 * t.nt) fx_load_ext<P, LS, 9>(p, t, type, in, q0, emax);
+    else fx_load_ext<P, LS, 19>(p, t, type, in, q0, emax);
+    fx_stage<P, pl.r[0], 1, false, FX_TILE, true, 0>(t, nullptr, words, FxFromS<LS>{t.S}, FxToS<LS>{t.S});
   }
-  fx_mid_stages<P, false, false, 1, pl.n, SCAN_LAST>(t, words);
+  fx_mid_stages<P, LS, false, false, 1, pl.n, SCAN_LAST>(t, words);
 }
 
-// Store of real data from the tile's last inverse stage; q: exponent of lane l's values.
-template <int P, class Q>
+// Store of real data from the tile's last inverse stage; lane_q(l, &q, &kind): scale of lane l's values.
+template <int P, int LS, class Q>
 __device__ __forceinline__ void fx_store_real(const PassParams& p, const FxTile& t, int type, double* out, int q0,
                                               unsigned* words, Q lane_q) {
   constexpr FxPlan pl = fx_plan(P);
   constexpr int R = pl.r[pl.n - 1], Ns = P / R;
-  cfx* S = t.S;
-  const int LS = t.LS, nd = p.n_data, N = p.N;
+  const int nd = p.n_data, N = p.N;
   const int bt = base_type(type);
   const bool rev = is_reversed(type);
   const bool node = p.center == C_NODE;
   const bool odd0 = node && (bt == T_OO || bt == T_OE || bt == T_OU), oddN = node && (bt == T_OO || bt == T_EO);
+  const bool dup = bt == T_PER && node && nd > N;
   const long long ls = p.ao.ls, js = p.ao.js;
   const int npen = p.npen;
-  auto put = [&](int l, int pos, int i, const cfx& v) {
-    const int qa = q0 + 2 * l;
-    if (qa >= npen) return;
-    int q, kind;
-    lane_q(l, &q, &kind);
-    const bool zero = (odd0 && pos == 0) || (oddN && pos == N);
-    double* o = out + (long long)qa * ls + (long long)i * js;
-    o[0] = zero ? 0.0 : enc(v.x, q, kind);
-    if (qa + 1 < npen) o[ls] = zero ? 0.0 : enc(v.y, q, kind);
-  };
   if (!p.fx_host) {
-    const bool dup = bt == T_PER && node && nd > N;
     fx_stage<P, R, Ns, true, FX_TILE, false, pl.n - 1>(
-        t, nullptr, words, [=](int i, int l) { return S[i * LS + l]; },
-        [&](int o, int l, const cfx& v) {
-          if (o < nd && !(dup && o == N)) put(l, o, rev ? nd - 1 - o : o, v);
-          if (dup && o == 0) put(l, 0, N, v);
+        t, nullptr, words, FxFromS<LS>{t.S}, [&](auto R_, auto Ns_, int o, int l, const cfx* v) {
+          const int qa = q0 + 2 * l;
+          if (qa >= npen) return;
+          int q, kind;
+          lane_q(l, &q, &kind);
+          const bool two = qa + 1 < npen;
+          double* d = out + (long long)qa * ls + (long long)(rev ? nd - 1 - o : o) * js;
+          const long long step = (rev ? -(long long)Ns_.value : (long long)Ns_.value) * js;
+          if (dup && o == 0) {  // phi_N := phi_0
+            d[(long long)N * js] = enc_any(v[0].x, q, kind);
+            if (two) d[(long long)N * js + ls] = enc_any(v[0].y, q, kind);
+          }
+          const int lim = (dup ? N : nd) - o;
+          // odd node faces hold 0
+          const int z0 = odd0 ? -o : -1, zN = oddN ? N - o : -1;
+          if (kind == 0) {
+#pragma unroll
+            for (int r = 0; r < R_.value; ++r, d += step) {
+              if (r * Ns_.value >= lim) continue;
+              const bool z = r * Ns_.value == z0 || r * Ns_.value == zN;
+              d[0] = z ? 0.0 : enc(v[r].x, q);
+              if (two) d[ls] = z ? 0.0 : enc(v[r].y, q);
+            }
+          } else {
+#pragma unroll
+            for (int r = 0; r < R_.value; ++r, d += step) {
+              if (r * Ns_.value >= lim) continue;
+              const bool z = r * Ns_.value == z0 || r * Ns_.value == zN;
+              d[0] = z ? 0.0 : enc_slow(v[r].x, q, kind);
+              if (two) d[ls] = z ? 0.0 : enc_slow(v[r].y, q, kind);
+            }
+          }
         });
     return;
   }
-  fx_stage<P, R, Ns, true, FX_TILE, true, pl.n - 1>(
-      t, nullptr, words, [=](int i, int l) { return S[i * LS + l]; },
-      [=](int o, int l, const cfx& v) { S[o * LS + l] = v; });
+  fx_stage<P, R, Ns, true, FX_TILE, true, pl.n - 1>(t, nullptr, words, FxFromS<LS>{t.S}, FxToS<LS>{t.S});
   for (int idx = t.tid; idx < nd * t.W; idx += t.nt) {
-    const int l = idx / nd, i = idx % nd;
-    const int pos = (bt == T_PER && node && i == N) ? 0 : (rev ? nd - 1 - i : i);
-    put(l, pos, i, S[pos * LS + l]);
+    const int l = idx / nd, i = idx % nd, qa = q0 + 2 * l;
+    if (qa >= npen) continue;
+    const int pos = dup && i == N ? 0 : (rev ? nd - 1 - i : i);
+    const bool zero = (odd0 && pos == 0) || (oddN && pos == N);
+    const cfx v = t.S[pos * LS + l];
+    int q, kind;
+    lane_q(l, &q, &kind);
+    double* d = out + (long long)qa * ls + (long long)i * js;
+    d[0] = zero ? 0.0 : enc_any(v.x, q, kind);
+    if (qa + 1 < npen) d[ls] = zero ? 0.0 : enc_any(v.y, q, kind);
   }
 }
 
@@ -376,19 +416,19 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr bool REAL = KIND == K_FWD_REAL || KIND == K_INV_REAL || KIND == K_FUSED_REAL;
   constexpr bool FUSED = KIND == K_FUSED_REAL || KIND == K_FUSED_C2C;
-  const FxSmem m = fx_smem(smraw, P, p.W, p.LS);
+  constexpr int LS = fx_ls(KIND == K_FUSED_C2C, P);
+  const FxSmem m = fx_smem(smraw, P, p.W, LS);
   const int tid = threadIdx.x, nt = blockDim.x;
   FxTile t;
   t.S = m.S;
   t.W = p.W;
   t.lw = p.lw;
-  t.LS = p.LS;
   t.tid = tid;
   t.nt = nt;
   t.tw = (const fxw*)p.tw;
   constexpr FxPlan pl = fx_plan(P);
   constexpr int ns = pl.n, half = P / 2, R0 = pl.r[0], RL = pl.r[ns - 1];
-  const int W = p.W, LS = p.LS;
+  const int W = p.W;
   cfx* S = m.S;
   const int q0 = blockIdx.x * (REAL ? 2 * W : W);
   // fused pass: rows o and n - o share a Green slice and run back to back
@@ -424,11 +464,11 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
   }
   // exponent of a fixed-point value of lane l after the forward (or a single inverse) transform
   constexpr int shift = kFxTwShift * (ns - 1) - kFxBias;
-  auto from_s = [=](int i, int l) { return S[i * LS + l]; };
-  auto to_s = [=](int i, int l, const cfx& v) { S[i * LS + l] = v; };
+  const FxFromS<LS> from_s{S};
+  const FxToS<LS> to_s{S};
 
   if constexpr (KIND == K_FWD_REAL) {
-    fx_forward_real<P, false>(p, t, type, (const double*)p.in + bi, q0, m.emax, wf);
+    fx_forward_real<P, LS, false>(p, t, type, (const double*)p.in + bi, q0, m.emax, wf);
     const int bt = base_type(type);
     const bool cplx = bt == T_PER || bt == T_UNB, quarter = is_quarter(bt), oddo = is_odd_origin(bt);
     const bool cell = p.center == C_CELL;
@@ -446,8 +486,8 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
         const long long off = bo + (long long)qa * p.ao.ls + (long long)k * p.ao.js;
         if (cplx) {
           double2* out = (double2*)p.out;
-          out[off] = make_double2(enc(A.x, q, kind), enc(A.y, q, kind));
-          if (two) out[off + p.ao.ls] = make_double2(enc(B.x, q, kind), enc(B.y, q, kind));
+          out[off] = make_double2(enc_any(A.x, q, kind), enc_any(A.y, q, kind));
+          if (two) out[off + p.ao.ls] = make_double2(enc_any(B.x, q, kind), enc_any(B.y, q, kind));
         } else {
           double* out = (double*)p.out;
           if (cell) {
@@ -455,8 +495,8 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
             A = fx_cmul<false>(A, w);
             B = fx_cmul<false>(B, w);
           }
-          out[off] = enc(oddo ? -A.y : A.x, q, kind);
-          if (two) out[off + p.ao.ls] = enc(oddo ? -B.y : B.x, q, kind);
+          out[off] = enc_any(oddo ? -A.y : A.x, q, kind);
+          if (two) out[off + p.ao.ls] = enc_any(oddo ? -B.y : B.x, q, kind);
         }
       }
     }
@@ -527,15 +567,15 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
     }
     __syncthreads();
     fx_stage<P, R0, 1, true, FX_TILE, true, 0>(t, nullptr, wi, from_s, to_s);
-    fx_mid_stages<P, true, false, 1, ns - 1>(t, wi);
+    fx_mid_stages<P, LS, true, false, 1, ns - 1>(t, wi);
     const int add = shift + (quarter ? 1 : 0);
-    fx_store_real<P>(p, t, type, (double*)p.out + bo, q0, wi, [&](int lane, int* q, int* kind) {
+    fx_store_real<P, LS>(p, t, type, (double*)p.out + bo, q0, wi, [&](int lane, int* q, int* kind) {
       const int Ee = max(m.emax[lane], kFxMinE);
       *q = Ee + add - fx_shifted<P>(m.words, W, lane, false, false, true);
       *kind = fx_out_kind(Ee, *q);
     });
   } else if constexpr (KIND == K_FUSED_REAL) {
-    fx_forward_real<P, true>(p, t, type, (const double*)p.in + bi, q0, m.emax, wf);
+    fx_forward_real<P, LS, true>(p, t, type, (const double*)p.in + bi, q0, m.emax, wf);
     const bool quarter = is_quarter(base_type(type));
     unsigned mo = 0;
     {
@@ -569,13 +609,14 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
     const int up = fx_free_in(wg[tid & (W - 1)]);
     fx_stage<P, R0, 1, true, FX_TILE, true, 0>(
         t, nullptr, wi,
-        [=](int i, int l) {
-          const cfx z = S[i * LS + l];
-          return fx_make(z.x << up, z.y << up);
+        [=](auto R, auto nbf, int j, int l, cfx* v) {
+          from_s(R, nbf, j, l, v);
+#pragma unroll
+          for (int r = 0; r < R.value; ++r) v[r] = fx_make(v[r].x << up, v[r].y << up);
         },
         to_s);
-    fx_mid_stages<P, true, false, 1, ns - 1>(t, wi);
-    fx_store_real<P>(p, t, type, (double*)p.out + bo, q0, wi, [&](int lane, int* q, int* kind) {
+    fx_mid_stages<P, LS, true, false, 1, ns - 1>(t, wi);
+    fx_store_real<P, LS>(p, t, type, (double*)p.out + bo, q0, wi, [&](int lane, int* q, int* kind) {
       const int Ee = max(m.emax[lane], kFxMinE);
       *q = Ee - fx_shifted<P>(m.words, W, lane, true, true, true) + 2 * shift + kFxBias - 1 + 64 + max(m.gexp[2 * lane], m.gexp[2 * lane + 1]);
       *kind = fx_out_kind(Ee, *q);
@@ -586,28 +627,42 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
     double2* out = (double2*)p.out + bo;
     const int npen = p.npen, n_in = KIND == K_INV_C2C ? P : p.n_use;
     const long long ils = p.ai.ls, ijs = p.ai.js, ols = p.ao.ls, ojs = p.ao.js;
-    auto load = [=](int i, int l) {
-      cfx v = fx_make(0, 0);
-      if (i < n_in && q0 + l < npen) {
-        const longlong2 c = *reinterpret_cast<const longlong2*>(&in[(long long)(q0 + l) * ils + (long long)i * ijs]);
-        v = fx_make(c.x, c.y);
+    auto load = [=](auto R, auto nbf, int j, int l, cfx* v) {
+      const longlong2* c = reinterpret_cast<const longlong2*>(in) + (long long)(q0 + l) * ils + (long long)j * ijs;
+      const long long step = (long long)nbf.value * ijs;
+      const int lim = q0 + l < npen ? n_in - j : 0;
+#pragma unroll
+      for (int r = 0; r < R.value; ++r, c += step) {
+        longlong2 x = make_longlong2(0, 0);
+        if (r * nbf.value < lim) x = *c;
+        v[r] = fx_make(x.x, x.y);
       }
-      return v;
     };
     const int l0 = tid & (W - 1);
     const int n_out = KIND == K_FWD_C2C ? P : p.n_data;
+    // node-centred periodic: phi_N := phi_0
     const int dup = (KIND != K_FWD_C2C && p.type == T_PER && p.center == C_NODE && p.n_data > p.N) ? p.N : -1;
     int q = 0, kind = 0;
     bool store_ok = true;
-    auto store = [&](int i, int l, const cfx& v) {
+    auto store = [&](auto R, auto Ns, int o, int l, const cfx* v) {
       if (q0 + l >= npen || !store_ok) return;
-      const double2 d = make_double2(enc(v.x, q, kind), enc(v.y, q, kind));
-      if (i < n_out && i != dup) out[(long long)(q0 + l) * ols + (long long)i * ojs] = d;
-      if (i == 0 && dup >= 0) out[(long long)(q0 + l) * ols + (long long)dup * ojs] = d;
+      double2* d = out + (long long)(q0 + l) * ols + (long long)o * ojs;
+      const long long step = (long long)Ns.value * ojs;
+      const int lim = n_out - o;
+      if (dup >= 0 && o == 0) d[(long long)dup * ojs] = make_double2(enc_any(v[0].x, q, kind), enc_any(v[0].y, q, kind));
+      if (kind == 0) {
+#pragma unroll
+        for (int r = 0; r < R.value; ++r, d += step)
+          if (r * Ns.value < lim) *d = make_double2(enc(v[r].x, q), enc(v[r].y, q));
+      } else {
+#pragma unroll
+        for (int r = 0; r < R.value; ++r, d += step)
+          if (r * Ns.value < lim) *d = make_double2(enc_slow(v[r].x, q, kind), enc_slow(v[r].y, q, kind));
+      }
     };
     if constexpr (KIND == K_FUSED_C2C) {
       fx_stage<P, R0, 1, false, FX_RAW, true, 0>(t, emax, wf, load, to_s);
-      fx_mid_stages<P, false, false, 1, ns, true>(t, wf);
+      fx_mid_stages<P, LS, false, false, 1, ns, true>(t, wf);
       // u^ = G^ f^ in the first inverse stage (radices reversed)
       if (tma_g) {
         if (!mbar_wait_bounded(m.mbar, p.errflag, 1, p.dbg_wait & 1)) store_ok = false;
@@ -617,15 +672,23 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
       const long long* G = (const long long*)p.g.stored + go;
       const long long* Gs = m.G;
       const int upx = fx_free_tw(wf[(ns - 1) * W + l0]);
-      auto gained = [=](int i, int l) {
-        const cfx z = S[i * LS + l];
-        const int g3 = min(i, P - i);
-        const long long g = tma_g ? Gs[g3 * W + l] : __ldg(&G[g3 * st3]);
-        const int gh = (int)(g >> 32), gl = (int)g;
-        return fx_make(fx_mul(z.x << upx, gh, gl), fx_mul(z.y << upx, gh, gl));
+      auto gained = [=](auto R, auto nbf, int j, int l, cfx* v) {
+        from_s(R, nbf, j, l, v);
+        // folded mode of position i = j + r nbf: i in the lower half, P - i in the upper one
+        const long long* g = tma_g ? Gs + l : G;
+        const long long gs = tma_g ? (long long)W : st3;
+        const long long *lo = g + j * gs, *hi = g + (P - j) * gs;
+        const long long step = nbf.value * gs;
+#pragma unroll
+        for (int r = 0; r < R.value; ++r) {
+          const bool low = 2 * (r + 1) <= R.value || (2 * r < R.value && 2 * (j + r * nbf.value) <= P);
+          const long long x = low ? lo[r * step] : hi[-(r * step)];
+          const int gh = (int)(x >> 32), gl = (int)x;
+          v[r] = fx_make(fx_mul(v[r].x << upx, gh, gl), fx_mul(v[r].y << upx, gh, gl));
+        }
       };
       fx_stage<P, RL, 1, true, FX_GAIN, true, 0>(t, wg, wi, gained, to_s);
-      fx_mid_stages<P, true, true, 1, ns - 1>(t, wi);
+      fx_mid_stages<P, LS, true, true, 1, ns - 1>(t, wi);
       const int E = max(m.emax[l0], kFxMinE);
       q = E - fx_shifted<P>(m.words, W, l0, true, true, true) + 2 * shift + kFxBias + 64 + m.gexp[l0];
       kind = fx_out_kind(E, q);
@@ -633,7 +696,7 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
     } else {
       constexpr bool INV = KIND == K_INV_C2C;
       fx_stage<P, R0, 1, INV, FX_RAW, true, 0>(t, emax, wf, load, to_s);
-      fx_mid_stages<P, INV, false, 1, ns - 1>(t, wf);
+      fx_mid_stages<P, LS, INV, false, 1, ns - 1>(t, wf);
       const int E = max(m.emax[l0], kFxMinE);
       q = E + shift - fx_shifted<P>(m.words, W, l0, true, false, false);
       kind = fx_out_kind(E, q);

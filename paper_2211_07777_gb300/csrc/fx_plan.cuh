@@ -102,6 +102,21 @@ __host__ __device__ constexpr int fx_ept(int P) {
   }
   return e;
 }
+// Lanes of a full tile and the stride of its rows: about 2048 complex values per CTA (32 KB, 128-192 threads of up
+// to 128 registers, so that four CTAs share an SM), 4096 in the fused complex pass, whose code is the longest:
+// warps of one CTA run the same stretch of it and share its instruction fetches (unbounded 128^3 197 -> 186 us,
+// 192^3 895 -> 840; the other passes 0-8% slower with 4096, all 10-30% slower with 8192).  At least 4 lanes
+// (64 contiguous bytes along x) up to P = 1024.
+__host__ __device__ constexpr int fx_width(bool fused_c2c, int P) {
+  int W = 1;
+  while (W < 32 && 2 * W * P <= (fused_c2c ? 4096 : 2048)) W *= 2;
+  const int wmin = P <= 1024 ? 4 : (P <= 2048 ? 2 : 1);
+  return W < wmin ? wmin : W;
+}
+__host__ __device__ constexpr int fx_ls(bool fused_c2c, int P) {
+  const int W = fx_width(fused_c2c, P);
+  return W == 1 ? 1 : W + 1;
+}
 __host__ __device__ constexpr int fx_prod(int P, int s0, int s1) {
   int n = 1;
   for (int s = s0; s < s1; ++s) n *= fx_plan(P).r[s];
