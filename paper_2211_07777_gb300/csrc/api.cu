@@ -105,6 +105,7 @@ struct DirPlan {
   double h = 0, L = 0, wscale = 0, wshift = 0;
   RadixPlan rp{};
   void* tw = nullptr;
+  void* tw2 = nullptr;  // of the FP32 lane-pair passes
 };
 
 struct Launch {
@@ -210,6 +211,23 @@ static int make_twiddles_uncached(int P, int prec, void** out) {
   return FLUPS_OK;
 }
 
+// Twiddles c - i s = exp(-2 pi i m/(2P)) of the FP32 lane-pair passes: (c, c, s, s).
+constexpr int kF2Tables = 4;
+int make_twiddles_f2(int P, void** out) {
+  const int M = 2 * P;
+  std::vector<float> h((size_t)4 * M);
+  for (int m = 0; m < M; ++m) {
+    const long double a = 3.141592653589793238462643383279502884L * (long double)m / (long double)P;
+    h[4 * m] = h[4 * m + 1] = (float)cosl(a);
+    h[4 * m + 2] = h[4 * m + 3] = (float)sinl(a);
+  }
+  void* d = nullptr;
+  CK(cudaMalloc(&d, (size_t)M * 16));
+  CK(cudaMemcpy(d, h.data(), (size_t)M * 16, cudaMemcpyHostToDevice));
+  *out = d;
+  return FLUPS_OK;
+}
+
 // Twiddles of the fixed-point passes, exp(-2 pi i m/(2P)) 2^60 in signed 32-bit halves (fx64.cuh).
 constexpr int kFxTables = 3;  // their key beside the precisions
 int make_twiddles_fx(int P, void** out) {
@@ -247,7 +265,8 @@ int make_twiddles(int P, int prec, void** out) {
     return FLUPS_OK;
   }
   void* d = nullptr;
-  const int rc = prec == kFxTables ? make_twiddles_fx(P, &d) : make_twiddles_uncached(P, prec, &d);
+  const int rc = prec == kFxTables ? make_twiddles_fx(P, &d)
+                 : prec == kF2Tables ? make_twiddles_f2(P, &d) : make_twiddles_uncached(P, prec, &d);
   if (rc) return rc;
   g_tw_cache[key] = d;
   *out = d;
@@ -452,7 +471,6 @@ void fx_geom(Launch& L, int axis, bool packed) {
   nt = std::max(32, (nt + 31) / 32 * 32);
   p.W = W;
   p.lw = ilog2(W);
-  p.LS = fx_ls(fused_c2c, P);
   p.fx = 1;
   p.ct = 0;
   p.hz = 0;
@@ -460,9 +478,51 @@ void fx_geom(Launch& L, int axis, bool packed) {
   L.grid.x = (unsigned)((need + W - 1) / W);
   L.nthr = nt;
   // alignment, mbarrier block, tile, Green offsets and exponents, lane exponents, renormalisation words
-  L.smem = 128 + 128 + (size_t)P * p.LS * 16 + (size_t)W * (2 * 8 + 4 + 2 * 4 + kFxSlots * 4);
+  L.smem = 128 + 128 + (size_t)fx_tile_values(fused_c2c, P) * 16 + (size_t)W * (2 * 8 + 4 + 2 * 4 + kFxSlots * 4);
   p.rowx = (axis == 0 && p.center == C_CELL && (p.type == T_PER || p.type == T_UNB) &&
             (L.kind == K_FWD_REAL || L.kind == K_INV_REAL)) ? 1 : 0;
+}
+
+// Tile of an FP32 lane-pair pass (after fill_geom): as fx_geom, a lane holding two complex or four real pencils.
+void f2_geom(Launch& L, const DirPlan& dp, int axis, bool packed) {
+  PassParams& p = L.p;
+  const int P = p.P, per = packed ? 4 : 2;
+  int W = fx_width(false, P);
+  const int need = (p.npen + per - 1) / per;
+  while (W > 1 && W / 2 >= need) W /= 2;
+  auto ctas = [&](int w) { return (long long)((need + w - 1) / w) * L.grid.y * L.grid.z; };
+  while (W > 1 && ctas(W) < 2 * 152 && W * P >= 512) W /= 2;
+  const int ept = fx_ept(P);
+  int nt = (P * W + ept - 1) / ept;
+  if (ctas(W) * nt < 152 * 256) nt = std::max(nt, std::min(256, P * W / 4));
+  nt = std::max(32, (nt + 31) / 32 * 32);
+  p.W = W;
+  p.lw = ilog2(W);
+  p.f2 = 1;
+  p.rowx = (axis == 0 && p.center == C_CELL && (p.type == T_PER || p.type == T_UNB) &&
+            (L.kind == K_FWD_REAL || L.kind == K_INV_REAL)) ? 1 : 0;
+  p.ct = 0;
+  p.hz = 0;
+  p.ept = 0;
+  p.tw = dp.tw2;
+  L.grid.x = (unsigned)((need + W - 1) / W);
+  L.nthr = nt;
+  L.smem = 128 + 128 + (size_t)fx_tile_values(false, P) * 16 + (size_t)W * (4 * 8 + 4 * 4);
+}
+
+// 16-byte accesses of a lane-pair pass: pencils adjacent in memory, rows and base 16-byte aligned.
+void set_f2_vec(PassParams& p, int kind) {
+  p.f2_vec = 0;
+  if (!p.f2 || p.axis == 0) return;
+  const int t = p.ctypes & 15;
+  const bool modes = t == T_PER || t == T_UNB;  // complex modes (the components share the family)
+  auto ok = [&](const void* ptr, const ArrDesc& a, bool cplx) {
+    const long long v = cplx ? 2 : 4;
+    return ((uintptr_t)ptr & 15) == 0 && a.ls == 1 && a.js % v == 0 && a.os % v == 0 && a.cs % v == 0;
+  };
+  const bool c2c = kind == K_FWD_C2C || kind == K_INV_C2C || kind == K_FUSED_C2C;
+  if (ok(p.in, p.ai, c2c || (kind == K_INV_REAL && modes))) p.f2_vec |= 1;
+  if (ok(p.out, p.ao, c2c || (kind == K_FWD_REAL && modes))) p.f2_vec |= 2;
 }
 
 // CTAs per SM the compile-time kernels are built for (their __launch_bounds__ minimum).
@@ -890,7 +950,7 @@ void encode_input_map(Launch& L, int prec) {
 // wavefronts on bank conflicts (unbounded 512x256x256 FP32 under ncu).
 void set_rowx(Launch& L, int prec) {
   PassParams& p = L.p;
-  if (p.fx) return;
+  if (p.fx || p.f2) return;
   p.rowx = 0;
   if (!p.ct || p.axis != 0 || (prec != FLUPS_F32 && prec != FLUPS_F64E) || p.W != 4 || p.center != C_CELL) return;
   if (L.kind != K_FWD_REAL && L.kind != K_INV_REAL) return;
@@ -934,6 +994,27 @@ void set_rows_bulk(Launch& L, int prec) {
   L.smem = total;
 }
 
+// FP32 passes on pairs of lanes in packed arithmetic (f2_passes.cu) or on the kernels of pass_kernels.cuh, by
+// measurement on GB300 (us per pass, old / lane pairs):
+// - lengths with a factor 3, which had only the runtime-shaped tiles: always (192^3: 473 / 238 fused, 104 / 59
+//   complex, 150-200 / 60-75 symmetric; 48^3 fused 16 / 14);
+// - powers of two: real passes along y or z (256-point periodic 78 / 64 and 76 / 53) and symmetric ones along
+//   x (512 points: 90 / 86 and 123 / 82); x passes of periodic and unbounded data up to 128 points (20 / 12,
+//   23 / 16; 256 points 51 / 58 and 47 / 88), the forward one also at 512 (76 / 74), while 1024 and 2048 points have
+//   their register-chained row kernels;
+// - complex passes of powers of two: never (256 points 14 / 16, fused 31 / 47; 1024 points fused 1912 / 3077): the
+//   column kernels prefetch their tiles by TMA and hold twice the warps.
+bool use_f2(const flups_solver_s* s, const Launch& L, const DirPlan& dp, int axis) {
+  if (s->topo.prec != FLUPS_F32) return false;
+  const int P = dp.P;
+  if (P & (P - 1)) return true;
+  if (L.kind == K_FUSED_REAL) return true;
+  if (L.kind != K_FWD_REAL && L.kind != K_INV_REAL) return false;
+  const bool modes = dp.type == T_PER || dp.type == T_UNB;
+  if (axis != 0 || !modes) return true;
+  return P <= 128 || (P == 512 && L.kind == K_FWD_REAL);
+}
+
 int build_passes(flups_solver_s* s, cudaStream_t st) {
   const int prec = s->topo.prec, center = s->topo.center, nc = s->topo.ncomp;
   const int* o = s->order;
@@ -957,6 +1038,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     fill_geom(L, s->dir[o[0]], o[0], s->dims[0], s->dims[1], prec, true, center, nc, 1, s->pitch[0], s->pitch[1]);
     L.p.ctypes = pack3(s->tf[0][o[0]], s->tf[1][o[0]], s->tf[2][o[0]]);
     if (s->fx) fx_geom(L, o[0], true);
+    else if (use_f2(s, L, s->dir[o[0]], o[0])) f2_geom(L, s->dir[o[0]], o[0], true);
     L.p.out = s->W1;
     L.out_buf = 1;
     L.user_in = 1;
@@ -974,6 +1056,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     fill_geom(L, s->dir[o[1]], o[1], s->dims[1], s->dims[2], prec, real, center, nc, 1, s->pitch[1], s->pitch[2]);
     L.p.ctypes = pack3(s->tf[0][o[1]], s->tf[1][o[1]], s->tf[2][o[1]]);
     if (s->fx) fx_geom(L, o[1], real);
+    else if (use_f2(s, L, s->dir[o[1]], o[1])) f2_geom(L, s->dir[o[1]], o[1], real);
     L.p.in = s->W1;
     L.p.out = s->W2;
     L.in_buf = 1;
@@ -994,6 +1077,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
               s->pitch[2]);
     L.p.ctypes = pack3(s->tf[0][o[2]], s->tf[1][o[2]], s->tf[2][o[2]]);
     if (s->fx) fx_geom(L, o[2], real);
+    else if (!curl && use_f2(s, L, dp, o[2])) f2_geom(L, dp, o[2], real);
     L.p.in = s->W2;
     L.p.out = s->W2;
     L.in_buf = 2;
@@ -1034,13 +1118,14 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
           L.p.gmap = s->gmaps_dev;
       }
     }
-    if (s->fx && !real && o[2] != 0 && dp.gext == dp.P / 2 + 1 && g.fold[0] == 0) {
-      // fixed-point fused column pass: the Green slice by TMA while the forward transform runs, where
+    if ((L.p.fx || L.p.f2) && !real && o[2] != 0 && g.stored && dp.gext == dp.P / 2 + 1 && g.fold[0] == 0) {
+      // fused column pass of the fixed-point or lane-pair kernels: the Green slice by TMA while the forward transform runs, where
       // two CTAs still fit an SM with it
-      const size_t gbytes = 128 + (size_t)L.p.W * (dp.P / 2 + 1) * sizeof(long long);
+      const int gw = L.p.f2 ? 2 * L.p.W : L.p.W;
+      const size_t gbytes = 128 + (size_t)gw * (dp.P / 2 + 1) * es;
       // (the slice's last row is a copy of its own, which must start on 128 bytes)
-      if (2 * (L.smem + gbytes + 1024) <= 228 * 1024 && (size_t)(dp.P / 2) * L.p.W * sizeof(long long) % 128 == 0 &&
-          green_tensor_maps(s, o[2], L.p.W, dp.P, prec, &L.p.gbox, st)) {
+      if (2 * (L.smem + gbytes + 1024) <= 228 * 1024 && (size_t)(dp.P / 2) * gw * es % 128 == 0 &&
+          green_tensor_maps(s, o[2], gw, dp.P, prec, &L.p.gbox, st)) {
         L.smem += gbytes;
         L.p.gpre = 1;
         L.p.gmap = s->gmaps_dev;
@@ -1065,6 +1150,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     fill_geom(L, s->dir[o[1]], o[1], s->dims[2], s->dims[1], prec, real, center, nc, 1, s->pitch[2], s->pitch[1]);
     L.p.ctypes = pack3(s->tu[0][o[1]], s->tu[1][o[1]], s->tu[2][o[1]]);
     if (s->fx) fx_geom(L, o[1], real);
+    else if (use_f2(s, L, s->dir[o[1]], o[1])) f2_geom(L, s->dir[o[1]], o[1], real);
     L.p.in = s->W2;
     L.p.out = s->W1;
     L.in_buf = 2;
@@ -1081,6 +1167,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     fill_geom(L, s->dir[o[0]], o[0], s->dims[1], s->dims[0], prec, true, center, nc, 1, s->pitch[1], s->pitch[0]);
     L.p.ctypes = pack3(s->tu[0][o[0]], s->tu[1][o[0]], s->tu[2][o[0]]);
     if (s->fx) fx_geom(L, o[0], true);
+    else if (use_f2(s, L, s->dir[o[0]], o[0])) f2_geom(L, s->dir[o[0]], o[0], true);
     L.p.in = s->W1;
     L.in_buf = 1;
     L.user_out = 1;
@@ -1094,8 +1181,10 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
   for (Launch& L : s->passes) set_rowx(L, prec);  // before set_rows_bulk (flups_setup): the staged rows follow the tile
   for (const Launch& L : s->passes)
     if (L.smem > 227 * 1024 || L.nthr > 1024) return FLUPS_ESIZE;
-  if (s->fx)
-    for (const Launch& L : s->passes) CK(limit_fx(L.kind, L.p.P));
+  for (const Launch& L : s->passes) {
+    if (L.p.fx) CK(limit_fx(L.kind, L.p.P));
+    if (L.p.f2) CK(limit_f2(L.kind, L.p.P));
+  }
   return FLUPS_OK;
 }
 
@@ -1276,6 +1365,7 @@ int flups_setup(flups_solver s, void* stream, size_t* workspace_bytes) {
   }
   for (int d = 0; d < 3; ++d) {
     int rc = make_twiddles(s->dir[d].P, s->fx ? kFxTables : prec, &s->dir[d].tw);
+    if (!rc && prec == FLUPS_F32) rc = make_twiddles(s->dir[d].P, kF2Tables, &s->dir[d].tw2);
     if (rc) return rc;
     s->ws_bytes += (size_t)4 * s->dir[d].P * es;
   }
@@ -1345,7 +1435,8 @@ static int solve_impl(flups_solver s, void* phi, const void* rhs, void* ws, void
       encode_input_map(Lw, prec);
       set_rows_bulk(Lw, prec);
     }
-    if (p.fx) p.fx_host = p.axis == 0 && ((L.user_in && host_in) || (L.user_out && host_out));
+    set_f2_vec(p, L.kind);
+    if (p.fx || p.f2) p.fx_host = p.axis == 0 && ((L.user_in && host_in) || (L.user_out && host_out));
     else if (p.rowx && ((L.user_in && host_in) || (L.user_out && host_out))) {
       p.rowx = 0;
       Lw.nthr = L.gnthr;
@@ -1485,6 +1576,7 @@ int flups_solve_pass(flups_solver s, int i, void* phi, const void* rhs, void* st
   p.dbg_wait = s->dbg_wait;
   if (L.user_in) p.in = rhs;
   if (L.user_out) p.out = phi;
+  set_f2_vec(p, L.kind);
   cudaError_t e = L.kind >= K_CURL_REAL
                       ? launch_curl(L.kind, s->topo.prec, p, L.grid, L.nthr, L.smem, (cudaStream_t)stream)
                       : launch_pass(L.kind, s->topo.prec, p, L.grid, L.nthr, L.smem, (cudaStream_t)stream);

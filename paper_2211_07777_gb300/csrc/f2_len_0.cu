@@ -1,0 +1,4 @@
+// FP32 lane-pair passes of the lengths of FX_SHARD_0.
+#include "f2_kernels.cuh"
+
+F2_UNIT(0)

@@ -36,12 +36,12 @@ struct FxSmem {
   long long* G;       // staged slice, (P/2 + 1) x W
 };
 
-__device__ __forceinline__ FxSmem fx_smem(unsigned char* smraw, int P, int W, int LS) {
+__device__ __forceinline__ FxSmem fx_smem(unsigned char* smraw, int W, int rows) {
   FxSmem m;
   unsigned char* base = smraw + ((128u - (smem_u32(smraw) & 127u)) & 127u);
   m.mbar = reinterpret_cast<unsigned long long*>(base);
   m.S = reinterpret_cast<cfx*>(base + 128);
-  m.goff = reinterpret_cast<long long*>(base + 128 + (size_t)P * LS * sizeof(cfx));
+  m.goff = reinterpret_cast<long long*>(base + 128 + (size_t)rows * sizeof(cfx));
   m.emax = reinterpret_cast<int*>(m.goff + 2 * W);
   m.gexp = m.emax + W;
   m.words = reinterpret_cast<unsigned*>(m.gexp + 2 * W);
@@ -96,23 +96,29 @@ struct FxTile {
   int W, lw, tid, nt;
   const fxw* tw;
 };
-// Rows of the tile are LS values apart at compile time (fx_ls), so that a butterfly's accesses are offsets
+// Rows of the tile are a compile-time number of values apart (FxRows), so that a butterfly's accesses are offsets
 // from one address; narrower tiles of small grids keep the stride.
 // Values j + r nbf of a butterfly from the tile, and its outputs o + r Ns into it
-template <int LS> struct FxFromS {
+template <class RW> struct FxFromS {
   const cfx* S;
   template <int R, int nbf> __device__ __forceinline__ void operator()(ic<R>, ic<nbf>, int j, int l, cfx* v) const {
-    const cfx* s = S + j * LS + l;
+    const cfx* s = S + RW::at(j) + l;
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = s[r * nbf * LS];
+    for (int r = 0; r < R; ++r) {
+      if constexpr (RW::linear(nbf)) v[r] = s[RW::at(r * nbf)];
+      else v[r] = S[RW::at(j + r * nbf) + l];
+    }
   }
 };
-template <int LS> struct FxToS {
+template <class RW> struct FxToS {
   cfx* S;
   template <int R, int Ns> __device__ __forceinline__ void operator()(ic<R>, ic<Ns>, int o, int l, const cfx* v) const {
-    cfx* s = S + o * LS + l;
+    cfx* s = S + RW::at(o) + l;
 #pragma unroll
-    for (int r = 0; r < R; ++r) s[r * Ns * LS] = v[r];
+    for (int r = 0; r < R; ++r) {
+      if constexpr (RW::linear(Ns) || (Ns == 1 && R == RW::B)) s[RW::at(r * Ns)] = v[r];
+      else S[RW::at(o + r * Ns) + l] = v[r];
+    }
   }
 };
 
@@ -226,13 +232,13 @@ __device__ __forceinline__ void fx_stage(const FxTile& t, unsigned* lanes, unsig
 
 // Stages [s, s1) of the plan inside the tile (REV: radices in reverse order); words: the transform's slots.
 // SCAN_LAST: the last stage's outputs are scanned too.
-template <int P, int LS, bool INV, bool REV, int s, int s1, bool SCAN_LAST = false>
+template <int P, class RW, bool INV, bool REV, int s, int s1, bool SCAN_LAST = false>
 __device__ __forceinline__ void fx_mid_stages(const FxTile& t, unsigned* words) {
   if constexpr (s < s1) {
     constexpr FxPlan pl = fx_plan(P);
     constexpr int R = pl.r[REV ? pl.n - 1 - s : s], Ns = REV ? fx_prod(P, pl.n - s, pl.n) : fx_prod(P, 0, s);
-    fx_stage<P, R, Ns, INV, FX_TILE, true, s, SCAN_LAST>(t, nullptr, words, FxFromS<LS>{t.S}, FxToS<LS>{t.S});
-    fx_mid_stages<P, LS, INV, REV, s + 1, s1, SCAN_LAST>(t, words);
+    fx_stage<P, R, Ns, INV, FX_TILE, true, s, SCAN_LAST>(t, nullptr, words, FxFromS<RW>{t.S}, FxToS<RW>{t.S});
+    fx_mid_stages<P, RW, INV, REV, s + 1, s1, SCAN_LAST>(t, words);
   }
 }
 
@@ -264,7 +270,7 @@ __device__ __forceinline__ void fx_green_base(const PassParams& p, int q, int o,
 
 // Load of real data pairs whose extension is built in the tile (symmetric and semi-unbounded directions, and
 // every real pass on pinned host arrays): items (lane, i < n_data), at most U per thread.
-template <int P, int LS, int U>
+template <int P, class RW, int U>
 __device__ __forceinline__ void fx_load_ext(const PassParams& p, const FxTile& t, int type, const double* in, int q0,
                                             int* emax) {
   const int W = t.W, N = p.N, nd = p.n_data, tot = nd * W;
@@ -291,7 +297,7 @@ __device__ __forceinline__ void fx_load_ext(const PassParams& p, const FxTile& t
   const int nz = zero_ranges(bt, p.center, N, lo, hi);
   for (int z = 0; z < nz; ++z)
     for (int idx = t.tid; idx < (min(hi[z], P) - lo[z]) * W; idx += t.nt)
-      S[(lo[z] + (idx >> t.lw)) * LS + (idx & (W - 1))] = fx_make(0, 0);
+      S[RW::at(lo[z] + (idx >> t.lw)) + (idx & (W - 1))] = fx_make(0, 0);
   if (!p.fx_host) {
     unsigned m = 0;
 #pragma unroll
@@ -309,13 +315,13 @@ __device__ __forceinline__ void fx_load_ext(const PassParams& p, const FxTile& t
     const int dix = rev ? nd - 1 - i : i;
     int pos[4], sg[4];
     const int n = images(bt, p.center, N, dix, pos, sg);
-    for (int k = 0; k < n; ++k) S[pos[k] * LS + l] = sg[k] > 0 ? v : fx_make(-v.x, -v.y);
+    for (int k = 0; k < n; ++k) S[RW::at(pos[k]) + l] = sg[k] > 0 ? v : fx_make(-v.x, -v.y);
   }
   __syncthreads();
 }
 
 // Forward transform of real data into the tile: pairs (row q0 + 2l, row q0 + 2l + 1).
-template <int P, int LS, bool SCAN_LAST>
+template <int P, class RW, bool SCAN_LAST>
 __device__ __forceinline__ void fx_forward_real(const PassParams& p, const FxTile& t, int type, const double* in,
                                                 int q0, int* emax, unsigned* words) {
   constexpr FxPlan pl = fx_plan(P);
@@ -335,17 +341,17 @@ __device__ __forceinline__ void fx_forward_real(const PassParams& p, const FxTil
             v[k] = fx_make(k * nbf.value < la ? __double_as_longlong(r[0]) : 0,
                            k * nbf.value < lb ? __double_as_longlong(r[ls]) : 0);
         },
-        FxToS<LS>{t.S});
+        FxToS<RW>{t.S});
   } else {
-    if (p.n_data * t.W <= 9 * t.nt) fx_load_ext<P, LS, 9>(p, t, type, in, q0, emax);
-    else fx_load_ext<P, LS, 19>(p, t, type, in, q0, emax);
-    fx_stage<P, pl.r[0], 1, false, FX_TILE, true, 0>(t, nullptr, words, FxFromS<LS>{t.S}, FxToS<LS>{t.S});
+    if (p.n_data * t.W <= 9 * t.nt) fx_load_ext<P, RW, 9>(p, t, type, in, q0, emax);
+    else fx_load_ext<P, RW, 19>(p, t, type, in, q0, emax);
+    fx_stage<P, pl.r[0], 1, false, FX_TILE, true, 0>(t, nullptr, words, FxFromS<RW>{t.S}, FxToS<RW>{t.S});
   }
-  fx_mid_stages<P, LS, false, false, 1, pl.n, SCAN_LAST>(t, words);
+  fx_mid_stages<P, RW, false, false, 1, pl.n, SCAN_LAST>(t, words);
 }
 
 // Store of real data from the tile's last inverse stage; lane_q(l, &q, &kind): scale of lane l's values.
-template <int P, int LS, class Q>
+template <int P, class RW, class Q>
 __device__ __forceinline__ void fx_store_real(const PassParams& p, const FxTile& t, int type, double* out, int q0,
                                               unsigned* words, Q lane_q) {
   constexpr FxPlan pl = fx_plan(P);
@@ -360,7 +366,7 @@ __device__ __forceinline__ void fx_store_real(const PassParams& p, const FxTile&
   const int npen = p.npen;
   if (!p.fx_host) {
     fx_stage<P, R, Ns, true, FX_TILE, false, pl.n - 1>(
-        t, nullptr, words, FxFromS<LS>{t.S}, [&](auto R_, auto Ns_, int o, int l, const cfx* v) {
+        t, nullptr, words, FxFromS<RW>{t.S}, [&](auto R_, auto Ns_, int o, int l, const cfx* v) {
           const int qa = q0 + 2 * l;
           if (qa >= npen) return;
           int q, kind;
@@ -395,13 +401,13 @@ __device__ __forceinline__ void fx_store_real(const PassParams& p, const FxTile&
         });
     return;
   }
-  fx_stage<P, R, Ns, true, FX_TILE, true, pl.n - 1>(t, nullptr, words, FxFromS<LS>{t.S}, FxToS<LS>{t.S});
+  fx_stage<P, R, Ns, true, FX_TILE, true, pl.n - 1>(t, nullptr, words, FxFromS<RW>{t.S}, FxToS<RW>{t.S});
   for (int idx = t.tid; idx < nd * t.W; idx += t.nt) {
     const int l = idx / nd, i = idx % nd, qa = q0 + 2 * l;
     if (qa >= npen) continue;
     const int pos = dup && i == N ? 0 : (rev ? nd - 1 - i : i);
     const bool zero = (odd0 && pos == 0) || (oddN && pos == N);
-    const cfx v = t.S[pos * LS + l];
+    const cfx v = t.S[RW::at(pos) + l];
     int q, kind;
     lane_q(l, &q, &kind);
     double* d = out + (long long)qa * ls + (long long)i * js;
@@ -416,8 +422,8 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr bool REAL = KIND == K_FWD_REAL || KIND == K_INV_REAL || KIND == K_FUSED_REAL;
   constexpr bool FUSED = KIND == K_FUSED_REAL || KIND == K_FUSED_C2C;
-  constexpr int LS = fx_ls(KIND == K_FUSED_C2C, P);
-  const FxSmem m = fx_smem(smraw, P, p.W, LS);
+  using RW = FxRows<P, (KIND == K_FUSED_C2C)>;
+  const FxSmem m = fx_smem(smraw, p.W, RW::size);
   const int tid = threadIdx.x, nt = blockDim.x;
   FxTile t;
   t.S = m.S;
@@ -464,11 +470,11 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
   }
   // exponent of a fixed-point value of lane l after the forward (or a single inverse) transform
   constexpr int shift = kFxTwShift * (ns - 1) - kFxBias;
-  const FxFromS<LS> from_s{S};
-  const FxToS<LS> to_s{S};
+  const FxFromS<RW> from_s{S};
+  const FxToS<RW> to_s{S};
 
   if constexpr (KIND == K_FWD_REAL) {
-    fx_forward_real<P, LS, false>(p, t, type, (const double*)p.in + bi, q0, m.emax, wf);
+    fx_forward_real<P, RW, false>(p, t, type, (const double*)p.in + bi, q0, m.emax, wf);
     const int bt = base_type(type);
     const bool cplx = bt == T_PER || bt == T_UNB, quarter = is_quarter(bt), oddo = is_odd_origin(bt);
     const bool cell = p.center == C_CELL;
@@ -481,7 +487,7 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
       const bool two = qa + 1 < p.npen;
       for (int k = tid >> p.lw; k < nm; k += nt >> p.lw) {
         const int kk = quarter ? 2 * k + 1 : k, km = kk == 0 ? 0 : P - kk;
-        const cfx zk = S[kk * LS + l], zm = S[km * LS + l];
+        const cfx zk = S[RW::at(kk) + l], zm = S[RW::at(km) + l];
         cfx A = fx_make(zk.x + zm.x, zk.y - zm.y), B = fx_make(zk.y + zm.y, zm.x - zk.x);
         const long long off = bo + (long long)qa * p.ao.ls + (long long)k * p.ao.js;
         if (cplx) {
@@ -540,7 +546,7 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
     }
     lane_max(m.emax, mx, W, l, tid);
     if (quarter)  // even modes of the quarter-wave types are zero
-      for (int idx = tid; idx < half * W; idx += nt) S[2 * (idx >> p.lw) * LS + (idx & (W - 1))] = fx_make(0, 0);
+      for (int idx = tid; idx < half * W; idx += nt) S[RW::at(2 * (idx >> p.lw)) + (idx & (W - 1))] = fx_make(0, 0);
     __syncthreads();
     const int E = max(m.emax[l], kFxMinE);
     // the half-sample phase divides by 2^4: such coefficients keep 4 more bits
@@ -562,20 +568,20 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
           B = fx_cmul<true>(B, w);
         }
       }
-      S[kk * LS + l] = fx_make(A.x - B.y, A.y + B.x);
-      if (kk != 0 && 2 * kk != P) S[(P - kk) * LS + l] = fx_make(A.x + B.y, B.x - A.y);
+      S[RW::at(kk) + l] = fx_make(A.x - B.y, A.y + B.x);
+      if (kk != 0 && 2 * kk != P) S[RW::at(P - kk) + l] = fx_make(A.x + B.y, B.x - A.y);
     }
     __syncthreads();
     fx_stage<P, R0, 1, true, FX_TILE, true, 0>(t, nullptr, wi, from_s, to_s);
-    fx_mid_stages<P, LS, true, false, 1, ns - 1>(t, wi);
+    fx_mid_stages<P, RW, true, false, 1, ns - 1>(t, wi);
     const int add = shift + (quarter ? 1 : 0);
-    fx_store_real<P, LS>(p, t, type, (double*)p.out + bo, q0, wi, [&](int lane, int* q, int* kind) {
+    fx_store_real<P, RW>(p, t, type, (double*)p.out + bo, q0, wi, [&](int lane, int* q, int* kind) {
       const int Ee = max(m.emax[lane], kFxMinE);
       *q = Ee + add - fx_shifted<P>(m.words, W, lane, false, false, true);
       *kind = fx_out_kind(Ee, *q);
     });
   } else if constexpr (KIND == K_FUSED_REAL) {
-    fx_forward_real<P, LS, true>(p, t, type, (const double*)p.in + bi, q0, m.emax, wf);
+    fx_forward_real<P, RW, true>(p, t, type, (const double*)p.in + bi, q0, m.emax, wf);
     const bool quarter = is_quarter(base_type(type));
     unsigned mo = 0;
     {
@@ -587,7 +593,7 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
       const long long* G = (const long long*)p.g.stored;
       for (int k = tid >> p.lw; k <= half; k += nt >> p.lw) {
         const int km = k == 0 ? 0 : P - k;
-        cfx zk = S[k * LS + l], zm = S[km * LS + l];
+        cfx zk = S[RW::at(k) + l], zm = S[RW::at(km) + l];
         zk = fx_make(zk.x << upx, zk.y << upx);
         zm = fx_make(zm.x << upx, zm.y << upx);
         cfx A = fx_make(0, 0), B = A;
@@ -600,8 +606,8 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
         }
         const cfx zp = fx_make(A.x - B.y, A.y + B.x), zq = fx_make(A.x + B.y, B.x - A.y);
         mo |= fx_mag(zp.x) | fx_mag(zp.y) | fx_mag(zq.x) | fx_mag(zq.y);
-        S[k * LS + l] = zp;
-        if (k != 0 && 2 * k != P) S[km * LS + l] = zq;
+        S[RW::at(k) + l] = zp;
+        if (k != 0 && 2 * k != P) S[RW::at(km) + l] = zq;
       }
       lane_or(wg, mo, W, l, tid);
     }
@@ -615,8 +621,8 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
           for (int r = 0; r < R.value; ++r) v[r] = fx_make(v[r].x << up, v[r].y << up);
         },
         to_s);
-    fx_mid_stages<P, LS, true, false, 1, ns - 1>(t, wi);
-    fx_store_real<P, LS>(p, t, type, (double*)p.out + bo, q0, wi, [&](int lane, int* q, int* kind) {
+    fx_mid_stages<P, RW, true, false, 1, ns - 1>(t, wi);
+    fx_store_real<P, RW>(p, t, type, (double*)p.out + bo, q0, wi, [&](int lane, int* q, int* kind) {
       const int Ee = max(m.emax[lane], kFxMinE);
       *q = Ee - fx_shifted<P>(m.words, W, lane, true, true, true) + 2 * shift + kFxBias - 1 + 64 + max(m.gexp[2 * lane], m.gexp[2 * lane + 1]);
       *kind = fx_out_kind(Ee, *q);
@@ -662,7 +668,7 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
     };
     if constexpr (KIND == K_FUSED_C2C) {
       fx_stage<P, R0, 1, false, FX_RAW, true, 0>(t, emax, wf, load, to_s);
-      fx_mid_stages<P, LS, false, false, 1, ns, true>(t, wf);
+      fx_mid_stages<P, RW, false, false, 1, ns, true>(t, wf);
       // u^ = G^ f^ in the first inverse stage (radices reversed)
       if (tma_g) {
         if (!mbar_wait_bounded(m.mbar, p.errflag, 1, p.dbg_wait & 1)) store_ok = false;
@@ -688,7 +694,7 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
         }
       };
       fx_stage<P, RL, 1, true, FX_GAIN, true, 0>(t, wg, wi, gained, to_s);
-      fx_mid_stages<P, LS, true, true, 1, ns - 1>(t, wi);
+      fx_mid_stages<P, RW, true, true, 1, ns - 1>(t, wi);
       const int E = max(m.emax[l0], kFxMinE);
       q = E - fx_shifted<P>(m.words, W, l0, true, true, true) + 2 * shift + kFxBias + 64 + m.gexp[l0];
       kind = fx_out_kind(E, q);
@@ -696,7 +702,7 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
     } else {
       constexpr bool INV = KIND == K_INV_C2C;
       fx_stage<P, R0, 1, INV, FX_RAW, true, 0>(t, emax, wf, load, to_s);
-      fx_mid_stages<P, LS, INV, false, 1, ns - 1>(t, wf);
+      fx_mid_stages<P, RW, INV, false, 1, ns - 1>(t, wf);
       const int E = max(m.emax[l0], kFxMinE);
       q = E + shift - fx_shifted<P>(m.words, W, l0, true, false, false);
       kind = fx_out_kind(E, q);

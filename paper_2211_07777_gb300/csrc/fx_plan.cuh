@@ -4,7 +4,7 @@
 namespace flups {
 
 // Lengths and their radices, fewest stages first, then the cheapest split by operations per value and
-// threads left idle.
+// threads left idle; equal even radices first and last, whose stores have the widest strides (FxRows).
 #define FX_LENGTHS(X) \
   X(4, 2, 2, 2, 1, 1) \
   X(6, 2, 3, 2, 1, 1) \
@@ -23,7 +23,7 @@ namespace flups {
   X(72, 2, 12, 6, 1, 1) \
   X(81, 2, 9, 9, 1, 1) \
   X(96, 2, 12, 8, 1, 1) \
-  X(108, 3, 6, 6, 3, 1) \
+  X(108, 3, 6, 3, 6, 1) \
   X(128, 2, 16, 8, 1, 1) \
   X(144, 2, 12, 12, 1, 1) \
   X(162, 3, 9, 9, 2, 1) \
@@ -31,33 +31,33 @@ namespace flups {
   X(216, 3, 6, 6, 6, 1) \
   X(243, 4, 9, 3, 3, 3) \
   X(256, 2, 16, 16, 1, 1) \
-  X(288, 3, 12, 12, 2, 1) \
+  X(288, 3, 12, 2, 12, 1) \
   X(324, 3, 9, 9, 4, 1) \
   X(384, 3, 16, 8, 3, 1) \
-  X(432, 3, 12, 6, 6, 1) \
+  X(432, 3, 6, 12, 6, 1) \
   X(486, 4, 9, 9, 3, 2) \
   X(512, 3, 8, 8, 8, 1) \
-  X(576, 3, 12, 12, 4, 1) \
-  X(648, 4, 6, 6, 6, 3) \
+  X(576, 3, 12, 4, 12, 1) \
+  X(648, 4, 6, 6, 3, 6) \
   X(729, 3, 9, 9, 9, 1) \
-  X(768, 3, 16, 16, 3, 1) \
-  X(864, 3, 12, 12, 6, 1) \
+  X(768, 3, 16, 3, 16, 1) \
+  X(864, 3, 12, 6, 12, 1) \
   X(972, 4, 9, 9, 4, 3) \
-  X(1024, 3, 16, 8, 8, 1) \
-  X(1152, 3, 12, 12, 8, 1) \
+  X(1024, 3, 8, 16, 8, 1) \
+  X(1152, 3, 12, 8, 12, 1) \
   X(1296, 4, 6, 6, 6, 6) \
   X(1458, 4, 9, 9, 9, 2) \
-  X(1536, 4, 8, 8, 8, 3) \
+  X(1536, 4, 8, 8, 3, 8) \
   X(1728, 3, 12, 12, 12, 1) \
-  X(1944, 4, 9, 6, 6, 6) \
-  X(2048, 3, 16, 16, 8, 1) \
+  X(1944, 4, 6, 9, 6, 6) \
+  X(2048, 3, 16, 8, 16, 1) \
   X(2187, 4, 9, 9, 9, 3) \
-  X(2304, 3, 16, 12, 12, 1) \
-  X(2592, 4, 12, 6, 6, 6) \
+  X(2304, 3, 12, 16, 12, 1) \
+  X(2592, 4, 6, 12, 6, 6) \
   X(2916, 4, 9, 9, 9, 4) \
-  X(3072, 4, 16, 8, 8, 3) \
-  X(3456, 4, 12, 12, 12, 2) \
-  X(3888, 4, 12, 9, 6, 6) \
+  X(3072, 4, 8, 16, 3, 8) \
+  X(3456, 4, 12, 12, 2, 12) \
+  X(3888, 4, 6, 12, 9, 6) \
   X(4096, 3, 16, 16, 16, 1)
 
 
@@ -113,9 +113,21 @@ __host__ __device__ constexpr int fx_width(bool fused_c2c, int P) {
   const int wmin = P <= 1024 ? 4 : (P <= 2048 ? 2 : 1);
   return W < wmin ? wmin : W;
 }
-__host__ __device__ constexpr int fx_ls(bool fused_c2c, int P) {
-  const int W = fx_width(fused_c2c, P);
-  return W == 1 ? 1 : W + 1;
+// Rows of the tile in shared memory (16-byte values, W of them a row).  With 8 lanes a row is one 128-byte
+// wavefront of a quarter warp and no access conflicts; with fewer, a quarter warp touches 8 / W consecutive rows
+// (contiguous), except in the stores of a transform's first stage, whose rows are R apart: a gap of one row after
+// every B = R rows (R even) puts those on different banks.
+template <int P, bool FUSED_C2C> struct FxRows {
+  static constexpr int W = fx_width(FUSED_C2C, P);
+  static constexpr int B = W < 8 && fx_plan(P).r[0] % 2 == 0 ? fx_plan(P).r[0] : 0;
+  static constexpr int size = (P + (B ? (P - 1) / (B ? B : 1) : 0)) * W;
+  __host__ __device__ static constexpr int at(int i) { return (B ? i + i / (B ? B : 1) : i) * W; }
+  // at(j + r n) = at(j) + at(r n) for every j
+  __host__ __device__ static constexpr bool linear(int n) { return !B || n % (B ? B : 1) == 0; }
+};
+__host__ __device__ constexpr int fx_tile_values(bool fused_c2c, int P) {
+  const int W = fx_width(fused_c2c, P), r0 = fx_plan(P).r[0];
+  return (P + (W < 8 && r0 % 2 == 0 ? (P - 1) / r0 : 0)) * W;
 }
 __host__ __device__ constexpr int fx_prod(int P, int s0, int s1) {
   int n = 1;

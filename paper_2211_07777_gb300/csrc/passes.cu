@@ -41,6 +41,7 @@ cudaError_t set_pass_smem_limits() {
 }
 
 cudaError_t launch_pass(int kind, int prec, const PassParams& p, dim3 grid, int nthr, size_t smem, cudaStream_t st) {
+  if (p.f2) return launch_f2(kind, p, grid, nthr, smem, st);
   if (p.fx) return launch_fx(kind, p, grid, nthr, smem, st);
   if (p.ct && p.W == ct_small_width(p.P, prec)) return launch_ct_small(prec, p.P, kind, p, grid, nthr, smem, st);
   if (prec == 2) return p.ct ? launch_ct_df(p.P, kind, p, grid, nthr, smem, st)

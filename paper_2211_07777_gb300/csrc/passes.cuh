@@ -82,6 +82,8 @@ struct PassParams {
   int rows_off;
   int fx;                 // FP64-class pass in 64-bit fixed point (fx_passes.cu)
   int fx_host;            // such an x pass reads or writes pinned host memory: whole row pieces per warp
+  int f2;                 // FP32 pass on pairs of lanes in packed arithmetic (f2_passes.cu)
+  int f2_vec;             // its 16-byte accesses: bit 0 the input, bit 1 the output array
   int pdl;                // launched as a programmatic dependent of the stream's previous kernel: each CTA
                           // waits for the previous grid (complete, memory visible) before touching memory
   // column passes of the compile-time engine: the input tile by TMA (0 rows: loads from registers)
@@ -122,6 +124,9 @@ cudaError_t set_limits_ct_df_large();
 cudaError_t launch_fx(int kind, const PassParams& p, dim3 grid, int nthr, size_t smem, cudaStream_t st);
 // shared-memory limit of the kernel of that kind and length (per device, set when a plan is made)
 cudaError_t limit_fx(int kind, int P);
+// FP32 passes on pairs of lanes in packed arithmetic
+cudaError_t launch_f2(int kind, const PassParams& p, dim3 grid, int nthr, size_t smem, cudaStream_t st);
+cudaError_t limit_f2(int kind, int P);
 // narrow compile-time tiles for small grids: lanes per tile, 0 when not compiled
 int ct_small_width(int P, int prec);
 cudaError_t launch_ct_small(int prec, int P, int kind, const PassParams& p, dim3 grid, int nthr, size_t smem,

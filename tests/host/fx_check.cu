@@ -72,5 +72,11 @@ int main() {
 #define CHECK(P, N, r0, r1, r2, r3) \
   if (r0 * r1 * r2 * r3 != P || fx_prod(P, 0, fx_plan(P).n) != P || N < 2 || fx_ept(P) < 12 || fx_ept(P) > 18) return 2;
   FX_LENGTHS(CHECK)
+  // the tile's rows are distinct and inside the size that the planner allots
+#define ROWS(P, N, r0, r1, r2, r3)                                                                            \
+  if (FxRows<P, false>::size != fx_tile_values(false, P) || FxRows<P, true>::size != fx_tile_values(true, P)) return 3; \
+  for (int i = 0; i < P; ++i)                                                                                 \
+    if (FxRows<P, false>::at(i) + FxRows<P, false>::W > (i + 1 < P ? FxRows<P, false>::at(i + 1) : FxRows<P, false>::size)) return 4;
+  FX_LENGTHS(ROWS)
   return 0;
 }
