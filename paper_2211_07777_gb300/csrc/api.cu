@@ -106,6 +106,7 @@ struct DirPlan {
   RadixPlan rp{};
   void* tw = nullptr;
   void* tw2 = nullptr;  // of the FP32 lane-pair passes
+  void* twx = nullptr;  // of the fixed-point passes
 };
 
 struct Launch {
@@ -149,7 +150,8 @@ struct flups_solver_s {
   void* green_dev = nullptr;
   int* green_exp = nullptr;     // fixed-point spectrum: exponent of each pencil's slice
   int green_pitch = 0;          // x pitch (elements) of the stored spectrum
-  bool fx = false;              // passes in 64-bit fixed point (FP64-class Poisson solves)
+  bool fx = false;              // every pass in 64-bit fixed point (FP64-class Poisson solves)
+  bool fxp = false;             // the passes of the first two directions are (Biot-Savart solves too)
   bool share_green = false;     // look the stored spectrum up in (and add it to) the process-wide cache
   std::string green_key;        // its cache key when shared
   void* gmaps_dev = nullptr;    // TMA tensor maps of the stored spectrum (fused column pass)
@@ -454,11 +456,12 @@ void fill_geom(Launch& L, const DirPlan& dp, int axis, const int* din, const int
 
 // Tile of a fixed-point pass (after fill_geom): the full width of fx_width, narrower when the grid would leave SMs
 // idle (rows keep their stride).
-void fx_geom(Launch& L, int axis, bool packed) {
+void fx_geom(Launch& L, const DirPlan& dp, int axis, bool packed) {
   PassParams& p = L.p;
+  p.tw = dp.twx;
   const int P = p.P;
-  const bool fused_c2c = L.kind == K_FUSED_C2C;
-  int W = fx_width(fused_c2c, P);
+  const int cls = L.kind == K_FUSED_C2C ? FX_FUSED_C2C : FX_PLAIN;
+  int W = fx_width(cls, P);
   const int need = packed ? (p.npen + 1) / 2 : p.npen;
   while (W > 1 && W / 2 >= need) W /= 2;
   auto ctas = [&](int w) { return (long long)((need + w - 1) / w) * L.grid.y * L.grid.z; };
@@ -478,7 +481,7 @@ void fx_geom(Launch& L, int axis, bool packed) {
   L.grid.x = (unsigned)((need + W - 1) / W);
   L.nthr = nt;
   // alignment, mbarrier block, tile, Green offsets and exponents, lane exponents, renormalisation words
-  L.smem = 128 + 128 + (size_t)fx_tile_values(fused_c2c, P) * 16 + (size_t)W * (2 * 8 + 4 + 2 * 4 + kFxSlots * 4);
+  L.smem = 128 + 128 + (size_t)fx_tile_values(cls, P) * 16 + (size_t)W * (2 * 8 + 4 + 2 * 4 + kFxSlots * 4);
   p.rowx = (axis == 0 && p.center == C_CELL && (p.type == T_PER || p.type == T_UNB) &&
             (L.kind == K_FWD_REAL || L.kind == K_INV_REAL)) ? 1 : 0;
 }
@@ -486,15 +489,16 @@ void fx_geom(Launch& L, int axis, bool packed) {
 // Tile of an FP32 lane-pair pass (after fill_geom): as fx_geom, a lane holding two complex or four real pencils.
 void f2_geom(Launch& L, const DirPlan& dp, int axis, bool packed) {
   PassParams& p = L.p;
-  const int P = p.P, per = packed ? 4 : 2;
-  int W = fx_width(false, P);
+  const bool curl = L.kind >= K_CURL_REAL;
+  const int P = p.P, per = packed ? 4 : 2, cls = curl ? FX_CURL : FX_PLAIN;
+  int W = fx_width(cls, P);
   const int need = (p.npen + per - 1) / per;
   while (W > 1 && W / 2 >= need) W /= 2;
   auto ctas = [&](int w) { return (long long)((need + w - 1) / w) * L.grid.y * L.grid.z; };
   while (W > 1 && ctas(W) < 2 * 152 && W * P >= 512) W /= 2;
   const int ept = fx_ept(P);
   int nt = (P * W + ept - 1) / ept;
-  if (ctas(W) * nt < 152 * 256) nt = std::max(nt, std::min(256, P * W / 4));
+  if (ctas(W) * nt < 152 * 256) nt = std::max(nt, std::min(curl ? 128 : 256, P * W / 4));
   nt = std::max(32, (nt + 31) / 32 * 32);
   p.W = W;
   p.lw = ilog2(W);
@@ -506,8 +510,10 @@ void f2_geom(Launch& L, const DirPlan& dp, int axis, bool packed) {
   p.ept = 0;
   p.tw = dp.tw2;
   L.grid.x = (unsigned)((need + W - 1) / W);
-  L.nthr = nt;
-  L.smem = 128 + 128 + (size_t)fx_tile_values(false, P) * 16 + (size_t)W * (4 * 8 + 4 * 4);
+  L.nthr = curl ? 3 * nt : nt;
+  if (curl)  // three tiles, the lanes' derivative factors, Green offsets
+    L.smem = 3 * (size_t)fx_tile_values(cls, P) * 16 + (size_t)W * (per / 2 * 96 + per * (8 + 4));
+  else L.smem = 128 + 128 + (size_t)fx_tile_values(cls, P) * 16 + (size_t)W * (4 * 8 + 4 * 4);
 }
 
 // 16-byte accesses of a lane-pair pass: pencils adjacent in memory, rows and base 16-byte aligned.
@@ -520,7 +526,7 @@ void set_f2_vec(PassParams& p, int kind) {
     const long long v = cplx ? 2 : 4;
     return ((uintptr_t)ptr & 15) == 0 && a.ls == 1 && a.js % v == 0 && a.os % v == 0 && a.cs % v == 0;
   };
-  const bool c2c = kind == K_FWD_C2C || kind == K_INV_C2C || kind == K_FUSED_C2C;
+  const bool c2c = kind == K_FWD_C2C || kind == K_INV_C2C || kind == K_FUSED_C2C || kind == K_CURL_C2C;
   if (ok(p.in, p.ai, c2c || (kind == K_INV_REAL && modes))) p.f2_vec |= 1;
   if (ok(p.out, p.ao, c2c || (kind == K_FWD_REAL && modes))) p.f2_vec |= 2;
 }
@@ -650,12 +656,12 @@ int setup_green_compute(flups_solver_s* s, cudaStream_t st) {
     gp.nm = dp.gext;
     gp.rp = radix_plan(gp.P);
     // in 64-bit fixed point: GB300's FP64 units would make these passes the bulk of a plan's setup time
-    int rc = make_twiddles(gp.P, kFxTables, &gp.tw);
+    int rc = make_twiddles(gp.P, kFxTables, &gp.twx);
     if (rc) { cudaFreeAsync(g64, st); return rc; }
     Launch L{};
     L.kind = K_FWD_REAL;
     fill_geom(L, gp, d, q.gext, q.gext, FLUPS_F64, true, FLUPS_NODE, 1);
-    fx_geom(L, d, true);
+    fx_geom(L, gp, d, true);
     L.p.in = g64;
     L.p.out = g64;
     e = limit_fx(L.kind, gp.P);
@@ -998,21 +1004,24 @@ void set_rows_bulk(Launch& L, int prec) {
 // measurement on GB300 (us per pass, old / lane pairs):
 // - lengths with a factor 3, which had only the runtime-shaped tiles: always (192^3: 473 / 238 fused, 104 / 59
 //   complex, 150-200 / 60-75 symmetric; 48^3 fused 16 / 14);
+// - the Biot-Savart pass: always (128^3: 191 / 102 with an open axis, 59 / 50 periodic, 148 / 76 symmetric);
 // - powers of two: real passes along y or z (256-point periodic 78 / 64 and 76 / 53) and symmetric ones along
-//   x (512 points: 90 / 86 and 123 / 82); x passes of periodic and unbounded data up to 128 points (20 / 12,
-//   23 / 16; 256 points 51 / 58 and 47 / 88), the forward one also at 512 (76 / 74), while 1024 and 2048 points have
-//   their register-chained row kernels;
+//   x (512 points: 90 / 86 and 123 / 82); x passes of periodic and unbounded data where the grid is too small for the
+//   compile-time tiles (128^3 periodic 20 / 12 and 23 / 16; with those tiles 27 / 37 and 21 / 42 on three
+//   components), the forward one also at 512 points (366 / 342);
 // - complex passes of powers of two: never (256 points 14 / 16, fused 31 / 47; 1024 points fused 1912 / 3077): the
 //   column kernels prefetch their tiles by TMA and hold twice the warps.
 bool use_f2(const flups_solver_s* s, const Launch& L, const DirPlan& dp, int axis) {
   if (s->topo.prec != FLUPS_F32) return false;
   const int P = dp.P;
+  if (L.kind >= K_CURL_REAL)  // three times the threads of a tile, within the kernel's 512
+    return 3 * (((P * fx_width(FX_CURL, P) + fx_ept(P) - 1) / fx_ept(P) + 31) / 32 * 32) <= 512;
   if (P & (P - 1)) return true;
   if (L.kind == K_FUSED_REAL) return true;
   if (L.kind != K_FWD_REAL && L.kind != K_INV_REAL) return false;
   const bool modes = dp.type == T_PER || dp.type == T_UNB;
   if (axis != 0 || !modes) return true;
-  return P <= 128 || (P == 512 && L.kind == K_FWD_REAL);
+  return !L.p.ct || (P == 512 && L.kind == K_FWD_REAL);
 }
 
 int build_passes(flups_solver_s* s, cudaStream_t st) {
@@ -1037,7 +1046,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     L.kind = K_FWD_REAL;
     fill_geom(L, s->dir[o[0]], o[0], s->dims[0], s->dims[1], prec, true, center, nc, 1, s->pitch[0], s->pitch[1]);
     L.p.ctypes = pack3(s->tf[0][o[0]], s->tf[1][o[0]], s->tf[2][o[0]]);
-    if (s->fx) fx_geom(L, o[0], true);
+    if (s->fxp) fx_geom(L, s->dir[o[0]], o[0], true);
     else if (use_f2(s, L, s->dir[o[0]], o[0])) f2_geom(L, s->dir[o[0]], o[0], true);
     L.p.out = s->W1;
     L.out_buf = 1;
@@ -1055,7 +1064,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     L.kind = real ? K_FWD_REAL : K_FWD_C2C;
     fill_geom(L, s->dir[o[1]], o[1], s->dims[1], s->dims[2], prec, real, center, nc, 1, s->pitch[1], s->pitch[2]);
     L.p.ctypes = pack3(s->tf[0][o[1]], s->tf[1][o[1]], s->tf[2][o[1]]);
-    if (s->fx) fx_geom(L, o[1], real);
+    if (s->fxp) fx_geom(L, s->dir[o[1]], o[1], real);
     else if (use_f2(s, L, s->dir[o[1]], o[1])) f2_geom(L, s->dir[o[1]], o[1], real);
     L.p.in = s->W1;
     L.p.out = s->W2;
@@ -1076,15 +1085,16 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     fill_geom(L, dp, o[2], s->dims[2], s->dims[2], prec, real, center, curl ? 1 : nc, curl ? 3 : 1, s->pitch[2],
               s->pitch[2]);
     L.p.ctypes = pack3(s->tf[0][o[2]], s->tf[1][o[2]], s->tf[2][o[2]]);
-    if (s->fx) fx_geom(L, o[2], real);
-    else if (!curl && use_f2(s, L, dp, o[2])) f2_geom(L, dp, o[2], real);
+    if (s->fx) fx_geom(L, dp, o[2], real);
+    else if (use_f2(s, L, dp, o[2])) f2_geom(L, dp, o[2], real);
     L.p.in = s->W2;
     L.p.out = s->W2;
+    L.p.in_f64 = L.p.out_f64 = prec == FLUPS_F64E && s->fxp;  // between passes on FP64 arrays
     L.in_buf = 2;
     L.out_buf = 2;
     FusedGreen& g = L.p.g;
     if (curl) {
-      L.smem = 6 * (size_t)dp.P * L.p.LS * 2 * esize(prec) + (size_t)(real ? 2 : 1) * L.p.W * (prec == FLUPS_F32 ? 96 : 176) + 16;
+      if (!L.p.f2) L.smem = 6 * (size_t)dp.P * L.p.LS * 2 * esize(prec) + (size_t)(real ? 2 : 1) * L.p.W * (prec == FLUPS_F32 ? 96 : 176) + 16;
       g.utypes = pack3(s->tu[0][o[2]], s->tu[1][o[2]], s->tu[2][o[2]]);
       for (int d = 0; d < 3; ++d) {
         g.dsym[d] = s->dsym[d];
@@ -1118,7 +1128,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
           L.p.gmap = s->gmaps_dev;
       }
     }
-    if ((L.p.fx || L.p.f2) && !real && o[2] != 0 && g.stored && dp.gext == dp.P / 2 + 1 && g.fold[0] == 0) {
+    if ((L.p.fx || L.p.f2) && !curl && !real && o[2] != 0 && g.stored && dp.gext == dp.P / 2 + 1 && g.fold[0] == 0) {
       // fused column pass of the fixed-point or lane-pair kernels: the Green slice by TMA while the forward transform runs, where
       // two CTAs still fit an SM with it
       const int gw = L.p.f2 ? 2 * L.p.W : L.p.W;
@@ -1149,7 +1159,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     L.kind = real ? K_INV_REAL : K_INV_C2C;
     fill_geom(L, s->dir[o[1]], o[1], s->dims[2], s->dims[1], prec, real, center, nc, 1, s->pitch[2], s->pitch[1]);
     L.p.ctypes = pack3(s->tu[0][o[1]], s->tu[1][o[1]], s->tu[2][o[1]]);
-    if (s->fx) fx_geom(L, o[1], real);
+    if (s->fxp) fx_geom(L, s->dir[o[1]], o[1], real);
     else if (use_f2(s, L, s->dir[o[1]], o[1])) f2_geom(L, s->dir[o[1]], o[1], real);
     L.p.in = s->W2;
     L.p.out = s->W1;
@@ -1166,7 +1176,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     L.kind = K_INV_REAL;
     fill_geom(L, s->dir[o[0]], o[0], s->dims[1], s->dims[0], prec, true, center, nc, 1, s->pitch[1], s->pitch[0]);
     L.p.ctypes = pack3(s->tu[0][o[0]], s->tu[1][o[0]], s->tu[2][o[0]]);
-    if (s->fx) fx_geom(L, o[0], true);
+    if (s->fxp) fx_geom(L, s->dir[o[0]], o[0], true);
     else if (use_f2(s, L, s->dir[o[0]], o[0])) f2_geom(L, s->dir[o[0]], o[0], true);
     L.p.in = s->W1;
     L.in_buf = 1;
@@ -1326,8 +1336,8 @@ int flups_init_solver(flups_topo t, const int* bc, const double h[3], const doub
   // box a pass is one warp's chain of instructions, and the short FP64 columns of the warp engine are
   // faster (measured, us per solve, FP64 / fixed point: periodic 32^3 25.7 / 29.9, unbounded 16^3 25.1 / 29.0,
   // against periodic 36^3 39.8 / 28.6, unbounded 24^3 55.4 / 33.2, unbounded 64^3 230 / 76)
-  s->fx = t->prec != FLUPS_F32 && op == FLUPS_POISSON &&
-          (long long)s->dir[0].P * s->dir[1].P * s->dir[2].P > 65536;
+  s->fxp = t->prec != FLUPS_F32 && (long long)s->dir[0].P * s->dir[1].P * s->dir[2].P > 65536;
+  s->fx = s->fxp && op == FLUPS_POISSON;
   if (rc == FLUPS_OK) {
     int du = 0;
     for (int d = 0; d < 3; ++d) du += s->dir[d].unb;
@@ -1364,7 +1374,8 @@ int flups_setup(flups_solver s, void* stream, size_t* workspace_bytes) {
     }
   }
   for (int d = 0; d < 3; ++d) {
-    int rc = make_twiddles(s->dir[d].P, s->fx ? kFxTables : prec, &s->dir[d].tw);
+    int rc = s->fx ? FLUPS_OK : make_twiddles(s->dir[d].P, prec, &s->dir[d].tw);
+    if (!rc && s->fxp) rc = make_twiddles(s->dir[d].P, kFxTables, &s->dir[d].twx);
     if (!rc && prec == FLUPS_F32) rc = make_twiddles(s->dir[d].P, kF2Tables, &s->dir[d].tw2);
     if (rc) return rc;
     s->ws_bytes += (size_t)4 * s->dir[d].P * es;
@@ -1442,7 +1453,7 @@ static int solve_impl(flups_solver s, void* phi, const void* rhs, void* ws, void
       Lw.nthr = L.gnthr;
       if (!p.rows_bulk) Lw.smem = L.gsmem;
     }
-    cudaError_t e = L.kind >= K_CURL_REAL ? launch_curl(L.kind, prec, p, Lw.grid, Lw.nthr, Lw.smem, st)
+    cudaError_t e = L.kind >= K_CURL_REAL && !p.f2 ? launch_curl(L.kind, prec, p, Lw.grid, Lw.nthr, Lw.smem, st)
                                           : launch_pass(L.kind, prec, p, Lw.grid, Lw.nthr, Lw.smem, st);
     if (e) return cuda_fail(e, "pass launch");
     return FLUPS_OK;
@@ -1577,7 +1588,7 @@ int flups_solve_pass(flups_solver s, int i, void* phi, const void* rhs, void* st
   if (L.user_in) p.in = rhs;
   if (L.user_out) p.out = phi;
   set_f2_vec(p, L.kind);
-  cudaError_t e = L.kind >= K_CURL_REAL
+  cudaError_t e = L.kind >= K_CURL_REAL && !p.f2
                       ? launch_curl(L.kind, s->topo.prec, p, L.grid, L.nthr, L.smem, (cudaStream_t)stream)
                       : launch_pass(L.kind, s->topo.prec, p, L.grid, L.nthr, L.smem, (cudaStream_t)stream);
   if (e) return cuda_fail(e, "pass launch");

@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(512, 1) k_f2(const __grid_constant__ PassParam
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr bool REAL = KIND == K_FWD_REAL || KIND == K_INV_REAL || KIND == K_FUSED_REAL;
   constexpr bool FUSED = KIND == K_FUSED_REAL || KIND == K_FUSED_C2C;
-  using RW = FxRows<P, false>;
+  using RW = FxRows<P, FX_PLAIN>;
   constexpr FxPlan pl = fx_plan(P);
   constexpr int ns = pl.n, half = P / 2, R0 = pl.r[0], RL = pl.r[ns - 1];
   const int W = p.W;
@@ -569,6 +569,174 @@ __global__ void __launch_bounds__(512, 1) k_f2(const __grid_constant__ PassParam
   }
 }
 
+// ---------------------------------------------------------------------------
+// Fused last direction of the Biot-Savart solve: each third of the CTA transforms one component's tile in shared
+// memory, u^ = G^ (i w x f^) is taken point by point over the three (the derivative factors of curl.cu), and
+// each third transforms one result back.
+// ---------------------------------------------------------------------------
+struct F2Curl {       // per lane: the factors of the two non-axis directions, per source component
+  cf2 fac[2][3];
+};
+
+// Derivative factor along direction d of source component c at the pencil's mode: real for r2r coefficients
+// (sine-type sources +, cosine-type -), imaginary otherwise.
+__device__ __forceinline__ float2 f2_factor(const FusedGreen& g, int d, int c, int mode) {
+  const int kk = (g.role[d] == 0 && g.quarter[d]) ? 2 * mode + 1 : mode;
+  const float s = ((const float*)g.dsym[d])[kk];
+  if (g.role[d] == 0) return make_float2(((g.srcodd[d] >> c) & 1) ? s : -s, 0.f);
+  return make_float2(0.f, s);
+}
+// product of complex pairs
+__device__ __forceinline__ cf2 f2_mulc(cf2 a, cf2 b) {
+  return f2_make(f2_sub(f2_mul(a.x, b.x), f2_mul(a.y, b.y)), f2_fma(a.x, b.y, f2_mul(a.y, b.x)));
+}
+// u_c = G (D_a f_b - D_b f_a), (a, b) = (c + 1, c + 2); s3: symbol along the axis
+__device__ __forceinline__ void f2_curl(int axis, const F2Curl& f, f2 s3, f2 G, const cf2* F, cf2* U) {
+  const int d0 = axis == 0 ? 1 : 0;  // directions of fac[0], fac[1]
+  auto term = [&](int d, int c) {    // D_d f_c
+    if (d == axis) return f2_make(f2_neg(f2_mul(F[c].y, s3)), f2_mul(F[c].x, s3));
+    return f2_mulc(f.fac[d == d0 ? 0 : 1][c], F[c]);
+  };
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int a = (c + 1) % 3, b = (c + 2) % 3;
+    U[c] = f2_scale(term(a, b) - term(b, a), G);
+  }
+}
+
+template <bool REAL, int P>
+__global__ void __launch_bounds__(512, 1) k_f2_curl(const __grid_constant__ PassParams p) {
+  pass_entry(p);
+  extern __shared__ __align__(16) unsigned char smraw[];
+  using RW = FxRows<P, FX_CURL>;
+  constexpr FxPlan pl = fx_plan(P);
+  constexpr int ns = pl.n, half = P / 2, R0 = pl.r[0], RL = pl.r[ns - 1];
+  constexpr int per = REAL ? 4 : 2, NP = REAL ? 2 : 1;  // pencils and pencil pairs of a lane
+  const int W = p.W, tid = threadIdx.x, nt = blockDim.x, axis = p.axis;
+  cf2* S0 = reinterpret_cast<cf2*>(smraw);
+  F2Curl* fac = reinterpret_cast<F2Curl*>(S0 + 3 * RW::size);       // NP per lane
+  long long* goff = reinterpret_cast<long long*>(fac + NP * W);      // per lane: per
+  float* k2p = reinterpret_cast<float*>(goff + per * W);
+  const int q0 = blockIdx.x * per * W, o = blockIdx.y, npen = p.npen;
+  const long long bi = (long long)o * p.ai.os, bo = (long long)o * p.ao.os;
+  const FusedGreen& g = p.g;
+  for (int i = tid; i < per * W; i += nt) {
+    const int q = q0 + i;
+    f2_green_base(p, q, o, &goff[i], &k2p[i]);
+    // pencil i of the block: lane i / per; real lanes pair (q, q + 1) and (q + 2, q + 3)
+    float* dst = reinterpret_cast<float*>(&fac[(i / per) * NP + (i % per) / 2]);
+    int crd[3];
+    if (axis == 0) { crd[1] = q % g.dims1; crd[2] = q / g.dims1; crd[0] = 0; }
+    else if (axis == 1) { crd[0] = q; crd[2] = o; crd[1] = 0; }
+    else { crd[0] = q; crd[1] = o; crd[2] = 0; }
+    int e = 0;
+    for (int d = 0; d < 3; ++d) {
+      if (d == axis) continue;
+      for (int c = 0; c < 3; ++c) {
+        const float2 v = q < npen ? f2_factor(g, d, c, crd[d]) : make_float2(0.f, 0.f);
+        dst[(e * 3 + c) * 4 + (i & 1)] = v.x;
+        dst[(e * 3 + c) * 4 + 2 + (i & 1)] = v.y;
+      }
+      ++e;
+    }
+  }
+  __syncthreads();
+  const long long st3 = axis == 0 ? 1 : (axis == 1 ? (long long)g.gpitch : (long long)g.gpitch * g.gext[1]);
+  const float* sym3 = (const float*)g.dsym[axis];
+  const int l = tid & (W - 1);  // of the thread's transforms too: a third is a multiple of W threads
+  const int ql = q0 + per * l;
+  const long long ils = p.ai.ls, ijs = p.ai.js, ols = p.ao.ls, ojs = p.ao.js;
+  const int ntc = nt / 3, mine = tid / ntc;  // threads and number of this thread's component
+  const F2Tile t{S0 + mine * RW::size, W, p.lw, tid - mine * ntc, ntc, (const f2w*)p.tw};
+  {
+    if constexpr (REAL) {
+      f2_forward_real<P, RW>(p, t, comp_type(p, mine), (const float*)p.in + bi + mine * p.ai.cs, q0);
+    } else {
+      const float2* in = (const float2*)p.in + bi + mine * p.ai.cs + (long long)ql * ils;
+      const int n_in = p.n_use;
+      const bool vin = p.f2_vec & 1;
+      f2_stage<P, R0, 1, false, false, true>(
+          t,
+          [=](auto R, auto nbf, int j, int, cf2* v) {
+            const float2* s = in + (long long)j * ijs;
+            const long long step = (long long)nbf.value * ijs;
+            const int lim = ql < npen ? n_in - j : 0;
+#pragma unroll
+            for (int r = 0; r < R.value; ++r, s += step) {
+              v[r] = f2_make(0, 0);
+              if (r * nbf.value < lim) v[r] = f2_load2(s, ils, ql, npen, vin);
+            }
+          },
+          F2ToS<RW>{t.S});
+      f2_mid_stages<P, RW, false, false, 1, ns>(t);
+    }
+  }
+  if constexpr (REAL) {
+    const bool quarter = is_quarter(base_type(comp_type(p, 0)));
+    const f2 h = f2_dup(0.5f);
+#pragma unroll 1
+    for (int k = tid >> p.lw; k <= half; k += nt >> p.lw) {
+      const int km = k == 0 ? 0 : P - k;
+      const bool live = !quarter || (k & 1);
+      const int g3 = quarter ? max(k - 1, 0) >> 1 : k;
+      const f2 s3 = f2_dup(sym3[k]);
+      cf2 A[3], B[3], UA[3], UB[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const cf2* S = S0 + c * RW::size;
+        f2_split(S[RW::at(k) + l], S[RW::at(km) + l], A[c], B[c]);
+        UA[c] = UB[c] = f2_make(0, 0);
+      }
+      if (live) {
+        f2_curl(axis, fac[2 * l], s3, f2_mul(h, f2_green2(g, axis, &goff[4 * l], &k2p[4 * l], g3, st3)), A, UA);
+        f2_curl(axis, fac[2 * l + 1], s3, f2_mul(h, f2_green2(g, axis, &goff[4 * l + 2], &k2p[4 * l + 2], g3, st3)), B, UB);
+      }
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        cf2* S = S0 + c * RW::size;
+        S[RW::at(k) + l] = f2_make(f2_sub(UA[c].x, UB[c].y), f2_add(UA[c].y, UB[c].x));
+        if (k != 0 && 2 * k != P) S[RW::at(km) + l] = f2_make(f2_add(UA[c].x, UB[c].y), f2_sub(UB[c].x, UA[c].y));
+      }
+    }
+  } else {
+#pragma unroll 1
+    for (int k = tid >> p.lw; k < P; k += nt >> p.lw) {
+      cf2 F[3], U[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) F[c] = S0[c * RW::size + RW::at(k) + l];
+      f2_curl(axis, fac[l], f2_dup(sym3[k]), f2_green2(g, axis, &goff[2 * l], &k2p[2 * l], min(k, P - k), st3), F, U);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) S0[c * RW::size + RW::at(k) + l] = U[c];
+    }
+  }
+  __syncthreads();
+  {
+    const F2FromS<RW> from_s{t.S};
+    if constexpr (REAL) {
+      f2_stage<P, R0, 1, true, true, true>(t, from_s, F2ToS<RW>{t.S});
+      f2_mid_stages<P, RW, true, false, 1, ns - 1>(t);
+      f2_store_real<P, RW>(p, t, (g.utypes >> (4 * mine)) & 15, (float*)p.out + bo + mine * p.ao.cs, q0);
+    } else {
+      f2_stage<P, RL, 1, true, true, true>(t, from_s, F2ToS<RW>{t.S});
+      f2_mid_stages<P, RW, true, true, 1, ns - 1>(t);
+      float2* out = (float2*)p.out + bo + mine * p.ao.cs + (long long)ql * ols;
+      const int dup = (p.type == T_PER && p.center == C_NODE && p.n_data > p.N) ? p.N : -1;
+      const int n_out = p.n_data;
+      const bool vout = p.f2_vec & 2;
+      f2_stage<P, R0, P / R0, true, true, false>(t, from_s, [=](auto R, auto Ns, int o_, int, const cf2* v) {
+        if (ql >= npen) return;
+        float2* d = out + (long long)o_ * ojs;
+        const long long step = (long long)Ns.value * ojs;
+        const int lim = n_out - o_;
+        if (dup >= 0 && o_ == 0) f2_store2(d + (long long)dup * ojs, ols, ql, npen, vout, v[0]);
+#pragma unroll
+        for (int r = 0; r < R.value; ++r, d += step)
+          if (r * Ns.value < lim) f2_store2(d, ols, ql, npen, vout, v[r]);
+      });
+    }
+  }
+}
+
 }  // namespace
 
 template <int KIND, int P>
@@ -583,10 +751,14 @@ cudaError_t f2_launch(const PassParams& p, dim3 grid, int nthr, size_t smem, cud
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = p.pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k_f2<KIND, P>, p);
+  if constexpr (KIND >= K_CURL_REAL) return cudaLaunchKernelEx(&cfg, k_f2_curl<KIND == K_CURL_REAL, P>, p);
+  else return cudaLaunchKernelEx(&cfg, k_f2<KIND, P>, p);
 }
 template <int KIND, int P> cudaError_t f2_limit() {
-  return cudaFuncSetAttribute(k_f2<KIND, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  const int lim = 227 * 1024;
+  if constexpr (KIND >= K_CURL_REAL)
+    return cudaFuncSetAttribute(k_f2_curl<KIND == K_CURL_REAL, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  else return cudaFuncSetAttribute(k_f2<KIND, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
 }
 #define F2_KINDS(DO)                   \
   switch (kind) {                      \
@@ -596,6 +768,8 @@ template <int KIND, int P> cudaError_t f2_limit() {
     case K_INV_C2C: DO(K_INV_C2C);     \
     case K_FUSED_REAL: DO(K_FUSED_REAL); \
     case K_FUSED_C2C: DO(K_FUSED_C2C); \
+    case K_CURL_REAL: DO(K_CURL_REAL); \
+    case K_CURL_C2C: DO(K_CURL_C2C);   \
     default: return cudaErrorInvalidValue; \
   }
 template <int P>

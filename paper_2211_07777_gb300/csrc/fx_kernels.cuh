@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr bool REAL = KIND == K_FWD_REAL || KIND == K_INV_REAL || KIND == K_FUSED_REAL;
   constexpr bool FUSED = KIND == K_FUSED_REAL || KIND == K_FUSED_C2C;
-  using RW = FxRows<P, (KIND == K_FUSED_C2C)>;
+  using RW = FxRows<P, (KIND == K_FUSED_C2C ? FX_FUSED_C2C : FX_PLAIN)>;
   const FxSmem m = fx_smem(smraw, p.W, RW::size);
   const int tid = threadIdx.x, nt = blockDim.x;
   FxTile t;

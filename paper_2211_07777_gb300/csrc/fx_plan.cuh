@@ -107,9 +107,12 @@ __host__ __device__ constexpr int fx_ept(int P) {
 // warps of one CTA run the same stretch of it and share its instruction fetches (unbounded 128^3 197 -> 186 us,
 // 192^3 895 -> 840; the other passes 0-8% slower with 4096, all 10-30% slower with 8192).  At least 4 lanes
 // (64 contiguous bytes along x) up to P = 1024.
-__host__ __device__ constexpr int fx_width(bool fused_c2c, int P) {
+// FX_CURL: the Biot-Savart pass, which holds three components, about 1024 values each.
+enum FxTileClass : int { FX_PLAIN = 0, FX_FUSED_C2C = 1, FX_CURL = 2 };
+__host__ __device__ constexpr int fx_width(int cls, int P) {
   int W = 1;
-  while (W < 32 && 2 * W * P <= (fused_c2c ? 4096 : 2048)) W *= 2;
+  while (W < 32 && 2 * W * P <= (cls == FX_FUSED_C2C ? 4096 : (cls == FX_CURL ? 1024 : 2048))) W *= 2;
+  if (cls == FX_CURL) return W;
   const int wmin = P <= 1024 ? 4 : (P <= 2048 ? 2 : 1);
   return W < wmin ? wmin : W;
 }
@@ -117,16 +120,16 @@ __host__ __device__ constexpr int fx_width(bool fused_c2c, int P) {
 // wavefront of a quarter warp and no access conflicts; with fewer, a quarter warp touches 8 / W consecutive rows
 // (contiguous), except in the stores of a transform's first stage, whose rows are R apart: a gap of one row after
 // every B = R rows (R even) puts those on different banks.
-template <int P, bool FUSED_C2C> struct FxRows {
-  static constexpr int W = fx_width(FUSED_C2C, P);
+template <int P, int CLS> struct FxRows {
+  static constexpr int W = fx_width(CLS, P);
   static constexpr int B = W < 8 && fx_plan(P).r[0] % 2 == 0 ? fx_plan(P).r[0] : 0;
   static constexpr int size = (P + (B ? (P - 1) / (B ? B : 1) : 0)) * W;
   __host__ __device__ static constexpr int at(int i) { return (B ? i + i / (B ? B : 1) : i) * W; }
   // at(j + r n) = at(j) + at(r n) for every j
   __host__ __device__ static constexpr bool linear(int n) { return !B || n % (B ? B : 1) == 0; }
 };
-__host__ __device__ constexpr int fx_tile_values(bool fused_c2c, int P) {
-  const int W = fx_width(fused_c2c, P), r0 = fx_plan(P).r[0];
+__host__ __device__ constexpr int fx_tile_values(int cls, int P) {
+  const int W = fx_width(cls, P), r0 = fx_plan(P).r[0];
   return (P + (W < 8 && r0 % 2 == 0 ? (P - 1) / r0 : 0)) * W;
 }
 __host__ __device__ constexpr int fx_prod(int P, int s0, int s1) {

@@ -20,6 +20,19 @@ template <> __device__ __forceinline__ void st_real<dfloat>(dfloat* a, long long
   else reinterpret_cast<float2*>(a)[off] = make_float2(v.hi, v.lo);
 }
 
+// The same for complex values (a double-float pass between fixed-point ones reads and writes FP64 arrays).
+template <typename T> __device__ __forceinline__ cpx<T> ld_cplx(const cpx<T>* a, long long off, int f64) { return a[off]; }
+template <> __device__ __forceinline__ cdfloat ld_cplx<dfloat>(const cdfloat* a, long long off, int f64) {
+  if (!f64) return a[off];
+  const double2 q = reinterpret_cast<const double2*>(a)[off];
+  return mk<dfloat>(df_from_double(q.x), df_from_double(q.y));
+}
+template <typename T> __device__ __forceinline__ void st_cplx(cpx<T>* a, long long off, cpx<T> v, int f64) { a[off] = v; }
+template <> __device__ __forceinline__ void st_cplx<dfloat>(cdfloat* a, long long off, cdfloat v, int f64) {
+  if (f64) reinterpret_cast<double2*>(a)[off] = make_double2(df_to_double(v.x), df_to_double(v.y));
+  else a[off] = v;
+}
+
 // Index of element (row i, lane l) of a tile: the compile-time engine's layout (WC > 0) or rows of
 // LS elements (runtime engine).
 // log2 of a power of two, at compile time
@@ -306,7 +319,8 @@ __device__ __forceinline__ void load_cplx(const PassParams& p, const cpx<T>* __r
       ll[u] = lane;
       ii[u] = i;
       const int q = q0 + lane;
-      v[u] = (i >= 0 && q < p.npen) ? in[(long long)q * p.ai.ls + (long long)i * p.ai.js] : mk<T>((T)0, (T)0);
+      v[u] = (i >= 0 && q < p.npen) ? ld_cplx<T>(in, (long long)q * p.ai.ls + (long long)i * p.ai.js, p.in_f64)
+                                    : mk<T>((T)0, (T)0);
     }
 #pragma unroll
     for (int u = 0; u < LOADB; ++u)
@@ -327,7 +341,7 @@ __device__ __forceinline__ void store_cplx_data(const PassParams& p, cpx<T>* __r
     const int q = q0 + lane;
     if (q >= p.npen) continue;
     const int pos = (p.type == T_PER && p.center == C_NODE && i == p.N) ? 0 : i;
-    out[(long long)q * p.ao.ls + (long long)i * p.ao.js] = S[tix<T, WC>(pos, lane, LS)];
+    st_cplx<T>(out, (long long)q * p.ao.ls + (long long)i * p.ao.js, S[tix<T, WC>(pos, lane, LS)], p.out_f64);
   }
 }
 

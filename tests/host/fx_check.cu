@@ -74,9 +74,9 @@ int main() {
   FX_LENGTHS(CHECK)
   // the tile's rows are distinct and inside the size that the planner allots
 #define ROWS(P, N, r0, r1, r2, r3)                                                                            \
-  if (FxRows<P, false>::size != fx_tile_values(false, P) || FxRows<P, true>::size != fx_tile_values(true, P)) return 3; \
+  if (FxRows<P, FX_PLAIN>::size != fx_tile_values(FX_PLAIN, P) || FxRows<P, FX_CURL>::size != fx_tile_values(FX_CURL, P)) return 3; \
   for (int i = 0; i < P; ++i)                                                                                 \
-    if (FxRows<P, false>::at(i) + FxRows<P, false>::W > (i + 1 < P ? FxRows<P, false>::at(i + 1) : FxRows<P, false>::size)) return 4;
+    if (FxRows<P, FX_PLAIN>::at(i) + FxRows<P, FX_PLAIN>::W > (i + 1 < P ? FxRows<P, FX_PLAIN>::at(i + 1) : FxRows<P, FX_PLAIN>::size)) return 4;
   FX_LENGTHS(ROWS)
   return 0;
 }
