@@ -958,7 +958,7 @@ void set_rowx(Launch& L, int prec) {
   PassParams& p = L.p;
   if (p.fx || p.f2) return;
   p.rowx = 0;
-  if (!p.ct || p.axis != 0 || (prec != FLUPS_F32 && prec != FLUPS_F64E) || p.W != 4 || p.center != C_CELL) return;
+  if (!p.ct || p.axis != 0 || prec != FLUPS_F32 || p.W != 4 || p.center != C_CELL) return;
   if (L.kind != K_FWD_REAL && L.kind != K_INV_REAL) return;
   for (int c = 0; c < (int)L.grid.z; ++c) {
     const int t = (p.ctypes >> (4 * c)) & 15;
@@ -970,7 +970,7 @@ void set_rowx(Launch& L, int prec) {
   // measured at 512^3 (P = 1024): the forward pass runs best with 16 elements per thread (256
   // threads; 0.488 vs 0.516 ms with radix-32 stages), the inverse with radix-32 stages and its
   // rows staged by a bulk copy (0.453 ms; 0.492 with 16 elements per thread)
-  p.ept = (L.kind == K_FWD_REAL || prec != FLUPS_F32) ? 16 : ct_col_ept(p.P, prec, K_FWD_C2C);
+  p.ept = L.kind == K_FWD_REAL ? 16 : ct_col_ept(p.P, prec, K_FWD_C2C);
   L.nthr = p.P * p.W / p.ept;
   L.smem = (size_t)p.P * (p.W + 1) * 2 * esize(prec) + 256;
 }
@@ -1492,6 +1492,7 @@ int flups_solver_memory(flups_solver s, size_t* resident, size_t* transient, siz
   if (du > 0 || s->fx) {
     res += gn * es;
     tr += gn * sizeof(double) + (size_t)8 * 2 * gmax * sizeof(double);
+    if (du == 2) tr += gn * sizeof(double) / 3;  // the sampling's Chebyshev series, at most
   }
   for (int i = 1; i <= 2; ++i) ws += ws_array_bytes(s, i);
   ws += kStatusBlock;

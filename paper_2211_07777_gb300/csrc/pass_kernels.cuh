@@ -1093,7 +1093,7 @@ cudaError_t pass_launch(K kernel, const PassParams& p, dim3 grid, int nthr, size
 
 template <typename T, int PC, int WC, bool HZ>
 cudaError_t launch_kind_hz(int kind, const PassParams& p, dim3 grid, int nthr, size_t smem, cudaStream_t st) {
-  if constexpr (PC > 0 && (std::is_same<T, float>::value || std::is_same<T, dfloat>::value)) {
+  if constexpr (PC > 0 && std::is_same<T, float>::value) {
     if (p.axis == 0 && p.rowx && (kind == K_FWD_REAL || kind == K_INV_REAL)) {
       const bool fwd = kind == K_FWD_REAL;
       if constexpr (has_ept32<T, PC>()) {
@@ -1162,7 +1162,7 @@ cudaError_t set_limits_hz() {
     if ((e = cudaFuncSetAttribute(k_fwd_c2c_col<T, PC, WC, HZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
     if ((e = cudaFuncSetAttribute(k_inv_c2c_col<T, PC, WC, HZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
     if ((e = cudaFuncSetAttribute(k_fused_c2c_col<T, PC, WC, HZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
-    if constexpr (std::is_same<T, float>::value || std::is_same<T, dfloat>::value) {
+    if constexpr (std::is_same<T, float>::value) {
       if ((e = cudaFuncSetAttribute(k_fwd_rowx<T, PC, WC, HZ, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
       if ((e = cudaFuncSetAttribute(k_inv_rowx<T, PC, WC, HZ, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
       if constexpr (has_ept32<T, PC>()) {

@@ -6,6 +6,9 @@
 namespace flups {
 
 int ct_tile_width(int P, int prec, int axis, int kind) {
+  // double-float: only problems below the fixed-point passes' size and the Biot-Savart pass are left, on the
+  // runtime-shaped tiles
+  if (prec == 2) return 0;
   // FP32 at P = 1024 (measured at 512^3): 4 lanes for the x passes (row mode) and for the
   // single-transform column passes (radix-32, 128 threads: more CTAs per SM to overlap their
   // memory phases); 8 lanes for the fused column pass and the other passes
@@ -35,7 +38,6 @@ cudaError_t set_pass_smem_limits() {
   if (!e) e = set_limits_kind<dfloat, 0, 0>();
   if (!e) e = set_limits_ct_f32();
   if (!e) e = set_limits_ct_f64();
-  if (!e) e = set_limits_ct_df();
   if (!e) e = set_limits_ct_small();
   return e;
 }
@@ -44,8 +46,7 @@ cudaError_t launch_pass(int kind, int prec, const PassParams& p, dim3 grid, int 
   if (p.f2) return launch_f2(kind, p, grid, nthr, smem, st);
   if (p.fx) return launch_fx(kind, p, grid, nthr, smem, st);
   if (p.ct && p.W == ct_small_width(p.P, prec)) return launch_ct_small(prec, p.P, kind, p, grid, nthr, smem, st);
-  if (prec == 2) return p.ct ? launch_ct_df(p.P, kind, p, grid, nthr, smem, st)
-                             : launch_kind<dfloat, 0, 0>(kind, p, grid, nthr, smem, st);
+  if (prec == 2) return launch_kind<dfloat, 0, 0>(kind, p, grid, nthr, smem, st);
   if (p.ct) return prec == 0 ? launch_ct_f32(p.P, kind, p, grid, nthr, smem, st)
                              : launch_ct_f64(p.P, kind, p, grid, nthr, smem, st);
   return prec == 0 ? launch_kind<float, 0, 0>(kind, p, grid, nthr, smem, st)

@@ -115,11 +115,6 @@ cudaError_t launch_ct_f32(int P, int kind, const PassParams& p, dim3 grid, int n
 cudaError_t launch_ct_f64(int P, int kind, const PassParams& p, dim3 grid, int nthr, size_t smem, cudaStream_t st);
 cudaError_t set_limits_ct_f32();
 cudaError_t set_limits_ct_f64();
-cudaError_t launch_ct_df(int P, int kind, const PassParams& p, dim3 grid, int nthr, size_t smem, cudaStream_t st);
-cudaError_t set_limits_ct_df();
-cudaError_t launch_ct_df_large(int P, int kind, const PassParams& p, dim3 grid, int nthr, size_t smem,
-                               cudaStream_t st);
-cudaError_t set_limits_ct_df_large();
 // FP64-class Poisson passes in 64-bit block fixed point
 cudaError_t launch_fx(int kind, const PassParams& p, dim3 grid, int nthr, size_t smem, cudaStream_t st);
 // shared-memory limit of the kernel of that kind and length (per device, set when a plan is made)
