@@ -496,7 +496,7 @@ void f2_geom(Launch& L, const DirPlan& dp, int axis, bool packed) {
   while (W > 1 && W / 2 >= need) W /= 2;
   auto ctas = [&](int w) { return (long long)((need + w - 1) / w) * L.grid.y * L.grid.z; };
   while (W > 1 && ctas(W) < 2 * 152 && W * P >= 512) W /= 2;
-  const int ept = fx_ept(P);
+  const int ept = f2_ept(cls, P);
   int nt = (P * W + ept - 1) / ept;
   if (ctas(W) * nt < 152 * 256) nt = std::max(nt, std::min(curl ? 128 : 256, P * W / 4));
   nt = std::max(32, (nt + 31) / 32 * 32);
@@ -512,8 +512,8 @@ void f2_geom(Launch& L, const DirPlan& dp, int axis, bool packed) {
   L.grid.x = (unsigned)((need + W - 1) / W);
   L.nthr = curl ? 3 * nt : nt;
   if (curl)  // three tiles, the lanes' derivative factors, Green offsets
-    L.smem = 3 * (size_t)fx_tile_values(cls, P) * 16 + (size_t)W * (per / 2 * 96 + per * (8 + 4));
-  else L.smem = 128 + 128 + (size_t)fx_tile_values(cls, P) * 16 + (size_t)W * (4 * 8 + 4 * 4);
+    L.smem = 3 * (size_t)f2_tile_values(cls, P) * 16 + (size_t)W * (per / 2 * 96 + per * (8 + 4));
+  else L.smem = 128 + 128 + (size_t)f2_tile_values(cls, P) * 16 + (size_t)W * (4 * 8 + 4 * 4);
 }
 
 // 16-byte accesses of a lane-pair pass: pencils adjacent in memory, rows and base 16-byte aligned.
@@ -1015,7 +1015,7 @@ bool use_f2(const flups_solver_s* s, const Launch& L, const DirPlan& dp, int axi
   if (s->topo.prec != FLUPS_F32) return false;
   const int P = dp.P;
   if (L.kind >= K_CURL_REAL)  // three times the threads of a tile, within the kernel's 512
-    return 3 * (((P * fx_width(FX_CURL, P) + fx_ept(P) - 1) / fx_ept(P) + 31) / 32 * 32) <= 512;
+    return 3 * (((P * fx_width(FX_CURL, P) + f2_ept(FX_CURL, P) - 1) / f2_ept(FX_CURL, P) + 31) / 32 * 32) <= 512;
   if (P & (P - 1)) return true;
   if (L.kind == K_FUSED_REAL) return true;
   if (L.kind != K_FWD_REAL && L.kind != K_INV_REAL) return false;

@@ -3,7 +3,7 @@
 //
 // A CTA holds W lanes x P values of 16 bytes in shared memory, a value being one position of two complex
 // sequences: two neighbouring pencils of a complex pass, or four real pencils q .. q + 3 packed as
-// q + i (q + 2) and (q + 1) + i (q + 3).  The tile is transformed in place, whole butterflies of up to 18 values in
+// q + i (q + 2) and (q + 1) + i (q + 3).  The tile is transformed in place, whole butterflies of up to 9 values in
 // registers between two barriers; complex passes and the real passes of periodic and unbounded directions
 // read the first stage's inputs from memory and store the last stage's outputs from registers.
 #pragma once
@@ -17,6 +17,13 @@
 namespace flups {
 
 namespace {
+
+// Threads a kernel is compiled for: the block of a full tile, rounded up (small grids take at most 256)
+template <int P> struct F2Block {
+  static constexpr int n = (P * fx_width(FX_PLAIN, P) + f2_ept(FX_PLAIN, P) - 1) / f2_ept(FX_PLAIN, P);
+  static constexpr int threads = n <= 256 ? 256 : (n <= 512 ? 512 : 768);
+  static_assert(n <= 768, "threads of a tile");
+};
 
 template <int N> using ic2 = std::integral_constant<int, N>;
 
@@ -79,9 +86,9 @@ template <class RW> struct F2ToS {
 
 // One stage of radix R after a product Ns of earlier radices.  FROM_S: the inputs are the tile, which TO_S
 // overwrites.
-template <int P, int R, int Ns, bool INV, bool FROM_S, bool TO_S, class In, class Out>
+template <int P, class RW, int R, int Ns, bool INV, bool FROM_S, bool TO_S, class In, class Out>
 __device__ __forceinline__ void f2_stage(const F2Tile& t, In in, Out out) {
-  constexpr int NB = fx_nb(R), nbf = P / R;
+  constexpr int NB = RW::nb(R), nbf = P / R;
   const int total = nbf * t.W;
   const int lane = t.tid & (t.W - 1);
   cf2 v[NB][R];
@@ -115,9 +122,9 @@ __device__ __forceinline__ void f2_stage(const F2Tile& t, In in, Out out) {
 template <int P, class RW, bool INV, bool REV, int s, int s1>
 __device__ __forceinline__ void f2_mid_stages(const F2Tile& t) {
   if constexpr (s < s1) {
-    constexpr FxPlan pl = fx_plan(P);
-    constexpr int R = pl.r[REV ? pl.n - 1 - s : s], Ns = REV ? fx_prod(P, pl.n - s, pl.n) : fx_prod(P, 0, s);
-    f2_stage<P, R, Ns, INV, true, true>(t, F2FromS<RW>{t.S}, F2ToS<RW>{t.S});
+    constexpr F2Plan pl = RW::plan;
+    constexpr int R = pl.r[REV ? pl.n - 1 - s : s], Ns = REV ? RW::prod(pl.n - s, pl.n) : RW::prod(0, s);
+    f2_stage<P, RW, R, Ns, INV, true, true>(t, F2FromS<RW>{t.S}, F2ToS<RW>{t.S});
     f2_mid_stages<P, RW, INV, REV, s + 1, s1>(t);
   }
 }
@@ -215,12 +222,12 @@ __device__ __forceinline__ void f2_load_ext(const PassParams& p, const F2Tile& t
 // Forward transform of real data into the tile.
 template <int P, class RW>
 __device__ __forceinline__ void f2_forward_real(const PassParams& p, const F2Tile& t, int type, const float* in, int q0) {
-  constexpr FxPlan pl = fx_plan(P);
+  constexpr F2Plan pl = RW::plan;
   if ((type == T_PER || type == T_UNB) && !p.fx_host) {
     const int nu = p.n_use, npen = p.npen;
     const long long ls = p.ai.ls, js = p.ai.js;
     const bool vec = p.f2_vec & 1;
-    f2_stage<P, pl.r[0], 1, false, false, true>(
+    f2_stage<P, RW, pl.r[0], 1, false, false, true>(
         t,
         [=](auto R, auto nbf, int j, int l, cf2* v) {
           const int q = q0 + 4 * l;
@@ -236,7 +243,7 @@ __device__ __forceinline__ void f2_forward_real(const PassParams& p, const F2Til
         F2ToS<RW>{t.S});
   } else {
     f2_load_ext<P, RW>(p, t, type, in, q0);
-    f2_stage<P, pl.r[0], 1, false, true, true>(t, F2FromS<RW>{t.S}, F2ToS<RW>{t.S});
+    f2_stage<P, RW, pl.r[0], 1, false, true, true>(t, F2FromS<RW>{t.S}, F2ToS<RW>{t.S});
   }
   f2_mid_stages<P, RW, false, false, 1, pl.n>(t);
 }
@@ -244,7 +251,7 @@ __device__ __forceinline__ void f2_forward_real(const PassParams& p, const F2Til
 // Store of real data from the tile's last inverse stage.
 template <int P, class RW>
 __device__ __forceinline__ void f2_store_real(const PassParams& p, const F2Tile& t, int type, float* out, int q0) {
-  constexpr FxPlan pl = fx_plan(P);
+  constexpr F2Plan pl = RW::plan;
   constexpr int R = pl.r[pl.n - 1], Ns = P / R;
   const int nd = p.n_data, N = p.N;
   const int bt = base_type(type);
@@ -256,7 +263,7 @@ __device__ __forceinline__ void f2_store_real(const PassParams& p, const F2Tile&
   const int npen = p.npen;
   const bool vec = p.f2_vec & 2;
   if (!p.fx_host) {
-    f2_stage<P, R, Ns, true, true, false>(
+    f2_stage<P, RW, R, Ns, true, true, false>(
         t, F2FromS<RW>{t.S}, [&](auto R_, auto Ns_, int o, int l, const cf2* v) {
           const int q = q0 + 4 * l;
           if (q >= npen) return;
@@ -274,7 +281,7 @@ __device__ __forceinline__ void f2_store_real(const PassParams& p, const F2Tile&
         });
     return;
   }
-  f2_stage<P, R, Ns, true, true, true>(t, F2FromS<RW>{t.S}, F2ToS<RW>{t.S});
+  f2_stage<P, RW, R, Ns, true, true, true>(t, F2FromS<RW>{t.S}, F2ToS<RW>{t.S});
   for (int idx = t.tid; idx < nd * t.W; idx += t.nt) {
     const int l = idx / nd, i = idx % nd, q = q0 + 4 * l;
     if (q >= npen) continue;
@@ -350,13 +357,13 @@ __device__ __forceinline__ void f2_split(cf2 zk, cf2 zm, cf2& A, cf2& B) {
 }
 
 template <int KIND, int P>
-__global__ void __launch_bounds__(512, 1) k_f2(const __grid_constant__ PassParams p) {
+__global__ void __launch_bounds__(F2Block<P>::threads, 768 / F2Block<P>::threads) k_f2(const __grid_constant__ PassParams p) {
   pass_entry(p);
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr bool REAL = KIND == K_FWD_REAL || KIND == K_INV_REAL || KIND == K_FUSED_REAL;
   constexpr bool FUSED = KIND == K_FUSED_REAL || KIND == K_FUSED_C2C;
-  using RW = FxRows<P, FX_PLAIN>;
-  constexpr FxPlan pl = fx_plan(P);
+  using RW = F2Rows<P, FX_PLAIN>;
+  constexpr F2Plan pl = RW::plan;
   constexpr int ns = pl.n, half = P / 2, R0 = pl.r[0], RL = pl.r[ns - 1];
   const int W = p.W;
   const F2Smem m = f2_smem(smraw, W, RW::size);
@@ -480,7 +487,7 @@ __global__ void __launch_bounds__(512, 1) k_f2(const __grid_constant__ PassParam
       }
     }
     __syncthreads();
-    f2_stage<P, R0, 1, true, true, true>(t, from_s, to_s);
+    f2_stage<P, RW, R0, 1, true, true, true>(t, from_s, to_s);
     f2_mid_stages<P, RW, true, false, 1, ns - 1>(t);
     f2_store_real<P, RW>(p, t, type, (float*)p.out + bo, q0);
   } else if constexpr (KIND == K_FUSED_REAL) {
@@ -503,7 +510,7 @@ __global__ void __launch_bounds__(512, 1) k_f2(const __grid_constant__ PassParam
       }
     }
     __syncthreads();
-    f2_stage<P, R0, 1, true, true, true>(t, from_s, to_s);
+    f2_stage<P, RW, R0, 1, true, true, true>(t, from_s, to_s);
     f2_mid_stages<P, RW, true, false, 1, ns - 1>(t);
     f2_store_real<P, RW>(p, t, type, (float*)p.out + bo, q0);
   } else {
@@ -538,7 +545,7 @@ __global__ void __launch_bounds__(512, 1) k_f2(const __grid_constant__ PassParam
         if (r * Ns.value < lim) f2_store2(d, ols, ql, npen, vout, v[r]);
     };
     if constexpr (KIND == K_FUSED_C2C) {
-      f2_stage<P, R0, 1, false, false, true>(t, load, to_s);
+      f2_stage<P, RW, R0, 1, false, false, true>(t, load, to_s);
       f2_mid_stages<P, RW, false, false, 1, ns>(t);
       // u^ = G^ f^ in the first inverse stage (radices reversed)
       if (tma_g) {
@@ -557,14 +564,14 @@ __global__ void __launch_bounds__(512, 1) k_f2(const __grid_constant__ PassParam
           v[r] = f2_scale(v[r], g);
         }
       };
-      f2_stage<P, RL, 1, true, true, true>(t, gained, to_s);
+      f2_stage<P, RW, RL, 1, true, true, true>(t, gained, to_s);
       f2_mid_stages<P, RW, true, true, 1, ns - 1>(t);
-      f2_stage<P, R0, P / R0, true, true, false>(t, from_s, store);
+      f2_stage<P, RW, R0, P / R0, true, true, false>(t, from_s, store);
     } else {
       constexpr bool INV = KIND == K_INV_C2C;
-      f2_stage<P, R0, 1, INV, false, true>(t, load, to_s);
+      f2_stage<P, RW, R0, 1, INV, false, true>(t, load, to_s);
       f2_mid_stages<P, RW, INV, false, 1, ns - 1>(t);
-      f2_stage<P, RL, P / RL, INV, true, false>(t, from_s, store);
+      f2_stage<P, RW, RL, P / RL, INV, true, false>(t, from_s, store);
     }
   }
 }
@@ -608,8 +615,8 @@ template <bool REAL, int P>
 __global__ void __launch_bounds__(512, 1) k_f2_curl(const __grid_constant__ PassParams p) {
   pass_entry(p);
   extern __shared__ __align__(16) unsigned char smraw[];
-  using RW = FxRows<P, FX_CURL>;
-  constexpr FxPlan pl = fx_plan(P);
+  using RW = F2Rows<P, FX_CURL>;
+  constexpr F2Plan pl = RW::plan;
   constexpr int ns = pl.n, half = P / 2, R0 = pl.r[0], RL = pl.r[ns - 1];
   constexpr int per = REAL ? 4 : 2, NP = REAL ? 2 : 1;  // pencils and pencil pairs of a lane
   const int W = p.W, tid = threadIdx.x, nt = blockDim.x, axis = p.axis;
@@ -655,7 +662,7 @@ __global__ void __launch_bounds__(512, 1) k_f2_curl(const __grid_constant__ Pass
       const float2* in = (const float2*)p.in + bi + mine * p.ai.cs + (long long)ql * ils;
       const int n_in = p.n_use;
       const bool vin = p.f2_vec & 1;
-      f2_stage<P, R0, 1, false, false, true>(
+      f2_stage<P, RW, R0, 1, false, false, true>(
           t,
           [=](auto R, auto nbf, int j, int, cf2* v) {
             const float2* s = in + (long long)j * ijs;
@@ -713,17 +720,17 @@ __global__ void __launch_bounds__(512, 1) k_f2_curl(const __grid_constant__ Pass
   {
     const F2FromS<RW> from_s{t.S};
     if constexpr (REAL) {
-      f2_stage<P, R0, 1, true, true, true>(t, from_s, F2ToS<RW>{t.S});
+      f2_stage<P, RW, R0, 1, true, true, true>(t, from_s, F2ToS<RW>{t.S});
       f2_mid_stages<P, RW, true, false, 1, ns - 1>(t);
       f2_store_real<P, RW>(p, t, (g.utypes >> (4 * mine)) & 15, (float*)p.out + bo + mine * p.ao.cs, q0);
     } else {
-      f2_stage<P, RL, 1, true, true, true>(t, from_s, F2ToS<RW>{t.S});
+      f2_stage<P, RW, RL, 1, true, true, true>(t, from_s, F2ToS<RW>{t.S});
       f2_mid_stages<P, RW, true, true, 1, ns - 1>(t);
       float2* out = (float2*)p.out + bo + mine * p.ao.cs + (long long)ql * ols;
       const int dup = (p.type == T_PER && p.center == C_NODE && p.n_data > p.N) ? p.N : -1;
       const int n_out = p.n_data;
       const bool vout = p.f2_vec & 2;
-      f2_stage<P, R0, P / R0, true, true, false>(t, from_s, [=](auto R, auto Ns, int o_, int, const cf2* v) {
+      f2_stage<P, RW, R0, P / R0, true, true, false>(t, from_s, [=](auto R, auto Ns, int o_, int, const cf2* v) {
         if (ql >= npen) return;
         float2* d = out + (long long)o_ * ojs;
         const long long step = (long long)Ns.value * ojs;

@@ -138,4 +138,115 @@ __host__ __device__ constexpr int fx_prod(int P, int s0, int s1) {
   return n;
 }
 
+// ---------------------------------------------------------------------------
+// Plans of the FP32 lane-pair passes.  Their kernels wait for memory rather than for arithmetic, so a thread takes one
+// butterfly of at most 9 values: half the registers of the plans above, twice the warps per SM (unbounded 192^3 447 ->
+// 372 us, channel 256^3 338 -> 300).  Lengths that would need a fourth stage keep the plans above (768 points
+// 60 us against 80), and so does the Biot-Savart pass, whose three tiles fill the SM (256 points 101 against 130).
+// ---------------------------------------------------------------------------
+#define F2_LENGTHS(X) \
+  X(4, 2, 2, 2, 1, 1, 1) \
+  X(6, 2, 3, 2, 1, 1, 1) \
+  X(8, 2, 4, 2, 1, 1, 1) \
+  X(9, 2, 3, 3, 1, 1, 1) \
+  X(12, 2, 4, 3, 1, 1, 1) \
+  X(16, 2, 8, 2, 1, 1, 1) \
+  X(18, 2, 9, 2, 1, 1, 1) \
+  X(24, 2, 8, 3, 1, 1, 1) \
+  X(27, 2, 9, 3, 1, 1, 1) \
+  X(32, 2, 8, 4, 1, 1, 1) \
+  X(36, 2, 6, 6, 1, 1, 1) \
+  X(48, 2, 8, 6, 1, 1, 1) \
+  X(54, 2, 9, 6, 1, 1, 1) \
+  X(64, 2, 8, 8, 1, 1, 1) \
+  X(72, 2, 9, 8, 1, 1, 1) \
+  X(81, 2, 9, 9, 1, 1, 1) \
+  X(96, 3, 8, 4, 3, 1, 1) \
+  X(108, 3, 9, 4, 3, 1, 1) \
+  X(128, 3, 8, 2, 8, 1, 1) \
+  X(144, 3, 9, 8, 2, 1, 1) \
+  X(162, 3, 9, 9, 2, 1, 1) \
+  X(192, 3, 8, 3, 8, 1, 1) \
+  X(216, 3, 6, 6, 6, 1, 1) \
+  X(243, 3, 9, 9, 3, 1, 1) \
+  X(256, 3, 8, 4, 8, 1, 1) \
+  X(288, 3, 9, 8, 4, 1, 1) \
+  X(324, 3, 9, 9, 4, 1, 1) \
+  X(384, 3, 8, 6, 8, 1, 1) \
+  X(432, 3, 9, 8, 6, 1, 1) \
+  X(486, 3, 9, 9, 6, 1, 1) \
+  X(512, 3, 8, 8, 8, 1, 1) \
+  X(576, 3, 8, 9, 8, 1, 1) \
+  X(648, 3, 9, 9, 8, 1, 1) \
+  X(729, 3, 9, 9, 9, 1, 1) \
+  X(768, 3, 16, 3, 16, 1, 1) \
+  X(864, 3, 12, 6, 12, 1, 1) \
+  X(972, 4, 9, 9, 4, 3, 1) \
+  X(1024, 3, 8, 16, 8, 1, 1) \
+  X(1152, 3, 12, 8, 12, 1, 1) \
+  X(1296, 4, 6, 6, 6, 6, 1) \
+  X(1458, 4, 9, 9, 9, 2, 1) \
+  X(1536, 4, 8, 8, 3, 8, 1) \
+  X(1728, 3, 12, 12, 12, 1, 1) \
+  X(1944, 4, 6, 9, 6, 6, 1) \
+  X(2048, 3, 16, 8, 16, 1, 1) \
+  X(2187, 4, 9, 9, 9, 3, 1) \
+  X(2304, 3, 12, 16, 12, 1, 1) \
+  X(2592, 4, 9, 9, 8, 4, 1) \
+  X(2916, 4, 9, 9, 9, 4, 1) \
+  X(3072, 4, 8, 16, 3, 8, 1) \
+  X(3456, 4, 12, 12, 2, 12, 1) \
+  X(3888, 4, 6, 12, 9, 6, 1) \
+  X(4096, 3, 16, 16, 16, 1, 1)
+
+struct F2Plan {
+  int n, r[5];
+};
+__host__ __device__ constexpr F2Plan f2_plan(int P) {
+  switch (P) {
+#define F2_ROW(P, n, a, b, c, d, e) \
+  case P: return F2Plan{n, {a, b, c, d, e}};
+    F2_LENGTHS(F2_ROW)
+#undef F2_ROW
+  }
+  return F2Plan{0, {1, 1, 1, 1, 1}};
+}
+__host__ __device__ constexpr F2Plan f2_plan_of(int cls, int P) {
+  if (cls != FX_CURL) return f2_plan(P);
+  const FxPlan f = fx_plan(P);
+  return F2Plan{f.n, {f.r[0], f.r[1], f.r[2], f.r[3], 1}};
+}
+// butterflies of radix R a thread takes: one of the small plans' butterflies, as many as in fx_nb in the others
+__host__ __device__ constexpr int f2_nb(int cls, int P, int R) {
+  const F2Plan f = f2_plan_of(cls, P);
+  const bool small = cls != FX_CURL && f.n <= 3 && f.r[0] <= 9 && f.r[1] <= 9 && f.r[2] <= 9;
+  return !small ? fx_nb(R) : (R == 4 ? 2 : (R == 3 ? 3 : (R == 2 ? 4 : 1)));
+}
+__host__ __device__ constexpr int f2_ept(int cls, int P) {
+  int e = 18;
+  for (int s = 0; s < f2_plan_of(cls, P).n; ++s) {
+    const int R = f2_plan_of(cls, P).r[s], v = R * f2_nb(cls, P, R);
+    if (v < e) e = v;
+  }
+  return e;
+}
+template <int P, int CLS> struct F2Rows {
+  static constexpr int W = fx_width(CLS, P);
+  static constexpr F2Plan plan = f2_plan_of(CLS, P);
+  static constexpr int B = W < 8 && plan.r[0] % 2 == 0 ? plan.r[0] : 0;
+  static constexpr int size = (P + (B ? (P - 1) / (B ? B : 1) : 0)) * W;
+  __host__ __device__ static constexpr int at(int i) { return (B ? i + i / (B ? B : 1) : i) * W; }
+  __host__ __device__ static constexpr bool linear(int n) { return !B || n % (B ? B : 1) == 0; }
+  __host__ __device__ static constexpr int nb(int R) { return f2_nb(CLS, P, R); }
+  __host__ __device__ static constexpr int prod(int s0, int s1) {
+    int n = 1;
+    for (int s = s0; s < s1; ++s) n *= f2_plan_of(CLS, P).r[s];
+    return n;
+  }
+};
+__host__ __device__ constexpr int f2_tile_values(int cls, int P) {
+  const int W = fx_width(cls, P), r0 = f2_plan_of(cls, P).r[0];
+  return (P + (W < 8 && r0 % 2 == 0 ? (P - 1) / r0 : 0)) * W;
+}
+
 }  // namespace flups

@@ -78,5 +78,10 @@ int main() {
   for (int i = 0; i < P; ++i)                                                                                 \
     if (FxRows<P, FX_PLAIN>::at(i) + FxRows<P, FX_PLAIN>::W > (i + 1 < P ? FxRows<P, FX_PLAIN>::at(i + 1) : FxRows<P, FX_PLAIN>::size)) return 4;
   FX_LENGTHS(ROWS)
+#define ROWS2(P, N, r0, r1, r2, r3, r4)                                                                           \
+  if (F2Rows<P, FX_PLAIN>::size != f2_tile_values(FX_PLAIN, P) || F2Rows<P, FX_CURL>::size != f2_tile_values(FX_CURL, P)) \
+    return 5;                                                                                                     \
+  if (r0 * r1 * r2 * r3 * r4 != P || F2Rows<P, FX_PLAIN>::prod(0, N) != P || f2_ept(FX_PLAIN, P) < 6) return 6;
+  F2_LENGTHS(ROWS2)
   return 0;
 }
