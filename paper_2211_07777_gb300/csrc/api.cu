@@ -1332,11 +1332,19 @@ int flups_init_solver(flups_topo t, const int* bc, const double h[3], const doub
     }
   }
   if (rc == FLUPS_OK) rc = build_plan(s);
-  // FP64-class Poisson solves run in 64-bit fixed point, except the smallest: up to 2^16 points of the extended
-  // box a pass is one warp's chain of instructions, and the short FP64 columns of the warp engine are
-  // faster (measured, us per solve, FP64 / fixed point: periodic 32^3 25.7 / 29.9, unbounded 16^3 25.1 / 29.0,
-  // against periodic 36^3 39.8 / 28.6, unbounded 24^3 55.4 / 33.2, unbounded 64^3 230 / 76)
-  s->fxp = t->prec != FLUPS_F32 && (long long)s->dir[0].P * s->dir[1].P * s->dir[2].P > 65536;
+  // FP64-class solves run in 64-bit fixed point, except the smallest, where a pass is one warp's chain of
+  // instructions and the short columns of the warp engine are as fast or faster.  Measured, us per solve without / with
+  // fixed point, by points of the extension: FP64 periodic 16^3 22.4 / 24.0, 27^3 34.4 / 35.3, 32^3 25.8 / 25.7, 32 x 32
+  // x 36 31.4 / 25.1, open 18^3 (46656) 36.9 / 22.8, walls and open 16^3 (65536) 39.0 / 34.3, Biot-Savart periodic 36^3
+  // 73.8 / 51.2.  The double-float passes are faster than the FP64 ones: 32 x 32 x 36 (36864) 24.6 / 25.0, periodic 36^3
+  // 32.0 / 24.1, open 18^3 29.4 / 22.8, but in powers of two, whose columns stay in registers, walls and open 16^3
+  // 30.6 / 34.3; around their curl Biot-Savart at 8 x 8 x 972 127 / 148.
+  {
+    bool pow2 = true;
+    for (int d = 0; d < 3; ++d) pow2 &= (s->dir[d].P & (s->dir[d].P - 1)) == 0;
+    const long long least = t->prec == FLUPS_F64 ? 32768 : (pow2 || op == FLUPS_BIOT_SAVART ? 65536 : 36864);
+    s->fxp = t->prec != FLUPS_F32 && (long long)s->dir[0].P * s->dir[1].P * s->dir[2].P > least;
+  }
   s->fx = s->fxp && op == FLUPS_POISSON;
   if (rc == FLUPS_OK) {
     int du = 0;

@@ -82,3 +82,15 @@ def test_non_finite_input_makes_the_solution_nan(bad):
 
 def test_both_fp64_precisions_run_the_same_passes():
     assert np.array_equal(_solve(_field(), F.F64), _solve(_field(), F.F64E))
+
+
+# both sides of the line between the warp engine and fixed point: extensions of 32768, 36864 and 46656 points
+@pytest.mark.parametrize("prec", [F.F64, F.F64E])
+@pytest.mark.parametrize("n", [(32, 32, 32), (32, 32, 36), (36, 36, 36), (8, 16, 512)])
+def test_sizes_around_the_line_match_the_oracle(n, prec):
+    f = np.random.default_rng(sum(n)).standard_normal(n[::-1])
+    h = (1.0 / max(n),) * 3
+    got = cuda_solve(f, ((PER, PER),) * 3, CELL, prec, "spectral", h=h, L=tuple(v * h[0] for v in n))[0]
+    ref = oracle.solve(f, oracle.Problem(bc=((PER, PER),) * 3, h=h, center=CELL, kernel="spectral"))
+    # double-float passes (at most 15 butterfly levels of 2u, u = 2^-48, per direction and way) bound the pair
+    assert np.linalg.norm(got - ref) < 6 * 15 * 2.0 ** -47 * np.linalg.norm(ref)
