@@ -20,12 +20,15 @@ template <> __device__ __forceinline__ void st_real<dfloat>(dfloat* a, long long
   else reinterpret_cast<float2*>(a)[off] = make_float2(v.hi, v.lo);
 }
 
-// The same for complex values (a double-float pass between fixed-point ones reads and writes FP64 arrays).
-template <typename T> __device__ __forceinline__ cpx<T> ld_cplx(const cpx<T>* a, long long off, int f64) { return a[off]; }
-template <> __device__ __forceinline__ cdfloat ld_cplx<dfloat>(const cdfloat* a, long long off, int f64) {
-  if (!f64) return a[off];
-  const double2 q = reinterpret_cast<const double2*>(a)[off];
-  return mk<dfloat>(df_from_double(q.x), df_from_double(q.y));
+// The same for complex values (a double-float pass between fixed-point ones reads and writes FP64 arrays).  Loads take
+// the element's 16 bytes as they are and convert where it is used: a branch between the loads of a batch would wait
+// for each before the next.
+template <typename T> __device__ __forceinline__ cpx<T> from_array(cpx<T> v, int f64) { return v; }
+template <> __device__ __forceinline__ cdfloat from_array<dfloat>(cdfloat v, int f64) {
+  if (!f64) return v;
+  return mk<dfloat>(
+      df_from_double(__hiloint2double(__float_as_int(v.x.lo), __float_as_int(v.x.hi))),
+      df_from_double(__hiloint2double(__float_as_int(v.y.lo), __float_as_int(v.y.hi))));
 }
 template <typename T> __device__ __forceinline__ void st_cplx(cpx<T>* a, long long off, cpx<T> v, int f64) { a[off] = v; }
 template <> __device__ __forceinline__ void st_cplx<dfloat>(cdfloat* a, long long off, cdfloat v, int f64) {
@@ -319,12 +322,12 @@ __device__ __forceinline__ void load_cplx(const PassParams& p, const cpx<T>* __r
       ll[u] = lane;
       ii[u] = i;
       const int q = q0 + lane;
-      v[u] = (i >= 0 && q < p.npen) ? ld_cplx<T>(in, (long long)q * p.ai.ls + (long long)i * p.ai.js, p.in_f64)
+      v[u] = (i >= 0 && q < p.npen) ? in[(long long)q * p.ai.ls + (long long)i * p.ai.js]
                                     : mk<T>((T)0, (T)0);
     }
 #pragma unroll
     for (int u = 0; u < LOADB; ++u)
-      if (ii[u] >= 0) S[tix<T, WC>(ii[u], ll[u], LS)] = v[u];
+      if (ii[u] >= 0) S[tix<T, WC>(ii[u], ll[u], LS)] = from_array<T>(v[u], p.in_f64);
   }
 }
 
