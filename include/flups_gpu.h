@@ -52,10 +52,11 @@ typedef enum {
 typedef enum { FLUPS_EVEN = 0, FLUPS_ODD = 1, FLUPS_PER = 3, FLUPS_UNB = 4 } flups_bc;
 /* Data layout (Section 2.1). */
 typedef enum { FLUPS_CELL = 0, FLUPS_NODE = 1 } flups_center;
-/* Arithmetic of the transforms.  FLUPS_F64E: FP64 arrays (as FLUPS_F64) with
- * the transforms in double-float arithmetic on the FP32 units (about 48
- * significant bits, error within the FP64 path's 1e-12 bound); every size,
- * boundary condition, kernel and operator of the other paths. */
+/* Arithmetic of the transforms.  FLUPS_F64 and FLUPS_F64E both
+ * work on FP64 arrays and transform in 64-bit block fixed point on the
+ * integer units; small problems and the Biot-Savart curl run in FP64
+ * (FLUPS_F64) or in double-float arithmetic on the FP32 units (FLUPS_F64E:
+ * about 48 significant bits, error within the FP64 path's 1e-12 bound). */
 typedef enum { FLUPS_F32 = 0, FLUPS_F64 = 1, FLUPS_F64E = 2 } flups_prec;
 /* Operator. */
 typedef enum { FLUPS_POISSON = 0, FLUPS_BIOT_SAVART = 1 } flups_op;
@@ -298,11 +299,11 @@ int flups_solver_check(flups_solver s, int* code);
  * receives the FP64 real-space samples G(k_s, r_u) the setup transforms, the
  * Green index x fastest over the extents of every direction (unbounded-like:
  * r = g h, g = 0..M; spectral: the folded mode), and spectrum (n values) the
- * stored spectrum as the fused pass reads it, converted to double (the
- * double-float path stores hi + lo float pairs): the
+ * stored spectrum as the fused pass reads it, converted to double (double-float
+ * passes store hi + lo float pairs, fixed-point ones integers): the
  * samples' DCT-I along each unbounded-like direction (Section 2.3: the kernel
  * symmetrised on the extended domain, transformed there; computed in
- * double-float arithmetic on the FP32 units) times prod(h_u)/(P1 P2 P3).
+ * 64-bit fixed point) times prod(h_u)/(P1 P2 P3).
  * n must be the product of the extents.  Only for solvers with a stored
  * spectrum (some direction unbounded or semi-unbounded; else FLUPS_ESTATE).
  * Synchronous; allocates a temporary device buffer.  No counterpart in the paper. */

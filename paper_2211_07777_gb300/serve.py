@@ -34,8 +34,8 @@ def vector_bc(bc):
 
 
 def engine_prec(req: W.Request, fp64_engine: str = "native") -> int:
-    """Arithmetic path for a request.  FP64-class requests run natively, or -- with
-    fp64_engine="df" -- on the double-float path (FP64 tolerance on the FP32 units)."""
+    """Arithmetic path for a request.  FP64-class requests run as FP64, or -- with
+    fp64_engine="df" -- as FP64E (the same passes except in small problems and the curl)."""
     if fp64_engine == "df" and req.prec == F.F64:
         return F.F64E
     return req.prec
