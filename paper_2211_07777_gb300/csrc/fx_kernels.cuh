@@ -269,13 +269,16 @@ __device__ __forceinline__ void fx_green_base(const PassParams& p, int q, int o,
 }
 
 // Load of real data pairs whose extension is built in the tile (symmetric and semi-unbounded directions, and
-// every real pass on pinned host arrays): items (lane, i < n_data), at most U per thread.
+// every real pass on pinned host arrays): items (lane, i < n_data), at most U per thread.  Values that the extension
+// has no place for (odd node faces, the duplicate periodic node) count as 0 before the lane's exponent is taken.
 template <int P, class RW, int U>
 __device__ __forceinline__ void fx_load_ext(const PassParams& p, const FxTile& t, int type, const double* in, int q0,
                                             int* emax) {
   const int W = t.W, N = p.N, nd = p.n_data, tot = nd * W;
   const int bt = base_type(type);
-  const bool rev = is_reversed(type);
+  const bool rev = is_reversed(type), node = p.center == C_NODE;
+  const int z0 = node && (bt == T_OO || bt == T_OE || bt == T_OU) ? 0 : -1;
+  const int zN = node && (bt == T_OO || bt == T_EO || bt == T_PER) ? N : -1;
   cfx* S = t.S;
   double a[U], b[U];
 #pragma unroll
@@ -286,9 +289,10 @@ __device__ __forceinline__ void fx_load_ext(const PassParams& p, const FxTile& t
       const int l = p.fx_host ? idx / nd : idx & (W - 1), i = p.fx_host ? idx % nd : idx >> t.lw;
       const int qa = q0 + 2 * l;
       const long long off = (long long)qa * p.ai.ls + (long long)i * p.ai.js;
-      if (qa < p.npen) a[u] = in[off];
-      if (qa + 1 < p.npen) b[u] = in[off + p.ai.ls];
-      if (p.type == T_PER && i >= N) a[u] = b[u] = 0.0;  // the duplicate node is not used
+      const int dix = rev ? nd - 1 - i : i;
+      const bool used = dix != z0 && dix != zN;
+      if (used && qa < p.npen) a[u] = in[off];
+      if (used && qa + 1 < p.npen) b[u] = in[off + p.ai.ls];
       if (p.fx_host) atomicMax(&emax[l], (int)(max(abs_hi(a[u]), abs_hi(b[u])) >> 20));
     }
   }

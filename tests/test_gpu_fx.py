@@ -80,6 +80,37 @@ def test_non_finite_input_makes_the_solution_nan(bad):
     assert np.isnan(_solve(f)).all()
 
 
+# Node-centred odd faces: the extension holds zeros there, whatever the caller's array has
+@pytest.mark.parametrize("host", [False, True], ids=["device", "pinned"])
+@pytest.mark.parametrize("bad", [1e20, np.nan])
+@pytest.mark.parametrize("prec", [F.F64, F.F64E], ids=["f64", "f64e"])
+@pytest.mark.parametrize("faces", [(O, O), (O, E), (E, O), (U, O), (O, U)], ids=["oo", "oe", "eo", "uo", "ou"])
+def test_values_on_odd_node_faces_take_no_part(faces, prec, bad, host):
+    import torch
+    bcs, n = (faces, (PER, PER), (PER, PER)), (36, 32, 32)  # x goes first
+    f = np.random.default_rng(6).standard_normal((n[2] + 1, n[1] + 1, n[0] + 1))
+    zero, dirty = f.copy(), f.copy()
+    for side in (0, 1):
+        if faces[side] == O:
+            zero[:, :, -side], dirty[:, :, -side] = 0.0, bad
+    out = []
+    with F.Solver((37, 33, 33), bcs, center=NODE, prec=prec, green="hej2" if U in faces else "spectral", h=(1 / 36,) * 3,
+                  L=tuple(v / 36 for v in n)) as s:
+        for a in (zero, dirty):
+            if host:
+                rhs = torch.from_numpy(a).pin_memory()
+                phi = torch.empty_like(rhs).pin_memory()
+                s.solve_host(phi, rhs)
+            else:
+                rhs = torch.from_numpy(a).cuda()
+                phi = torch.empty_like(rhs)
+                s.solve(phi, rhs)
+            torch.cuda.synchronize()
+            out.append(phi.cpu().numpy())
+    assert np.isfinite(out[0]).all()
+    assert np.array_equal(out[0], out[1])
+
+
 def test_both_fp64_precisions_run_the_same_passes():
     assert np.array_equal(_solve(_field(), F.F64), _solve(_field(), F.F64E))
 
