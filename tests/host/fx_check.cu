@@ -65,7 +65,30 @@ int main() {
     if (fx_halves(x.x) != (long long)(((unsigned long long)(unsigned)fx_hi(x.x) << 32) | (unsigned)fx_lo(x.x))) return 1;
     if ((ld)fx_hi(x.x) * 0x1p32L + fx_lo(x.x) != (ld)x.x) return 1;
   }
-  std::printf("cmul %.3Lg\nmul %.3Lg\ndecode %.3Lg\n", wc, wm, wd);
+  std::printf("cmul %.3Lg\nmul %.3Lg\ndecode %.4Lg\n", wc, wm, wd);
+  // Mean decoding error of positive values 2^-d below the lane's largest, beyond the ties' bias of half a unit of the
+  // value's own precision, and of values uniform up to the lane's largest: a one-sign field's errors must not add up.
+  ld worst = 0, all = 0;
+  for (int up = kFxUp; up <= kFxUp + kFxTwShift; up += kFxTwShift)
+    for (int d = 0; d <= 48; ++d) {
+      ld sum = 0;
+      const int n = 100000;
+      for (int i = 0; i < n; ++i) {
+        unsigned long long b = ((unsigned long long)(1000 - d) << 52) | (gen() >> 12);
+        double v;
+        std::memcpy(&v, &b, 8);
+        if (d == 0) {
+          v = (double)ldexpl((ld)gen() + ldexpl((ld)gen(), -64), 1000 - 1023 - 64);
+          std::memcpy(&b, &v, 8);
+        }
+        const ld e = fx_decode(b, 1000, up) - ldexpl(v, 1075 + up - 1000);
+        sum += e;
+        wd = std::fmax(wd, std::fabs(e));
+      }
+      if (d == 0) all = std::fmax(all, std::fabs(sum) / n);
+      else worst = std::fmax(worst, std::fabs(sum) / n - (d > up ? ldexpl(0.5L, up - d) : 0));
+    }
+  std::printf("decode_all %.4Lg\ndecode_mean %.3Lg\ndecode_binade %.3Lg\n", wd, all, worst);
   std::printf("zero %lld\nsubnormal %lld\n", fx_decode(0, kFxMinE), fx_decode(0x800fffffffffffffull, kFxMinE));
   std::printf("shr_even %lld\n", fx_shr(24, 4) * 100 + fx_shr(8, 4) * 10 + fx_shr(7, 0));  // 1.5 -> 2, 0.5 -> 0, 7
   // every plan multiplies to its length within the block limits

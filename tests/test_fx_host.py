@@ -39,6 +39,13 @@ def test_register_dfts_match_the_definition(errors, R):
 def test_products_and_decoding(errors):
     assert errors["cmul"] < 1.5      # two parts of at most 0.5 + 0.25 + 0.25 units
     assert errors["mul"] < 1.0
-    assert errors["decode"] <= 1.0   # truncated below the lane's last bit
+    assert errors["decode"] <= 0.5 and errors["decode_all"] <= 0.5   # rounded to nearest
     assert errors["zero"] == 0 and errors["subnormal"] == 0
     assert errors["shr_even"] == 207
+
+
+def test_decoding_has_no_preferred_direction(errors):
+    """Mean error over 100000 positive values, uniform and at each distance below the lane's largest: truncation has half
+    a unit, rounding to nearest a standard error of 0.3 / sqrt(100000) = 0.001 and the ties' bias, in all 2^-5 / 4 +
+    2^-6 / 8 + ... = 0.0104 of a unit for uniform values."""
+    assert errors["decode_mean"] < 0.015 and errors["decode_binade"] < 0.01
