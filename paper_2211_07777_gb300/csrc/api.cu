@@ -148,7 +148,6 @@ struct flups_solver_s {
   void* W1 = nullptr;
   void* W2 = nullptr;
   void* green_dev = nullptr;
-  int* green_exp = nullptr;     // fixed-point spectrum: exponent of each pencil's slice
   int green_pitch = 0;          // x pitch (elements) of the stored spectrum
   bool fx = false;              // every pass in 64-bit fixed point (FP64-class Poisson solves)
   bool fxp = false;             // the passes of the first two directions are (Biot-Savart solves too)
@@ -480,8 +479,8 @@ void fx_geom(Launch& L, const DirPlan& dp, int axis, bool packed) {
   p.ept = 0;
   L.grid.x = (unsigned)((need + W - 1) / W);
   L.nthr = nt;
-  // alignment, mbarrier block, tile, Green offsets and exponents, lane exponents, renormalisation words
-  L.smem = 128 + 128 + (size_t)fx_tile_values(cls, P) * 16 + (size_t)W * (2 * 8 + 4 + 2 * 4 + kFxSlots * 4);
+  // alignment, mbarrier block, tile, Green offsets, lane exponents, renormalisation words
+  L.smem = 128 + 128 + (size_t)fx_tile_values(cls, P) * 16 + (size_t)W * (2 * 8 + 4 + kFxSlots * 4);
   p.rowx = (axis == 0 && p.center == C_CELL && (p.type == T_PER || p.type == T_UNB) &&
             (L.kind == K_FWD_REAL || L.kind == K_INV_REAL)) ? 1 : 0;
 }
@@ -566,16 +565,17 @@ cudaError_t sample_green(const flups_solver_s* s, const GreenSampleParams& q, do
   return (s->green == FLUPS_LGF2) ? launch_lgf(g64, q.gext, q.h, st) : launch_green_sample(g64, q, st);
 }
 
+// Bytes of the stored spectrum: rows at green_pitch and, for the fixed-point passes, a block with its reference exponent.
+size_t green_stored_bytes(const flups_solver_s* s) {
+  return (size_t)s->green_pitch * s->dir[1].gext * s->dir[2].gext * esize(s->topo.prec) + (s->fx ? 16 : 0);
+}
+int* green_ref(const flups_solver_s* s) { return (int*)((char*)s->green_dev + green_stored_bytes(s) - 16); }
+
 // The spectrum g64 times scale into green_dev, in the passes' format.
 cudaError_t store_green(flups_solver_s* s, const double* g64, const int* gext, double scale, cudaStream_t st) {
   const long long n = (long long)gext[0] * gext[1] * gext[2];
-  if (!s->fx) return launch_green_finalize(g64, s->green_dev, s->topo.prec, n, gext[0], s->green_pitch, scale, st);
-  const int ax = s->order[2];
-  const size_t bytes = (size_t)(n / gext[ax]) * sizeof(int);
-  cudaError_t e = cudaMallocAsync((void**)&s->green_exp, bytes, st);
-  if (e) return e;
-  s->ws_bytes += bytes;
-  return launch_green_finalize_fx(g64, s->green_dev, s->green_exp, gext, s->green_pitch, ax, scale, !s->cplx[2], st);
+  if (s->fx) return launch_green_finalize_fx(g64, s->green_dev, green_ref(s), n, gext[0], s->green_pitch, scale, st);
+  return launch_green_finalize(g64, s->green_dev, s->topo.prec, n, gext[0], s->green_pitch, scale, st);
 }
 
 int setup_green_compute(flups_solver_s* s, cudaStream_t st) {
@@ -623,7 +623,7 @@ int setup_green_compute(flups_solver_s* s, cudaStream_t st) {
       const double* tabs[3] = {(const double*)s->tabs[0], (const double*)s->tabs[1], (const double*)s->tabs[2]};
       cudaError_t e = launch_green_spectral(g64, gext, tabs, s->green, 0.5 * s->eps * s->eps, 1.0 / Pprod, st);
       s->green_pitch = (gext[0] + 1) & ~1;  // 16-byte rows (8-byte elements)
-      const size_t padded = (size_t)s->green_pitch * gext[1] * gext[2] * 8;
+      const size_t padded = green_stored_bytes(s);
       if (!e) e = cudaMallocAsync(&s->green_dev, padded, st);
       if (!e) e = store_green(s, g64, gext, 1.0, st);
       cudaFreeAsync(g64, st);
@@ -673,7 +673,7 @@ int setup_green_compute(flups_solver_s* s, cudaStream_t st) {
   // x rows padded to 16 bytes (TMA tensor maps need 16-byte strides)
   const int per16 = (int)(16 / esize(prec));
   s->green_pitch = (q.gext[0] + per16 - 1) / per16 * per16;
-  const size_t padded = (size_t)s->green_pitch * q.gext[1] * q.gext[2] * esize(prec);
+  const size_t padded = green_stored_bytes(s);
   e = cudaMallocAsync(&s->green_dev, padded, st);
   if (e) { cudaFreeAsync(g64, st); return cuda_fail(e, "green alloc"); }
   e = store_green(s, g64, q.gext, scale, st);
@@ -693,7 +693,6 @@ int setup_green_compute(flups_solver_s* s, cudaStream_t st) {
 // serving runtime releases idle plans only).
 struct GreenEntry {
   void* dev;
-  int* gexp;
   int pitch;
   double bytes;
   size_t padded;
@@ -711,9 +710,7 @@ std::string green_cache_key(const flups_solver_s* s) {
   put(&s->topo.prec, sizeof s->topo.prec);
   put(&s->green, sizeof s->green);
   put(&s->eps, sizeof s->eps);
-  // fixed-point spectra depend on the fused direction and on whether its pass is real
-  const int fmt = s->fx ? 1 + s->order[2] + 3 * s->cplx[2] : 0;
-  put(&fmt, sizeof fmt);
+  put(&s->fx, sizeof s->fx);  // the fixed-point passes' own format
   for (int d = 0; d < 3; ++d) {
     const DirPlan& dp = s->dir[d];
     put(&dp.unb, sizeof dp.unb);
@@ -740,7 +737,6 @@ int setup_green(flups_solver_s* s, cudaStream_t st) {
     if (it != g_green_cache.end()) {
       it->second.refs++;
       s->green_dev = it->second.dev;
-      s->green_exp = it->second.gexp;
       s->green_pitch = it->second.pitch;
       s->green_bytes = it->second.bytes;
       s->green_key = key;
@@ -754,14 +750,12 @@ int setup_green(flups_solver_s* s, cudaStream_t st) {
   if (it != g_green_cache.end()) {
     // another solver stored the same spectrum meanwhile: use that copy
     cudaFreeAsync(s->green_dev, st);
-    if (s->green_exp) cudaFreeAsync(s->green_exp, st);
     it->second.refs++;
     s->green_dev = it->second.dev;
-    s->green_exp = it->second.gexp;
     s->green_pitch = it->second.pitch;
   } else {
-    const size_t padded = (size_t)s->green_pitch * s->dir[1].gext * s->dir[2].gext * esize(s->topo.prec);
-    g_green_cache[key] = GreenEntry{s->green_dev, s->green_exp, s->green_pitch, s->green_bytes, padded, 1};
+    const size_t padded = green_stored_bytes(s);
+    g_green_cache[key] = GreenEntry{s->green_dev, s->green_pitch, s->green_bytes, padded, 1};
   }
   s->green_key = key;
   return FLUPS_OK;
@@ -1108,7 +1102,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
       }
     }
     g.stored = s->green_dev;
-    g.gexp = s->green_exp;
+    g.gref = s->fx ? green_ref(s) : nullptr;
     for (int d = 0; d < 3; ++d) {
       g.tab[d] = s->tabs[d];
       g.gext[d] = s->dir[d].gext;
@@ -1496,7 +1490,6 @@ int flups_solver_memory(flups_solver s, size_t* resident, size_t* transient, siz
   }
   if (du == 0)
     for (int d = 0; d < 3; ++d) res += (size_t)s->dir[d].gext * es;
-  if (s->fx) res += gn / s->dir[s->order[2]].gext * sizeof(int);
   if (du > 0 || s->fx) {
     res += gn * es;
     tr += gn * sizeof(double) + (size_t)8 * 2 * gmax * sizeof(double);
@@ -1543,22 +1536,17 @@ int flups_debug_green(flups_solver s, double* samples, double* spectrum, long lo
   const size_t rows = (size_t)q.gext[1] * q.gext[2];
   std::vector<unsigned char> buf(rows * s->green_pitch * es);
   CK(cudaMemcpy(buf.data(), s->green_dev, buf.size(), cudaMemcpyDeviceToHost));
-  std::vector<int> gexp;
-  if (s->fx) {
-    gexp.resize((size_t)(cnt / q.gext[s->order[2]]));
-    CK(cudaMemcpy(gexp.data(), s->green_exp, gexp.size() * sizeof(int), cudaMemcpyDeviceToHost));
-  }
-  // element formats: FP32, fixed point with an exponent per pencil, FP64, or a pair of floats (hi, lo)
+  int ref = 0;
+  if (s->fx) CK(cudaMemcpy(&ref, green_ref(s), sizeof(int), cudaMemcpyDeviceToHost));
+  // element formats: FP32, a fixed-point factor (fx_green_pack), FP64, or a pair of floats (hi, lo)
   for (size_t r = 0; r < rows; ++r)
     for (int x = 0; x < q.gext[0]; ++x) {
       const size_t i = r * s->green_pitch + x;
       double v;
       if (es == 4) v = (double)((const float*)buf.data())[i];
       else if (s->fx) {
-        const int ax = s->order[2], y = (int)(r % q.gext[1]), z = (int)(r / q.gext[1]);
-        const int pen = ax == 0 ? y + q.gext[1] * z : x + q.gext[0] * (ax == 1 ? z : y);
-        const long long g = ((const long long*)buf.data())[i];
-        v = std::ldexp((double)((long long)(int)(g >> 32) * 4294967296LL + (int)g), gexp[pen]);
+        const fxg f = fx_green(((const unsigned long long*)buf.data())[i]);
+        v = std::ldexp((double)((long long)f.h * 4294967296LL + f.l), ref - f.d - 1075 - kFxGreenUp);
       }
       else if (s->topo.prec == FLUPS_F64E) v = (double)((const float*)buf.data())[2 * i] + (double)((const float*)buf.data())[2 * i + 1];
       else v = ((const double*)buf.data())[i];
@@ -1712,15 +1700,12 @@ static void release(flups_solver s, cudaStream_t st, bool async) {
     auto it = g_green_cache.find(s->green_key);
     if (it != g_green_cache.end() && --it->second.refs == 0) {
       fr(it->second.dev);
-      fr(it->second.gexp);
       g_green_cache.erase(it);
     }
     s->green_dev = nullptr;
-    s->green_exp = nullptr;
     s->green_key.clear();
   }
   fr(s->green_dev);
-  fr(s->green_exp);
   fr(s->stage);
   fr(s->errflag);
   fr(s->gmaps_dev);

@@ -22,18 +22,17 @@ namespace {
 
 // A tile's shared memory after the 128-byte block of its mbarrier: S, then lane exponents and Green
 // offsets, then the staged Green slice (128-byte aligned).
-// renormalisation slots: second to fourth stage forward (and before the Green product, one more), after the
-// product, second to fourth stage inverse
+// renormalisation slots: second to fourth stage forward (and before the Green product, one more), the products' top
+// bit, second to fourth stage inverse
 constexpr int kFxSlotFwd = 0, kFxSlotGain = 4, kFxSlotInv = 5;
 
 struct FxSmem {
   cfx* S;
   int* emax;          // W lane exponents
-  int* gexp;          // 2 W exponents of the pencils' Green slices
   unsigned* words;    // kFxSlots x W magnitudes (upper words ORed) behind the lanes' renormalisations
   long long* goff;    // 2 W Green offsets
   unsigned long long* mbar;
-  long long* G;       // staged slice, (P/2 + 1) x W
+  unsigned long long* G;  // staged slice, (P/2 + 1) x W
 };
 
 __device__ __forceinline__ FxSmem fx_smem(unsigned char* smraw, int W, int rows) {
@@ -43,10 +42,9 @@ __device__ __forceinline__ FxSmem fx_smem(unsigned char* smraw, int W, int rows)
   m.S = reinterpret_cast<cfx*>(base + 128);
   m.goff = reinterpret_cast<long long*>(base + 128 + (size_t)rows * sizeof(cfx));
   m.emax = reinterpret_cast<int*>(m.goff + 2 * W);
-  m.gexp = m.emax + W;
-  m.words = reinterpret_cast<unsigned*>(m.gexp + 2 * W);
+  m.words = reinterpret_cast<unsigned*>(m.emax + W);
   unsigned char* g = reinterpret_cast<unsigned char*>(m.words + kFxSlots * W);
-  m.G = reinterpret_cast<long long*>(g + ((128u - (smem_u32(g) & 127u)) & 127u));
+  m.G = reinterpret_cast<unsigned long long*>(g + ((128u - (smem_u32(g) & 127u)) & 127u));
   return m;
 }
 
@@ -124,13 +122,12 @@ template <class RW> struct FxToS {
 
 // Lane renormalisation.  The fixed factor 2^-4 of a twiddled stage is what the worst case needs; a lane whose
 // values did not grow (a spectrum of a few modes) would lose those bits at every stage.  From the second stage
-// of a transform on, and after the Green product, the lane's values are therefore shifted up to the bound
+// of a transform on, and before the Green product, the lane's values are therefore shifted up to the bound
 // again: the stage before ORs the magnitudes of its outputs' upper words per lane, the next one shifts by
-// the free bits, eight integer operations per value.  (Relative error against a 64-bit solution, mixed 256^3: 1e-13
+// the free bits, eight integer operations per value.  (The Green products are aligned one by one, fx_align.)  (Relative error against a 64-bit solution, mixed 256^3: 1e-13
 // to 1.7e-12 with the fixed factors alone, 4e-16 to 5e-15 with the shift from the third stage on.)
 enum FxSrc : int { FX_TILE = 0, FX_RAW = 1, FX_GAIN = 2 };
 __device__ __forceinline__ int fx_free_tw(unsigned w) { return max(__clz(w) - 3, 0); }    // parts below 2^61
-__device__ __forceinline__ int fx_free_in(unsigned w) { return max(__clz(w) - 7, 0); }    // parts below 2^57
 __device__ __forceinline__ unsigned fx_mag(long long x) {
   const int h = (int)(x >> 32);
   return (unsigned)(h ^ (h >> 31));
@@ -139,11 +136,16 @@ __device__ __forceinline__ void lane_or(unsigned* word, unsigned m, int W, int l
   for (int o = W; o < 32; o <<= 1) m |= __shfl_xor_sync(0xffffffffu, m, o);
   if ((tid & 31) < W) atomicOr(&word[lane], m);
 }
-// Shift that the renormalisations of lane l added: forward and inverse transforms of the plan, gain.
+// Largest top bit of the lane's products.
+__device__ __forceinline__ void lane_top(unsigned* word, int m, int W, int lane, int tid) {
+  for (int o = W; o < 32; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((tid & 31) < W) atomicMax(reinterpret_cast<int*>(&word[lane]), m);
+}
+// Shift that the renormalisations of lane l added: forward and inverse transforms of the plan, before the product.
 template <int P>
 __device__ __forceinline__ int fx_shifted(const unsigned* words, int W, int l, bool fwd, bool gain, bool inv) {
   constexpr int n = fx_plan(P).n;
-  int e = gain ? fx_free_in(words[kFxSlotGain * W + l]) + fx_free_tw(words[(kFxSlotFwd + n - 1) * W + l]) : 0;
+  int e = gain ? fx_free_tw(words[(kFxSlotFwd + n - 1) * W + l]) : 0;
 #pragma unroll
   for (int s = 1; s < n; ++s) {
     if (fwd) e += fx_free_tw(words[(kFxSlotFwd + s - 1) * W + l]);
@@ -153,8 +155,8 @@ __device__ __forceinline__ int fx_shifted(const unsigned* words, int W, int l, b
 }
 
 // One stage of radix R after a product Ns of earlier radices.  SRC: FX_RAW, In gives FP64 bits, aligned to the
-// lane's exponent (maxima in `lanes`) here; FX_GAIN, In gives products to renormalise (words `lanes`).  words:
-// the transform's slots; every stage but the first is renormalised.  In and Out move whole butterflies: values
+// lane's exponent (maxima in `lanes`) here; FX_GAIN, In gives Green products (FxGained) and aligns them to the lane's
+// largest (`lanes`).  words: the transform's slots; every stage but the first is renormalised.  In and Out move whole butterflies: values
 // at positions j + r P/R, outputs at o + r Ns.
 template <int P, int R, int Ns, bool INV, int SRC, bool TO_S, int s, bool SCAN_LAST = false, class In, class Out>
 __device__ __forceinline__ void fx_stage(const FxTile& t, unsigned* lanes, unsigned* words, In in, Out out) {
@@ -164,11 +166,13 @@ __device__ __forceinline__ void fx_stage(const FxTile& t, unsigned* lanes, unsig
   const int total = nbf * t.W;
   const int lane = t.tid & (t.W - 1);
   cfx v[NB][R];
+  int top = 0;
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
     const int idx = t.tid + b * t.nt, j = idx >> t.lw;
     if (idx < total) {
-      in(ic<R>(), ic<nbf>(), j, lane, v[b]);
+      if constexpr (SRC == FX_GAIN) top = max(top, in.products(ic<R>(), ic<nbf>(), j, lane, v[b]));
+      else in(ic<R>(), ic<nbf>(), j, lane, v[b]);
     } else {
 #pragma unroll
       for (int r = 0; r < R; ++r) v[b][r] = fx_make(0, 0);
@@ -189,18 +193,19 @@ __device__ __forceinline__ void fx_stage(const FxTile& t, unsigned* lanes, unsig
 #pragma unroll
       for (int r = 0; r < R; ++r) v[b][r] = fx_make(fx_decode(v[b][r].x, E), fx_decode(v[b][r].y, E));
   } else if constexpr (SRC == FX_GAIN) {
-    unsigned m = 0;
-#pragma unroll
-    for (int b = 0; b < NB; ++b)
-#pragma unroll
-      for (int r = 0; r < R; ++r) m |= fx_mag(v[b][r].x) | fx_mag(v[b][r].y);
-    lane_or(lanes, m, t.W, lane, t.tid);
+    lane_top(lanes, top, t.W, lane, t.tid);
     __syncthreads();
+    const int T = (int)lanes[lane];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const int idx = t.tid + b * t.nt, j = idx >> t.lw;
+      if (idx < total) in.align(ic<R>(), ic<nbf>(), j, T, v[b]);
+    }
   } else if constexpr (TO_S) {
     __syncthreads();  // every input is in registers before the tile is overwritten
   }
-  if constexpr (TW || SRC == FX_GAIN) {
-    const int n = SRC == FX_GAIN ? fx_free_in(lanes[lane]) : fx_free_tw(words[(s - 1) * t.W + lane]);
+  if constexpr (TW) {
+    const int n = fx_free_tw(words[(s - 1) * t.W + lane]);
 #pragma unroll
     for (int b = 0; b < NB; ++b)
 #pragma unroll
@@ -242,31 +247,60 @@ __device__ __forceinline__ void fx_mid_stages(const FxTile& t, unsigned* words) 
   }
 }
 
-// Green offset (axis term excluded) and exponent of pencil q; past the last pencil a zero offset and an
-// exponent that takes no part in a pair's common one.
-__device__ __forceinline__ void fx_green_base(const PassParams& p, int q, int o, long long* goff, int* gexp) {
+// Green offset (axis term excluded) of pencil q; 0 past the last pencil.
+__device__ __forceinline__ long long fx_green_base(const PassParams& p, int q, int o) {
   const FusedGreen& g = p.g;
-  *goff = 0;
-  *gexp = -(1 << 20);
-  if (q >= p.npen) return;
+  if (q >= p.npen) return 0;
   int c[3];
   if (p.axis == 0) { c[1] = q % g.dims1; c[2] = q / g.dims1; c[0] = 0; }
   else if (p.axis == 1) { c[0] = q; c[2] = o; c[1] = 0; }
   else { c[0] = q; c[1] = o; c[2] = 0; }
   const long long st[3] = {1, (long long)g.gpitch, (long long)g.gpitch * g.gext[1]};
-  long long off = 0, e = 0, es = 1;
+  long long off = 0;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     if (d == p.axis) continue;
     int gi = c[d];
     if (g.fold[d]) gi = min(gi, g.fold[d] - gi);
     off += gi * st[d];
-    e += gi * es;
-    es *= g.gext[d];
   }
-  *goff = off;
-  *gexp = g.gexp[e];
+  return off;
 }
+
+// Green products of a complex lane in the first inverse stage: u^ = G^ f^.  g: the lane's factors by folded mode, gs
+// apart, in the staged slice or in the stored spectrum; up: the modes' renormalisation.
+template <int P, class RW> struct FxGained {
+  const cfx* S;
+  const unsigned long long* g;
+  long long gs;
+  int up;
+  // factor of position j + r nbf: its own mode in the lower half, the mirrored one in the upper
+  template <int R, int nbf, class F> __device__ __forceinline__ void each(int j, F f) const {
+    const unsigned long long *lo = g + j * gs, *hi = g + (P - j) * gs;
+    const long long step = nbf * gs;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const bool low = 2 * (r + 1) <= R || (2 * r < R && 2 * (j + r * nbf) <= P);
+      f(r, low ? lo + r * step : hi - r * step);
+    }
+  }
+  template <int R, int nbf> __device__ __forceinline__ int products(ic<R>, ic<nbf>, int j, int l, cfx* v) const {
+    FxFromS<RW>{S}(ic<R>(), ic<nbf>(), j, l, v);
+    int top = 0;
+    each<R, nbf>(j, [&](int r, const unsigned long long* f) {
+      const fxg q = fx_green(*f);
+      v[r] = fx_make(fx_mul(v[r].x << up, q.h, q.l), fx_mul(v[r].y << up, q.h, q.l));
+      top = max(top, fx_top_bit(v[r], q.d));
+    });
+    return top;
+  }
+  // (the orders are read again: kept, they would take a register per value)
+  template <int R, int nbf> __device__ __forceinline__ void align(ic<R>, ic<nbf>, int j, int T, cfx* v) const {
+    each<R, nbf>(j, [&](int r, const unsigned long long* f) {
+      v[r] = fx_align(v[r], *reinterpret_cast<const int*>(f) & kFxGreenRange, T);
+    });
+  }
+};
 
 // Load of real data pairs whose extension is built in the tile (symmetric and semi-unbounded directions, and
 // every real pass on pinned host arrays): items (lane, i < n_data), at most U per thread.  Values that the extension
@@ -455,7 +489,7 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
   unsigned* emax = reinterpret_cast<unsigned*>(m.emax);
   const bool tma_g = FUSED && p.gpre && p.gmap;
   if constexpr (FUSED) {
-    for (int l = tid; l < (REAL ? 2 * W : W); l += nt) fx_green_base(p, q0 + l, o, &m.goff[l], &m.gexp[l]);
+    for (int l = tid; l < (REAL ? 2 * W : W); l += nt) m.goff[l] = fx_green_base(p, q0 + l, o);
     if (tma_g && tid == 0) mbar_init(m.mbar, 1);
   }
   __syncthreads();
@@ -587,48 +621,61 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
   } else if constexpr (KIND == K_FUSED_REAL) {
     fx_forward_real<P, RW, true>(p, t, type, (const double*)p.in + bi, q0, m.emax, wf);
     const bool quarter = is_quarter(base_type(type));
-    unsigned mo = 0;
     {
+      // the two pencils' products in place of the packed modes k and P - k, then, aligned, packed again
       const int l = tid & (W - 1), upx = fx_free_tw(wf[(ns - 1) * W + l]);
-      const long long ga = m.goff[2 * l], gb = m.goff[2 * l + 1];
-      const int ea = m.gexp[2 * l], eb = m.gexp[2 * l + 1], e = max(ea, eb);
-      const int sa = min(e - ea, 62), sb = min(e - eb, 62);
       const long long st3 = p.axis == 0 ? 1 : (p.axis == 1 ? (long long)p.g.gpitch : (long long)p.g.gpitch * p.g.gext[1]);
-      const long long* G = (const long long*)p.g.stored;
+      const unsigned long long* Ga = (const unsigned long long*)p.g.stored + m.goff[2 * l];
+      const unsigned long long* Gb = (const unsigned long long*)p.g.stored + m.goff[2 * l + 1];
+      int top = 0;
       for (int k = tid >> p.lw; k <= half; k += nt >> p.lw) {
+        if (quarter && !(k & 1)) continue;
         const int km = k == 0 ? 0 : P - k;
         cfx zk = S[RW::at(k) + l], zm = S[RW::at(km) + l];
         zk = fx_make(zk.x << upx, zk.y << upx);
         zm = fx_make(zm.x << upx, zm.y << upx);
+        const long long o3 = (quarter ? (k - 1) >> 1 : k) * st3;
+        const fxg fa = fx_green(__ldg(&Ga[o3])), fb = fx_green(__ldg(&Gb[o3]));
+        const cfx A = fx_make(fx_mul(zk.x + zm.x, fa.h, fa.l), fx_mul(zk.y - zm.y, fa.h, fa.l));
+        const cfx B = fx_make(fx_mul(zk.y + zm.y, fb.h, fb.l), fx_mul(zm.x - zk.x, fb.h, fb.l));
+        top = max(top, max(fx_top_bit(A, fa.d), fx_top_bit(B, fb.d)));
+        // modes 0 and P/2 are real
+        if (km == k) {
+          S[RW::at(k) + l] = fx_make(A.x, B.x);
+        } else {
+          S[RW::at(k) + l] = A;
+          S[RW::at(km) + l] = B;
+        }
+      }
+      lane_top(wg, top, W, l, tid);
+      __syncthreads();
+      const int T = (int)wg[l];
+      for (int k = tid >> p.lw; k <= half; k += nt >> p.lw) {
+        const int km = k == 0 ? 0 : P - k;
         cfx A = fx_make(0, 0), B = A;
         if (!quarter || (k & 1)) {
-          const int g3 = quarter ? (k - 1) >> 1 : k;
-          const long long va = __ldg(&G[ga + g3 * st3]), vb = __ldg(&G[gb + g3 * st3]);
-          const int ah = (int)(va >> 32), al = (int)va, bh = (int)(vb >> 32), bl = (int)vb;
-          A = fx_make(fx_shr(fx_mul(zk.x + zm.x, ah, al), sa), fx_shr(fx_mul(zk.y - zm.y, ah, al), sa));
-          B = fx_make(fx_shr(fx_mul(zk.y + zm.y, bh, bl), sb), fx_shr(fx_mul(zm.x - zk.x, bh, bl), sb));
+          const long long o3 = (quarter ? (k - 1) >> 1 : k) * st3;
+          A = S[RW::at(k) + l];
+          if (km == k) {
+            B.x = A.y;
+            A.y = 0;
+          } else {
+            B = S[RW::at(km) + l];
+          }
+          A = fx_align(A, (int)__ldg(&Ga[o3]) & kFxGreenRange, T);
+          B = fx_align(B, (int)__ldg(&Gb[o3]) & kFxGreenRange, T);
         }
-        const cfx zp = fx_make(A.x - B.y, A.y + B.x), zq = fx_make(A.x + B.y, B.x - A.y);
-        mo |= fx_mag(zp.x) | fx_mag(zp.y) | fx_mag(zq.x) | fx_mag(zq.y);
-        S[RW::at(k) + l] = zp;
-        if (k != 0 && 2 * k != P) S[RW::at(km) + l] = zq;
+        S[RW::at(k) + l] = fx_make(A.x - B.y, A.y + B.x);
+        if (km != k) S[RW::at(km) + l] = fx_make(A.x + B.y, B.x - A.y);
       }
-      lane_or(wg, mo, W, l, tid);
     }
     __syncthreads();
-    const int up = fx_free_in(wg[tid & (W - 1)]);
-    fx_stage<P, R0, 1, true, FX_TILE, true, 0>(
-        t, nullptr, wi,
-        [=](auto R, auto nbf, int j, int l, cfx* v) {
-          from_s(R, nbf, j, l, v);
-#pragma unroll
-          for (int r = 0; r < R.value; ++r) v[r] = fx_make(v[r].x << up, v[r].y << up);
-        },
-        to_s);
+    fx_stage<P, R0, 1, true, FX_TILE, true, 0>(t, nullptr, wi, from_s, to_s);
     fx_mid_stages<P, RW, true, false, 1, ns - 1>(t, wi);
     fx_store_real<P, RW>(p, t, type, (double*)p.out + bo, q0, wi, [&](int lane, int* q, int* kind) {
       const int Ee = max(m.emax[lane], kFxMinE);
-      *q = Ee - fx_shifted<P>(m.words, W, lane, true, true, true) + 2 * shift + kFxBias - 1 + 64 + max(m.gexp[2 * lane], m.gexp[2 * lane + 1]);
+      *q = Ee - fx_shifted<P>(m.words, W, lane, true, true, true) + 2 * shift + kFxBias - 1 +
+           fx_align_exp((int)wg[lane], *p.g.gref);
       *kind = fx_out_kind(Ee, *q);
     });
   } else {
@@ -679,28 +726,12 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
       }
       const long long go = m.goff[l0];
       const long long st3 = p.axis == 0 ? 1 : (p.axis == 1 ? (long long)p.g.gpitch : (long long)p.g.gpitch * p.g.gext[1]);
-      const long long* G = (const long long*)p.g.stored + go;
-      const long long* Gs = m.G;
-      const int upx = fx_free_tw(wf[(ns - 1) * W + l0]);
-      auto gained = [=](auto R, auto nbf, int j, int l, cfx* v) {
-        from_s(R, nbf, j, l, v);
-        // folded mode of position i = j + r nbf: i in the lower half, P - i in the upper one
-        const long long* g = tma_g ? Gs + l : G;
-        const long long gs = tma_g ? (long long)W : st3;
-        const long long *lo = g + j * gs, *hi = g + (P - j) * gs;
-        const long long step = nbf.value * gs;
-#pragma unroll
-        for (int r = 0; r < R.value; ++r) {
-          const bool low = 2 * (r + 1) <= R.value || (2 * r < R.value && 2 * (j + r * nbf.value) <= P);
-          const long long x = low ? lo[r * step] : hi[-(r * step)];
-          const int gh = (int)(x >> 32), gl = (int)x;
-          v[r] = fx_make(fx_mul(v[r].x << upx, gh, gl), fx_mul(v[r].y << upx, gh, gl));
-        }
-      };
+      const FxGained<P, RW> gained{S, tma_g ? m.G + l0 : (const unsigned long long*)p.g.stored + go,
+                                   tma_g ? (long long)W : st3, fx_free_tw(wf[(ns - 1) * W + l0])};
       fx_stage<P, RL, 1, true, FX_GAIN, true, 0>(t, wg, wi, gained, to_s);
       fx_mid_stages<P, RW, true, true, 1, ns - 1>(t, wi);
       const int E = max(m.emax[l0], kFxMinE);
-      q = E - fx_shifted<P>(m.words, W, l0, true, true, true) + 2 * shift + kFxBias + 64 + m.gexp[l0];
+      q = E - fx_shifted<P>(m.words, W, l0, true, true, true) + 2 * shift + kFxBias + fx_align_exp((int)wg[l0], *p.g.gref);
       kind = fx_out_kind(E, q);
       fx_stage<P, R0, P / R0, true, FX_TILE, false, ns - 1>(t, nullptr, wi, from_s, store);
     } else {

@@ -24,7 +24,6 @@
 
 #include <algorithm>
 
-
 #include "fx64.cuh"
 #include "green.cuh"
 
@@ -548,45 +547,21 @@ __global__ void k_green_finalize_df(const double* __restrict__ g, float2* __rest
   }
 }
 
-// Fixed-point storage for the FP64-class passes: every pencil along `axis` is aligned to its largest
-// value (|g| < 2^(53 + up)), its exponent kept beside (value = g 2^gexp).  A block takes 32 pencils, its 8 rows of
-// threads a part of the axis each; along x a warp reads one pencil after the other.  Bound by the latency of its
-// loads: one thread per pencil had 74 blocks of 128 for 49 x 193 pencils of 97 and took 36.8 us, this 13.6.
-__global__ void __launch_bounds__(256) k_green_finalize_fx(const double* __restrict__ g, long long* __restrict__ out,
-                                                           int* __restrict__ gexp, int gx, int gy, int gz, int gp,
-                                                           int axis, double scale, int up) {
-  __shared__ unsigned mx[32];
-  const int n0 = axis == 0 ? gy : gx, n1 = axis == 2 ? gy : gz, n = axis == 0 ? gx : (axis == 1 ? gy : gz);
-  const long long first = blockIdx.x * 32ll, tot = (long long)n0 * n1;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  if (threadIdx.x < 32) mx[threadIdx.x] = 0;
-  __syncthreads();
-  // thread (tx, ty): pencil tx, elements ty, ty + 8, ...; along x: pencils ty, ty + 8, ..., elements tx, tx + 32, ...
-  for (int pass = 0; pass < 2; ++pass) {
-    for (int q = axis == 0 ? ty : tx; q < 32; q += axis == 0 ? 8 : 32) {
-      const long long i = first + q;
-      if (i >= tot) continue;
-      const int a = (int)(i % n0), b = (int)(i / n0);
-      long long src, dst, ss, ds;
-      if (axis == 0) { src = (long long)gx * (a + (long long)gy * b); dst = (long long)gp * (a + (long long)gy * b); ss = ds = 1; }
-      else if (axis == 1) { src = a + (long long)gx * gy * b; dst = a + (long long)gp * gy * b; ss = gx; ds = gp; }
-      else { src = a + (long long)gx * b; dst = a + (long long)gp * b; ss = (long long)gx * gy; ds = (long long)gp * gy; }
-      const int k0 = axis == 0 ? tx : ty, dk = axis == 0 ? 32 : 8;
-      if (pass == 0) {
-        unsigned m = 0;
-        for (int k = k0; k < n; k += dk) m = max(m, (unsigned)__double2hiint(g[src + k * ss] * scale) & 0x7fffffffu);
-        atomicMax(&mx[q], m);
-      } else {
-        const int E = max((int)(mx[q] >> 20), kFxMinE);
-        for (int k = k0; k < n; k += dk)
-          out[dst + k * ds] =
-              fx_halves(fx_decode((unsigned long long)__double_as_longlong(g[src + k * ss] * scale), E, up));
-        // a pencil of zeros takes no part in a pair's common exponent
-        if (k0 == 0) gexp[i] = mx[q] ? E - 1075 - up : -(1 << 20);
-      }
-    }
-    __syncthreads();
-  }
+// Fixed-point passes: the largest biased exponent of the spectrum, then every factor's 53 bits with its binary orders
+// below it (fx_green_pack).
+__global__ void __launch_bounds__(256) k_green_top(const double* __restrict__ g, int* __restrict__ ref, long long n,
+                                                   double scale) {
+  int m = 0;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    m = max(m, (__double2hiint(g[i] * scale) >> 20) & 0x7ff);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(ref, m);
+}
+__global__ void k_green_finalize_fx(const double* __restrict__ g, unsigned long long* __restrict__ out,
+                                    const int* __restrict__ ref, long long n, int gx, int gp, double scale) {
+  const int top = *ref;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    out[(i / gx) * gp + i % gx] = fx_green_pack((unsigned long long)__double_as_longlong(g[i] * scale), top);
 }
 
 // Fully spectral kernels evaluated in FP64 (stored spectrum of the double-float path):
@@ -689,12 +664,13 @@ cudaError_t launch_green_finalize(const double* g, void* out, int prec, long lon
   return cudaGetLastError();
 }
 
-cudaError_t launch_green_finalize_fx(const double* g, void* out, int* gexp, const int* gext, int gp, int axis,
-                                     double scale, bool real_fused, cudaStream_t st) {
-  const long long n = (long long)gext[axis == 0 ? 1 : 0] * gext[axis == 2 ? 1 : 2];
-  k_green_finalize_fx<<<(unsigned)((n + 31) / 32), 256, 0, st>>>(
-      g, (long long*)out, gexp, gext[0], gext[1], gext[2], gp, axis, scale,
-      (real_fused ? kFxGreenBitsReal : kFxGreenBits) - 53);
+cudaError_t launch_green_finalize_fx(const double* g, void* out, int* ref, long long n, int gx, int gp, double scale,
+                                     cudaStream_t st) {
+  const long long blocks = std::min<long long>((n + 255) / 256, 152 * 16);
+  const cudaError_t e = cudaMemsetAsync(ref, 0, sizeof(int), st);
+  if (e) return e;
+  k_green_top<<<(unsigned)blocks, 256, 0, st>>>(g, ref, n, scale);
+  k_green_finalize_fx<<<(unsigned)blocks, 256, 0, st>>>(g, (unsigned long long*)out, ref, n, gx, gp, scale);
   return cudaGetLastError();
 }
 

@@ -29,10 +29,9 @@ void host_gauss_legendre(int n, double* x, double* w);
 // out[(i / gx) gp + i % gx] = g[i] scale in the path precision (x rows of gx values at pitch gp)
 cudaError_t launch_green_finalize(const double* g, void* out, int prec, long long n, int gx, int gp, double scale,
                                   cudaStream_t st);
-// the same for the fixed-point passes: pencils along `axis` with their exponents (gexp, over the other two
-// extents, lower direction fastest); real_fused: the fused pass is a real one
-cudaError_t launch_green_finalize_fx(const double* g, void* out, int* gexp, const int* gext, int gp, int axis,
-                                     double scale, bool real_fused, cudaStream_t st);
+// the same for the fixed-point passes (fx_green_pack); *ref receives the spectrum's largest biased exponent
+cudaError_t launch_green_finalize_fx(const double* g, void* out, int* ref, long long n, int gx, int gp, double scale,
+                                     cudaStream_t st);
 cudaError_t launch_green_spectral(double* g, const int* gext, const double* const* tabs, int kernel, double eps2h,
                                   double scale, cudaStream_t st);
 cudaError_t launch_special_eval(int which, const double* x, const double* y, double* out, int n, double eps,

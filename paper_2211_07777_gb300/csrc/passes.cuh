@@ -36,8 +36,7 @@ struct FusedGreen {
   const void* stored;     // stored real spectrum (path precision) or nullptr for closed form
   const void* tab[3];     // closed form: per-direction |w|^2 (or FD symbol) tables, path precision
   int gext[3];            // Green index extents (x, y, z)
-  const int* gexp;        // fixed-point spectrum (FP64-class Poisson passes): exponent of each pencil's slice
-                          // along the fused axis, over the other two Green extents (lower direction fastest)
+  const int* gref;        // fixed-point factors: the spectrum's largest biased exponent
   int gpitch;             // x pitch of the stored spectrum (elements): gext[0] rounded up to 16 bytes
   int fold[3];            // green index = fold ? min(i, fold - i) : i, for the two non-axis dirs
   int kernel;             // closed-form kernel id (0 spectral, 2..10 HEJ order, 100 LGF2)

@@ -62,7 +62,6 @@ int main() {
     unsigned long long b;
     std::memcpy(&b, &d, 8);
     wd = std::fmax(wd, std::fabs(ldexpl(d, kFxBias - E) - (ld)fx_decode(b, E)));
-    if (fx_halves(x.x) != (long long)(((unsigned long long)(unsigned)fx_hi(x.x) << 32) | (unsigned)fx_lo(x.x))) return 1;
     if ((ld)fx_hi(x.x) * 0x1p32L + fx_lo(x.x) != (ld)x.x) return 1;
   }
   std::printf("cmul %.3Lg\nmul %.3Lg\ndecode %.4Lg\n", wc, wm, wd);
@@ -89,6 +88,44 @@ int main() {
       else worst = std::fmax(worst, std::fabs(sum) / n - (d > up ? ldexpl(0.5L, up - d) : 0));
     }
   std::printf("decode_all %.4Lg\ndecode_mean %.3Lg\ndecode_binade %.3Lg\n", wd, all, worst);
+  // Green products: factors over 60 binary orders with modes over 60, the larger product of a pair aligned to 57 bits
+  ld wg = 0, wa = 0;
+  for (int t = 0; t < 100000; ++t) {
+    cfx p[2];
+    ld want[2];
+    int d[2], T = 0;
+    const int ref = 1023;
+    for (int i = 0; i < 2; ++i) {
+      const double g = std::ldexp((double)uni(), (int)(30 * uni()) - 40);
+      const long long x = (long long)(0x1.69p62L * uni() * std::pow((ld)2, 30 * (uni() - 1)));
+      unsigned long long b;
+      std::memcpy(&b, &g, 8);
+      const fxg q = fx_green(fx_green_pack(b, ref));
+      if (ldexpl((ld)q.h * 0x1p32L + q.l, ref - q.d - 1075 - kFxGreenUp) != (ld)g) return 7;
+      p[i] = fx_make(fx_mul(x, q.h, q.l), fx_mul(-x / 2, q.h, q.l));
+      d[i] = q.d;
+      want[i] = (ld)x * g;
+      wg = std::fmax(wg, std::fabs(ldexpl(want[i], 1075 + kFxGreenUp - 64 - ref + d[i]) - p[i].x));
+      const int b2 = fx_top_bit(p[i], d[i]);
+      T = b2 > T ? b2 : T;
+    }
+    cfx a[2];
+    for (int i = 0; i < 2; ++i) {
+      a[i] = fx_align(p[i], d[i], T);
+      // error of the alignment alone, in units of the aligned values
+      wa = std::fmax(wa, std::fabs(ldexpl((ld)p[i].x, kFxAligned + kFxGreenRange - d[i] - T) - a[i].x));
+      if (std::fabs(ldexpl(want[i], -fx_align_exp(T, ref)) - a[i].x) > 0x1p26L) return 12;  // a unit of a 31-bit product at most
+      if (std::llabs(a[i].x) > 1LL << kFxAligned || std::llabs(a[i].y) > 1LL << kFxAligned) return 8;
+    }
+    // a product of 33 bits or more reaches the top
+    if (std::llabs(p[0].x) >= 1LL << 33 && std::llabs(p[1].x) >= 1LL << 33 && std::llabs(a[0].x) < 1LL << (kFxAligned - 2) &&
+        std::llabs(a[1].x) < 1LL << (kFxAligned - 2))
+      return 9;
+  }
+  const fxg z = fx_green(fx_green_pack(0, 1000)), sb = fx_green(fx_green_pack(0x800fffffffffffffull, 1000));
+  if (z.h || z.l || sb.h || sb.l || z.d != kFxGreenRange) return 10;
+  if (fx_align(fx_make(0, 0), 0, fx_top_bit(fx_make(0, 0), 0)).x != 0) return 11;
+  std::printf("green %.3Lg\nalign %.3Lg\n", wg, wa);
   std::printf("zero %lld\nsubnormal %lld\n", fx_decode(0, kFxMinE), fx_decode(0x800fffffffffffffull, kFxMinE));
   std::printf("shr_even %lld\n", fx_shr(24, 4) * 100 + fx_shr(8, 4) * 10 + fx_shr(7, 0));  // 1.5 -> 2, 0.5 -> 0, 7
   // every plan multiplies to its length within the block limits

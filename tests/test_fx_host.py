@@ -44,6 +44,11 @@ def test_products_and_decoding(errors):
     assert errors["shr_even"] == 207
 
 
+def test_green_products_keep_their_own_exponent(errors):
+    assert errors["green"] < 1.0     # half a unit and the dropped low product (a quarter), of each product's own unit
+    assert errors["align"] <= 0.5    # one rounding at the scale of the lane's largest product
+
+
 def test_decoding_has_no_preferred_direction(errors):
     """Mean error over 100000 positive values, uniform and at each distance below the lane's largest: truncation has half
     a unit, rounding to nearest a standard error of 0.3 / sqrt(100000) = 0.001 and the ties' bias, in all 2^-5 / 4 +
