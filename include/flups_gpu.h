@@ -125,10 +125,12 @@ int flups_host_mapped(const void* host, size_t bytes);
 
 /* Releases the plan, the Green spectrum and the workspace (twiddle tables
  * are shared by all solvers of the process and kept until exit).  The
- * caller's arrays are never freed.  Safe on NULL.  flups_cleanup frees
- * synchronously; flups_cleanup_async frees in stream order on `stream`
- * without synchronising the device, and requires that no work using the
- * solver is still pending on other streams. */
+ * caller's arrays are never freed.  Safe on NULL.  flups_cleanup frees at
+ * once and waits for nothing: the caller makes sure that every solve is over
+ * (its stream synchronised; flups_solve_host returns after that) and that no
+ * graph with the solver's kernels is launched again.  flups_cleanup_async
+ * frees in stream order on `stream` without synchronising the device, and
+ * requires that no work using the solver is still pending on other streams. */
 int flups_cleanup(flups_solver s);
 int flups_cleanup_async(flups_solver s, void* stream);
 

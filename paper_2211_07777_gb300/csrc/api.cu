@@ -1681,8 +1681,8 @@ int flups_solve_host(flups_solver s, void* phi_host, const void* rhs_host, void*
   return FLUPS_OK;
 }
 
-// Frees the solver's own device buffers on `st` (stream-ordered) or, with
-// st == nullptr, synchronously.  Twiddle tables are shared and stay.
+// Frees the solver's own device buffers in stream order on `st` or at once.  cudaFree does not wait for kernels that
+// use stream-ordered memory, so the caller has waited for every solve.  Twiddle tables are shared and stay.
 static void release(flups_solver s, cudaStream_t st, bool async) {
   auto fr = [&](void* p) {
     if (!p) return;

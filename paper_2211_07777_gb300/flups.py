@@ -145,6 +145,26 @@ def _stream(s) -> int:
     return s.cuda_stream
 
 
+def _held(stream):
+    """The stream as an object that can be waited for later (None: the current device's legacy default stream)."""
+    if stream is None:
+        import torch
+        return torch.cuda.default_stream()
+    return stream
+
+
+def _wait(stream):
+    """Waits for the work on a stream.  A bare handle may have been destroyed meanwhile: the device is waited for.
+    Under stream capture nothing can be waited for."""
+    import torch
+    if torch.cuda.is_initialized() and torch.cuda.is_current_stream_capturing():
+        return
+    if hasattr(stream, "synchronize"):
+        stream.synchronize()
+    else:
+        torch.cuda.synchronize()
+
+
 # --- the C ABI, one function each -------------------------------------------------
 def flups_init_topo(n, center, ncomp, prec):
     h = ctypes.c_void_p()
@@ -397,17 +417,25 @@ class Solver:
             raise
         if share_green:
             _check(lib().flups_solver_share_green(self._s), "flups_solver_share_green")
+        self._streams = {}
         self.workspace_bytes = flups_setup(self._s, stream)
         self.info = flups_solver_info(self._s)
 
+    def _on(self, stream):
+        """Remembers a stream that the solver's kernels run on: close() waits for it."""
+        handle = _stream(stream)
+        if handle not in self._streams:
+            self._streams[handle] = _held(stream)
+        return stream
+
     def solve(self, phi, rhs, stream=None):
-        flups_solve(self._s, phi, rhs, stream)
+        flups_solve(self._s, phi, rhs, self._on(stream))
 
     def solve_pass(self, i, phi, rhs, stream=None):
-        flups_solve_pass(self._s, i, phi, rhs, stream)
+        flups_solve_pass(self._s, i, phi, rhs, self._on(stream))
 
     def solve_events(self, phi, rhs, events, stream=None):
-        flups_solve_events(self._s, phi, rhs, events, stream)
+        flups_solve_events(self._s, phi, rhs, events, self._on(stream))
 
     def pass_info(self, i):
         return flups_pass_info(self._s, i)
@@ -443,7 +471,10 @@ class Solver:
         self.close()
 
     def close(self):
+        """Frees the plan once the solves on its streams are over (flups_cleanup waits for nothing)."""
         if getattr(self, "_s", None) is not None:
+            for stream in getattr(self, "_streams", {}).values():
+                _wait(stream)
             flups_cleanup(self._s)
             self._s = None
         if getattr(self, "_topo", None) is not None:

@@ -135,3 +135,32 @@ def test_plan_order_matches_the_oracle_for_every_type_triple(lib):
     import oracle
     for types in itertools.product(list(_FACES), repeat=3):
         assert _plan_order(lib, types) == tuple(oracle.direction_order(types)), types
+
+
+def test_closing_a_solver_waits_for_the_streams_of_its_solves(lib, monkeypatch):
+    """The plan's memory is freed only after the solves on every stream that it was used on (and on the legacy default
+    stream, given as None)."""
+    log = []
+
+    class Stream:
+        def __init__(self, handle):
+            self.cuda_stream = handle
+
+        def synchronize(self):
+            log.append(("wait", self.cuda_stream))
+
+    monkeypatch.setattr(lib, "_held", lambda st: Stream(0) if st is None else st, raising=False)
+    monkeypatch.setattr(lib, "flups_solve", lambda s, phi, rhs, stream: log.append(("solve", lib._stream(stream))))
+    monkeypatch.setattr(lib, "flups_cleanup", lambda s: log.append(("free",)))
+    monkeypatch.setattr(lib, "flups_topo_free", lambda t: None)
+    s = object.__new__(lib.Solver)
+    s._s, s._topo, s._streams = 1, 1, {}
+    a, b = Stream(7), Stream(8)
+    for st in (a, b, a, None):
+        s.solve(None, None, st)
+    s.close()
+    assert log[:4] == [("solve", 7), ("solve", 8), ("solve", 7), ("solve", 0)]
+    assert sorted(log[4:7]) == [("wait", 0), ("wait", 7), ("wait", 8)]
+    assert log[7:] == [("free",)]
+    s.close()
+    assert len(log) == 8

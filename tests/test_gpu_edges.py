@@ -76,3 +76,28 @@ def test_longest_column_transform(prec):
     f, ref = _LONG["case"]
     out, _ = cuda_solve(f, bc, CELL, prec, "hej2")
     assert rel_linf(out, ref) < TOL[prec], rel_linf(out, ref)
+
+
+@pytest.mark.parametrize("side", [False, True], ids=["default-stream", "side-stream"])
+def test_a_solver_closed_at_once_finishes_its_solves(side):
+    """close() right after the launches: the next plan takes over the freed memory, and the results stand."""
+    import torch
+    n = (128, 128, 128)
+    f = torch.from_numpy(np.random.default_rng(9).standard_normal(n)).cuda()
+    bc = ((U, U),) * 3
+    stream = torch.cuda.Stream() if side else None
+    want = torch.empty_like(f)
+    with F.Solver(n, bc, prec=F.F64, green="hej2") as s:
+        s.solve(want, f)
+        torch.cuda.synchronize()
+    out = [torch.empty_like(f) for _ in range(8)]
+    torch.cuda.synchronize()
+    s = F.Solver(n, bc, prec=F.F64, green="hej2")
+    for o in out:
+        s.solve(o, f, stream)
+    s.close()
+    with F.Solver(n, bc, prec=F.F64, green="hej4") as other:
+        other.solve(torch.empty_like(f), f)
+        torch.cuda.synchronize()
+    for o in out:
+        assert torch.equal(o, want)
