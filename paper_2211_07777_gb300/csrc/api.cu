@@ -151,6 +151,8 @@ struct flups_solver_s {
   int green_pitch = 0;          // x pitch (elements) of the stored spectrum
   bool fx = false;              // every pass in 64-bit fixed point (FP64-class Poisson solves)
   bool fxp = false;             // the passes of the first two directions are (Biot-Savart solves too)
+  bool eval_green = false;      // fixed point, fully spectral: the fused pass evaluates the closed form (no stored spectrum)
+  int green_top = 0;            // its reference exponent, and that of a stored closed form
   bool share_green = false;     // look the stored spectrum up in (and add it to) the process-wide cache
   std::string green_key;        // its cache key when shared
   void* gmaps_dev = nullptr;    // TMA tensor maps of the stored spectrum (fused column pass)
@@ -565,11 +567,34 @@ cudaError_t sample_green(const flups_solver_s* s, const GreenSampleParams& q, do
   return (s->green == FLUPS_LGF2) ? launch_lgf(g64, q.gext, q.h, st) : launch_green_sample(g64, q, st);
 }
 
-// Bytes of the stored spectrum: rows at green_pitch and, for the fixed-point passes, a block with its reference exponent.
+bool fully_spectral(const flups_solver_s* s) { return !s->dir[0].unb && !s->dir[1].unb && !s->dir[2].unb; }
+
+// Bytes of the stored spectrum: rows at green_pitch and, where the fixed-point passes have their reference exponent from
+// the device, a block with it.
 size_t green_stored_bytes(const flups_solver_s* s) {
-  return (size_t)s->green_pitch * s->dir[1].gext * s->dir[2].gext * esize(s->topo.prec) + (s->fx ? 16 : 0);
+  return (size_t)s->green_pitch * s->dir[1].gext * s->dir[2].gext * esize(s->topo.prec) +
+         (s->fx && !fully_spectral(s) ? 16 : 0);
 }
-int* green_ref(const flups_solver_s* s) { return (int*)((char*)s->green_dev + green_stored_bytes(s) - 16); }
+int* green_ref(const flups_solver_s* s) {
+  return s->fx && !fully_spectral(s) ? (int*)((char*)s->green_dev + green_stored_bytes(s) - 16) : nullptr;
+}
+int top_exponent(double v) {
+  int e = 0;
+  std::frexp(v, &e);
+  return std::min(std::max(e + 1022, 1), 2046);
+}
+
+// Whether a fully spectral fixed-point plan may hold its spectrum: a large one (the smaller are nothing beside a
+// context's own memory) leaves room for the caller's two arrays.  Evaluating it in the pass needs no memory.
+bool room_for_spectrum(const flups_solver_s* s, size_t bytes) {
+  if (bytes < ((size_t)64 << 20)) return true;
+  size_t avail = 0, total = 0;
+  if (cudaMemGetInfo(&avail, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return avail >= bytes + 2 * (size_t)s->topo.n[0] * s->topo.n[1] * s->topo.n[2] * s->topo.ncomp * sizeof(double);
+}
 
 // The spectrum g64 times scale into green_dev, in the passes' format.
 cudaError_t store_green(flups_solver_s* s, const double* g64, const int* gext, double scale, cudaStream_t st) {
@@ -586,6 +611,7 @@ int setup_green_compute(flups_solver_s* s, cudaStream_t st) {
   for (int d = 0; d < 3; ++d) Pprod *= s->dir[d].P;
   if (du == 0) {
     // closed form on the fly: per-direction |w|^2 (or the 7-point FD symbol for LGF2)
+    double k2min = 0.0, k2step = 1e300;
     for (int d = 0; d < 3; ++d) {
       const DirPlan& dp = s->dir[d];
       std::vector<double> tab(dp.gext);
@@ -598,6 +624,8 @@ int setup_green_compute(flups_solver_s* s, cudaStream_t st) {
           tab[g] = w * w;
         }
       }
+      k2min += tab[0];
+      k2step = std::min(k2step, tab[1] - tab[0]);
       const size_t bytes = dp.gext * esize(prec);
       CK(cudaMallocAsync(&s->tabs[d], bytes, st));
       if (prec == FLUPS_F32) {
@@ -610,18 +638,42 @@ int setup_green_compute(flups_solver_s* s, cudaStream_t st) {
       }
       s->ws_bytes += bytes;
     }
-    if (prec == FLUPS_F64E || s->fx) {
-      // these passes read a stored spectrum: evaluate the closed form in FP64 once
-      int gext[3];
-      long long n = 1;
-      for (int d = 0; d < 3; ++d) {
-        gext[d] = s->dir[d].gext;
-        n *= gext[d];
+    if (!(k2min > 0.0)) k2min = k2step;  // the zero mode is left out
+    int gext[3];
+    long long n = 1;
+    for (int d = 0; d < 3; ++d) {
+      gext[d] = s->dir[d].gext;
+      n *= gext[d];
+    }
+    const double* tabs[3] = {(const double*)s->tabs[0], (const double*)s->tabs[1], (const double*)s->tabs[2]};
+    const double eps2h = 0.5 * s->eps * s->eps, scale = 1.0 / Pprod;
+    if (s->fx) {
+      // largest factor: the smallest |k|^2 above zero (every kernel falls with it)
+      s->green_top = top_exponent(2.0 * scale / k2min);  // (its rounding may carry into the next binary order)
+      s->green_pitch = (gext[0] + 1) & ~1;  // 16-byte rows
+      const size_t padded = green_stored_bytes(s);
+      if (!s->eval_green && !room_for_spectrum(s, padded)) s->eval_green = true;
+      if (!s->eval_green) {
+        const cudaError_t e = cudaMallocAsync(&s->green_dev, padded, st);
+        if (e == cudaErrorMemoryAllocation) {
+          cudaGetLastError();
+          s->green_dev = nullptr;
+          s->eval_green = true;
+        } else if (e) {
+          return cuda_fail(e, "green spectral");
+        }
       }
+      if (s->eval_green) return FLUPS_OK;
+      cudaError_t e = launch_green_spectral_fx(s->green_dev, gext, s->green_pitch, tabs, s->green, eps2h, scale, s->green_top, st);
+      if (!e) e = cudaStreamSynchronize(st);
+      if (e) return cuda_fail(e, "green spectral");
+      s->green_bytes = (double)n * 8;
+      s->ws_bytes += padded;
+    } else if (prec == FLUPS_F64E) {
+      // the double-float passes read a stored spectrum: evaluate the closed form in FP64 once
       double* g64 = nullptr;
       CK(cudaMallocAsync(&g64, n * sizeof(double), st));
-      const double* tabs[3] = {(const double*)s->tabs[0], (const double*)s->tabs[1], (const double*)s->tabs[2]};
-      cudaError_t e = launch_green_spectral(g64, gext, tabs, s->green, 0.5 * s->eps * s->eps, 1.0 / Pprod, st);
+      cudaError_t e = launch_green_spectral(g64, gext, tabs, s->green, eps2h, scale, st);
       s->green_pitch = (gext[0] + 1) & ~1;  // 16-byte rows (8-byte elements)
       const size_t padded = green_stored_bytes(s);
       if (!e) e = cudaMallocAsync(&s->green_dev, padded, st);
@@ -694,6 +746,7 @@ int setup_green_compute(flups_solver_s* s, cudaStream_t st) {
 struct GreenEntry {
   void* dev;
   int pitch;
+  int top;
   double bytes;
   size_t padded;
   int refs;
@@ -728,7 +781,7 @@ std::string green_cache_key(const flups_solver_s* s) {
 int setup_green(flups_solver_s* s, cudaStream_t st) {
   int du = 0;
   for (int d = 0; d < 3; ++d) du += s->dir[d].unb;
-  const bool stored = du > 0 || s->topo.prec == FLUPS_F64E || s->fx;
+  const bool stored = du > 0 || (s->fx ? !s->eval_green : s->topo.prec == FLUPS_F64E);
   if (!s->share_green || !stored) return setup_green_compute(s, st);
   const std::string key = green_cache_key(s);
   {
@@ -739,12 +792,13 @@ int setup_green(flups_solver_s* s, cudaStream_t st) {
       s->green_dev = it->second.dev;
       s->green_pitch = it->second.pitch;
       s->green_bytes = it->second.bytes;
+      s->green_top = it->second.top;
       s->green_key = key;
       return FLUPS_OK;
     }
   }
   const int rc = setup_green_compute(s, st);
-  if (rc || !s->green_dev) return rc;
+  if (rc || !s->green_dev) return rc;  // (no room for a spectrum: evaluated in the pass)
   std::lock_guard<std::mutex> lk(g_green_mu);
   auto it = g_green_cache.find(key);
   if (it != g_green_cache.end()) {
@@ -755,7 +809,7 @@ int setup_green(flups_solver_s* s, cudaStream_t st) {
     s->green_pitch = it->second.pitch;
   } else {
     const size_t padded = green_stored_bytes(s);
-    g_green_cache[key] = GreenEntry{s->green_dev, s->green_pitch, s->green_bytes, padded, 1};
+    g_green_cache[key] = GreenEntry{s->green_dev, s->green_pitch, s->green_top, s->green_bytes, padded, 1};
   }
   s->green_key = key;
   return FLUPS_OK;
@@ -1102,7 +1156,8 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
       }
     }
     g.stored = s->green_dev;
-    g.gref = s->fx ? green_ref(s) : nullptr;
+    g.gref = s->green_dev ? green_ref(s) : nullptr;
+    g.ref = s->green_top;
     for (int d = 0; d < 3; ++d) {
       g.tab[d] = s->tabs[d];
       g.gext[d] = s->dir[d].gext;
@@ -1122,6 +1177,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
           L.p.gmap = s->gmaps_dev;
       }
     }
+    if (L.p.fx && !g.stored) L.smem += 128 + (size_t)(real ? 2 : 1) * L.p.W * dp.gext * es;  // the slice, evaluated in the pass
     if ((L.p.fx || L.p.f2) && !curl && !real && o[2] != 0 && g.stored && dp.gext == dp.P / 2 + 1 && g.fold[0] == 0) {
       // fused column pass of the fixed-point or lane-pair kernels: the Green slice by TMA while the forward transform runs, where
       // two CTAs still fit an SM with it
@@ -1218,6 +1274,12 @@ int ensure_smem_limits() {
 
 namespace flups {
 void host_gauss_legendre(int n, double* x, double* w) { gauss_legendre(n, x, w); }
+// Before setup: the spectrum of a fully spectral fixed-point plan is evaluated in the pass (false: not such a plan).
+bool solver_evaluate_green(flups_solver s) {
+  if (s->ready || !s->fx || !fully_spectral(s)) return false;
+  s->eval_green = true;
+  return true;
+}
 }  // namespace flups
 
 extern "C" {
@@ -1490,7 +1552,9 @@ int flups_solver_memory(flups_solver s, size_t* resident, size_t* transient, siz
   }
   if (du == 0)
     for (int d = 0; d < 3; ++d) res += (size_t)s->dir[d].gext * es;
-  if (du > 0 || s->fx) {
+  if (du == 0 && s->fx) {
+    if (!s->eval_green) res += gn * es;
+  } else if (du > 0) {
     res += gn * es;
     tr += gn * sizeof(double) + (size_t)8 * 2 * gmax * sizeof(double);
     if (du == 2) tr += gn * sizeof(double) / 3;  // the sampling's Chebyshev series, at most
@@ -1537,7 +1601,7 @@ int flups_debug_green(flups_solver s, double* samples, double* spectrum, long lo
   std::vector<unsigned char> buf(rows * s->green_pitch * es);
   CK(cudaMemcpy(buf.data(), s->green_dev, buf.size(), cudaMemcpyDeviceToHost));
   int ref = 0;
-  if (s->fx) CK(cudaMemcpy(&ref, green_ref(s), sizeof(int), cudaMemcpyDeviceToHost));
+  if (green_ref(s)) CK(cudaMemcpy(&ref, green_ref(s), sizeof(int), cudaMemcpyDeviceToHost));
   // element formats: FP32, a fixed-point factor (fx_green_pack), FP64, or a pair of floats (hi, lo)
   for (size_t r = 0; r < rows; ++r)
     for (int x = 0; x < q.gext[0]; ++x) {

@@ -13,6 +13,7 @@
 
 #include "fx64.cuh"
 #include "fx_plan.cuh"
+#include "green.cuh"
 #include "pass_common.cuh"
 #include "passes.cuh"
 
@@ -32,7 +33,7 @@ struct FxSmem {
   unsigned* words;    // kFxSlots x W magnitudes (upper words ORed) behind the lanes' renormalisations
   long long* goff;    // 2 W Green offsets
   unsigned long long* mbar;
-  unsigned long long* G;  // staged slice, (P/2 + 1) x W
+  unsigned long long* G;  // staged slice: factors by folded mode and pencil
 };
 
 __device__ __forceinline__ FxSmem fx_smem(unsigned char* smraw, int W, int rows) {
@@ -247,7 +248,8 @@ __device__ __forceinline__ void fx_mid_stages(const FxTile& t, unsigned* words) 
   }
 }
 
-// Green offset (axis term excluded) of pencil q; 0 past the last pencil.
+// Green offset (axis term excluded) of pencil q, or, of a spectrum that is not stored, its partial |k|^2 (bits of a
+// double); 0 past the last pencil.
 __device__ __forceinline__ long long fx_green_base(const PassParams& p, int q, int o) {
   const FusedGreen& g = p.g;
   if (q >= p.npen) return 0;
@@ -257,14 +259,24 @@ __device__ __forceinline__ long long fx_green_base(const PassParams& p, int q, i
   else { c[0] = q; c[1] = o; c[2] = 0; }
   const long long st[3] = {1, (long long)g.gpitch, (long long)g.gpitch * g.gext[1]};
   long long off = 0;
+  double k2 = 0.0;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     if (d == p.axis) continue;
     int gi = c[d];
     if (g.fold[d]) gi = min(gi, g.fold[d] - gi);
     off += gi * st[d];
+    if (!g.stored) k2 += ((const double*)g.tab[d])[gi];
   }
-  return off;
+  return g.stored ? off : __double_as_longlong(k2);
+}
+// The tile's slice of a spectrum that is not stored: factors by folded mode, n pencils a row.
+__device__ __noinline__ void fx_green_eval(const FusedGreen& g, int axis, const long long* base, unsigned long long* G,
+                                           int n, int tid, int nt) {
+  const double* tab = (const double*)g.tab[axis];
+  for (int i = tid; i < g.gext[axis] * n; i += nt)
+    G[i] = fx_green_pack((unsigned long long)__double_as_longlong(green_spectral(
+                             __longlong_as_double(base[i % n]) + tab[i / n], g.kernel, g.eps2_half, g.scale)), g.ref);
 }
 
 // Green products of a complex lane in the first inverse stage: u^ = G^ f^.  g: the lane's factors by folded mode, gs
@@ -487,12 +499,15 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
   unsigned* wi = m.words + kFxSlotInv * W;
   unsigned* wg = m.words + kFxSlotGain * W;
   unsigned* emax = reinterpret_cast<unsigned*>(m.emax);
-  const bool tma_g = FUSED && p.gpre && p.gmap;
+  const bool tma_g = FUSED && p.gpre && p.gmap, eval_g = FUSED && !p.g.stored;
   if constexpr (FUSED) {
     for (int l = tid; l < (REAL ? 2 * W : W); l += nt) m.goff[l] = fx_green_base(p, q0 + l, o);
     if (tma_g && tid == 0) mbar_init(m.mbar, 1);
   }
   __syncthreads();
+  if constexpr (FUSED) {
+    if (eval_g) fx_green_eval(p.g, p.axis, m.goff, m.G, REAL ? 2 * W : W, tid, nt);
+  }
   if (tma_g && tid == 0) {
     const FusedGreen& g = p.g;
     const int od = p.axis == 2 ? 1 : 2;  // the direction o runs along
@@ -625,8 +640,9 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
       // the two pencils' products in place of the packed modes k and P - k, then, aligned, packed again
       const int l = tid & (W - 1), upx = fx_free_tw(wf[(ns - 1) * W + l]);
       const long long st3 = p.axis == 0 ? 1 : (p.axis == 1 ? (long long)p.g.gpitch : (long long)p.g.gpitch * p.g.gext[1]);
-      const unsigned long long* Ga = (const unsigned long long*)p.g.stored + m.goff[2 * l];
-      const unsigned long long* Gb = (const unsigned long long*)p.g.stored + m.goff[2 * l + 1];
+      const unsigned long long* Ga = eval_g ? m.G + 2 * l : (const unsigned long long*)p.g.stored + m.goff[2 * l];
+      const unsigned long long* Gb = eval_g ? Ga + 1 : (const unsigned long long*)p.g.stored + m.goff[2 * l + 1];
+      const long long gs = eval_g ? 2 * W : st3;
       int top = 0;
       for (int k = tid >> p.lw; k <= half; k += nt >> p.lw) {
         if (quarter && !(k & 1)) continue;
@@ -634,8 +650,8 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
         cfx zk = S[RW::at(k) + l], zm = S[RW::at(km) + l];
         zk = fx_make(zk.x << upx, zk.y << upx);
         zm = fx_make(zm.x << upx, zm.y << upx);
-        const long long o3 = (quarter ? (k - 1) >> 1 : k) * st3;
-        const fxg fa = fx_green(__ldg(&Ga[o3])), fb = fx_green(__ldg(&Gb[o3]));
+        const long long o3 = (quarter ? (k - 1) >> 1 : k) * gs;
+        const fxg fa = fx_green(Ga[o3]), fb = fx_green(Gb[o3]);
         const cfx A = fx_make(fx_mul(zk.x + zm.x, fa.h, fa.l), fx_mul(zk.y - zm.y, fa.h, fa.l));
         const cfx B = fx_make(fx_mul(zk.y + zm.y, fb.h, fb.l), fx_mul(zm.x - zk.x, fb.h, fb.l));
         top = max(top, max(fx_top_bit(A, fa.d), fx_top_bit(B, fb.d)));
@@ -654,7 +670,7 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
         const int km = k == 0 ? 0 : P - k;
         cfx A = fx_make(0, 0), B = A;
         if (!quarter || (k & 1)) {
-          const long long o3 = (quarter ? (k - 1) >> 1 : k) * st3;
+          const long long o3 = (quarter ? (k - 1) >> 1 : k) * gs;
           A = S[RW::at(k) + l];
           if (km == k) {
             B.x = A.y;
@@ -662,8 +678,8 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
           } else {
             B = S[RW::at(km) + l];
           }
-          A = fx_align(A, (int)__ldg(&Ga[o3]) & kFxGreenRange, T);
-          B = fx_align(B, (int)__ldg(&Gb[o3]) & kFxGreenRange, T);
+          A = fx_align(A, (int)Ga[o3] & kFxGreenRange, T);
+          B = fx_align(B, (int)Gb[o3] & kFxGreenRange, T);
         }
         S[RW::at(k) + l] = fx_make(A.x - B.y, A.y + B.x);
         if (km != k) S[RW::at(km) + l] = fx_make(A.x + B.y, B.x - A.y);
@@ -675,7 +691,7 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
     fx_store_real<P, RW>(p, t, type, (double*)p.out + bo, q0, wi, [&](int lane, int* q, int* kind) {
       const int Ee = max(m.emax[lane], kFxMinE);
       *q = Ee - fx_shifted<P>(m.words, W, lane, true, true, true) + 2 * shift + kFxBias - 1 +
-           fx_align_exp((int)wg[lane], *p.g.gref);
+           fx_align_exp((int)wg[lane], p.g.gref ? *p.g.gref : p.g.ref);
       *kind = fx_out_kind(Ee, *q);
     });
   } else {
@@ -726,12 +742,14 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
       }
       const long long go = m.goff[l0];
       const long long st3 = p.axis == 0 ? 1 : (p.axis == 1 ? (long long)p.g.gpitch : (long long)p.g.gpitch * p.g.gext[1]);
-      const FxGained<P, RW> gained{S, tma_g ? m.G + l0 : (const unsigned long long*)p.g.stored + go,
-                                   tma_g ? (long long)W : st3, fx_free_tw(wf[(ns - 1) * W + l0])};
+      const bool staged = tma_g || eval_g;
+      const FxGained<P, RW> gained{S, staged ? m.G + l0 : (const unsigned long long*)p.g.stored + go,
+                                   staged ? (long long)W : st3, fx_free_tw(wf[(ns - 1) * W + l0])};
       fx_stage<P, RL, 1, true, FX_GAIN, true, 0>(t, wg, wi, gained, to_s);
       fx_mid_stages<P, RW, true, true, 1, ns - 1>(t, wi);
       const int E = max(m.emax[l0], kFxMinE);
-      q = E - fx_shifted<P>(m.words, W, l0, true, true, true) + 2 * shift + kFxBias + fx_align_exp((int)wg[l0], *p.g.gref);
+      q = E - fx_shifted<P>(m.words, W, l0, true, true, true) + 2 * shift + kFxBias + 
+          fx_align_exp((int)wg[l0], p.g.gref ? *p.g.gref : p.g.ref);
       kind = fx_out_kind(E, q);
       fx_stage<P, R0, P / R0, true, FX_TILE, false, ns - 1>(t, nullptr, wi, from_s, store);
     } else {

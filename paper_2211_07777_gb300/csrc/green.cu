@@ -564,34 +564,23 @@ __global__ void k_green_finalize_fx(const double* __restrict__ g, unsigned long 
     out[(i / gx) * gp + i % gx] = fx_green_pack((unsigned long long)__double_as_longlong(g[i] * scale), top);
 }
 
-// Fully spectral kernels evaluated in FP64 (stored spectrum of the double-float path):
+// Fully spectral kernels evaluated in FP64 (stored spectra of the double-float and the fixed-point passes):
 // tab[d][g] holds |w_d|^2, or the 7-point symbol for LGF2; G = scale * f(sum_d tab[d][g_d]).
-__global__ void k_green_spectral(double* __restrict__ g, int gx, int gy, int gz, const double* __restrict__ t0,
-                                 const double* __restrict__ t1, const double* __restrict__ t2, int kernel,
-                                 double eps2h, double scale) {
+struct SpectralTabs {
+  const double* t[3];
+};
+template <bool FX>
+__global__ void k_green_spectral(void* __restrict__ out, int gx, int gy, int gz, int gp, SpectralTabs tab, int kernel,
+                                 double eps2h, double scale, int ref) {
   const long long tot = (long long)gx * gy * gz;
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < tot;
        idx += (long long)gridDim.x * blockDim.x) {
     const int i0 = (int)(idx % gx);
     const long long rest = idx / gx;
     const int i1 = (int)(rest % gy), i2 = (int)(rest / gy);
-    const double k2 = t0[i0] + t1[i1] + t2[i2];
-    double v = 0.0;
-    if (k2 > 0.0) {
-      if (kernel == 0 || kernel == 100) {
-        v = -1.0 / k2;
-      } else {
-        const int m = kernel / 2;
-        const double s = k2 * eps2h;
-        double acc = 1.0, term = 1.0;
-        for (int j = 1; j < m; ++j) {
-          term = term * s / j;
-          acc += term;
-        }
-        v = -exp(-s) * acc / k2;
-      }
-    }
-    g[idx] = v * scale;
+    const double v = green_spectral(tab.t[0][i0] + tab.t[1][i1] + tab.t[2][i2], kernel, eps2h, scale);
+    if (FX) ((unsigned long long*)out)[rest * gp + i0] = fx_green_pack((unsigned long long)__double_as_longlong(v), ref);
+    else ((double*)out)[rest * gp + i0] = v;
   }
 }
 
@@ -677,10 +666,17 @@ cudaError_t launch_green_finalize_fx(const double* g, void* out, int* ref, long 
 cudaError_t launch_green_spectral(double* g, const int* gext, const double* const* tabs, int kernel, double eps2h,
                                   double scale, cudaStream_t st) {
   const long long n = (long long)gext[0] * gext[1] * gext[2];
-  long long blocks = (n + 255) / 256;
-  if (blocks > 152 * 64) blocks = 152 * 64;
-  k_green_spectral<<<(unsigned)blocks, 256, 0, st>>>(g, gext[0], gext[1], gext[2], tabs[0], tabs[1], tabs[2], kernel,
-                                                     eps2h, scale);
+  const long long blocks = std::min<long long>((n + 255) / 256, 152 * 64);
+  k_green_spectral<false><<<(unsigned)blocks, 256, 0, st>>>(g, gext[0], gext[1], gext[2], gext[0],
+                                                            SpectralTabs{{tabs[0], tabs[1], tabs[2]}}, kernel, eps2h, scale, 0);
+  return cudaGetLastError();
+}
+cudaError_t launch_green_spectral_fx(void* out, const int* gext, int gp, const double* const* tabs, int kernel,
+                                     double eps2h, double scale, int ref, cudaStream_t st) {
+  const long long n = (long long)gext[0] * gext[1] * gext[2];
+  const long long blocks = std::min<long long>((n + 255) / 256, 152 * 64);
+  k_green_spectral<true><<<(unsigned)blocks, 256, 0, st>>>(out, gext[0], gext[1], gext[2], gp,
+                                                           SpectralTabs{{tabs[0], tabs[1], tabs[2]}}, kernel, eps2h, scale, ref);
   return cudaGetLastError();
 }
 

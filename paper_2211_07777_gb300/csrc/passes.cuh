@@ -36,7 +36,8 @@ struct FusedGreen {
   const void* stored;     // stored real spectrum (path precision) or nullptr for closed form
   const void* tab[3];     // closed form: per-direction |w|^2 (or FD symbol) tables, path precision
   int gext[3];            // Green index extents (x, y, z)
-  const int* gref;        // fixed-point factors: the spectrum's largest biased exponent
+  const int* gref;        // fixed-point factors: the spectrum's largest biased exponent (nullptr: it is ref)
+  int ref;
   int gpitch;             // x pitch of the stored spectrum (elements): gext[0] rounded up to 16 bytes
   int fold[3];            // green index = fold ? min(i, fold - i) : i, for the two non-axis dirs
   int kernel;             // closed-form kernel id (0 spectral, 2..10 HEJ order, 100 LGF2)

@@ -34,6 +34,12 @@
 
 #include "flups_gpu.h"
 
+namespace flups {
+// Fully spectral fixed-point plans can evaluate their spectrum in the pass instead of holding it (before setup; false:
+// not such a plan).
+bool solver_evaluate_green(flups_solver s);
+}
+
 namespace {
 
 double now_s() {
@@ -265,8 +271,9 @@ bool make_room(flups_server_s* sv, size_t need, Plan* keep) {
   return true;
 }
 
-// Host-only plan object for a request (validates it); no device memory yet.
-int new_plan(const flups_request& r, Plan** out) {
+// Host-only plan object for a request (validates it); no device memory yet.  A plan that does not fit the budget with
+// its spectrum goes without it where it can.
+int new_plan(const flups_request& r, size_t budget, Plan** out) {
   Plan* p = new (std::nothrow) Plan;
   if (!p) return FLUPS_ENOMEM;
   int rc = flups_init_topo(r.n, r.center, ncomp_of(r), r.prec, &p->topo);
@@ -274,14 +281,16 @@ int new_plan(const flups_request& r, Plan** out) {
     rc = flups_init_solver(p->topo, &r.bc[0][0][0], r.h, r.L, r.green, r.eps_over_h, r.op, r.diff, &p->solver);
   // plans of other face conditions often store the same Green spectrum: one copy for all of them
   if (rc == FLUPS_OK) rc = flups_solver_share_green(p->solver);
+  p->io = (size_t)r.n[0] * r.n[1] * r.n[2] * ncomp_of(r) * elem_bytes(r);
   if (rc == FLUPS_OK) rc = flups_solver_memory(p->solver, &p->resident, &p->transient, &p->ws);
+  if (rc == FLUPS_OK && p->resident + p->transient + p->slot_bytes() > budget && flups::solver_evaluate_green(p->solver))
+    rc = flups_solver_memory(p->solver, &p->resident, &p->transient, &p->ws);
   if (rc != FLUPS_OK) {
     if (p->solver) flups_cleanup(p->solver);
     if (p->topo) flups_topo_free(p->topo);
     delete p;
     return rc;
   }
-  p->io = (size_t)r.n[0] * r.n[1] * r.n[2] * ncomp_of(r) * elem_bytes(r);
   p->key = key_of(r);
   // setup cost ~ Green samples (the transient FP64 sample array), sampled by quadrature -- several
   // times dearer per sample -- when exactly two directions are unbounded-like
@@ -299,7 +308,7 @@ int try_start(flups_server_s* sv, Pending& pd) {
   auto it = sv->plans.find(key);
   if (it == sv->plans.end()) {
     // a new plan: reserve its memory and hand its setup to a worker; the request waits queued
-    int rc = new_plan(pd.rq, &p);
+    int rc = new_plan(pd.rq, sv->budget, &p);
     if (rc) return rc;
     const size_t need = p->resident + p->transient + p->slot_bytes();
     if (need > sv->budget) {
@@ -522,7 +531,7 @@ int flups_server_submit(flups_server sv, const flups_request* rq, const void* rh
   const std::string key = key_of(*rq);
   if (sv->plans.find(key) == sv->plans.end()) {
     Plan* p = nullptr;
-    int rc = new_plan(*rq, &p);
+    int rc = new_plan(*rq, sv->budget, &p);
     if (rc) {
       sv->st.rejected++;
       return rc;

@@ -124,6 +124,31 @@ def test_double_float_engine_in_the_mix_matches_native_fp64():
         assert np.abs(got - ref).max() <= tol * max(np.abs(ref).max(), 1e-300), r.rid
 
 
+@pytest.mark.parametrize("n,bc,kernel", [
+    ((48, 48, 48), ((F.PER, F.PER),) * 3, F.SPECTRAL),
+    ((64, 32, 27), ((F.PER, F.PER),) * 3, F.HEJ4),
+    ((32, 48, 36), ((F.EVEN, F.ODD), (F.ODD, F.ODD), (F.EVEN, F.EVEN)), F.SPECTRAL),
+    ((32, 24, 27), ((F.EVEN, F.EVEN), (F.ODD, F.ODD), (F.ODD, F.EVEN)), F.HEJ2),
+], ids=["complex", "complex-hej4", "real", "quarter-hej2"])
+def test_a_fully_spectral_plan_runs_in_the_memory_without_its_spectrum(n, bc, kernel):
+    """A budget for the workspace, the arrays and the tables alone: the request is taken, its factors are evaluated in
+    the pass, and the solution is the one with the stored spectrum to the factors' rounding."""
+    r = W.Request(rid=0, arrival_s=0.0, n=n, bc=bc, op=0, prec=F.F64, kernel=kernel)
+    half = {F.PER: lambda v: v // 2 + 1}
+    gext = [half[b[0]](v) if b[0] == F.PER else (v + 1 if b[0] == b[1] else v) for v, b in zip(n, bc)]
+    spectrum = 8 * int(np.prod(gext))
+    out = [serve.run_stream([r], budget, nstreams=1, closed_loop=True, keep={0})
+           for budget in (_need(r), _need(r) - spectrum)]
+    assert all(o["completed"] == 1 and o["errors"] == 0 for o in out)
+    assert out[0]["server"]["hbm_peak"] - out[1]["server"]["hbm_peak"] == spectrum
+    a, b = (o["outputs"][0].numpy() for o in out)
+    assert np.abs(a - b).max() <= 2e-15 * np.abs(a).max()
+    import oracle
+    ref = oracle.solve(W.request_rhs(r), oracle.Problem(bc=bc, h=tuple(1.0 / v for v in n), center=oracle.CELL,
+                                                        kernel=f"hej{kernel}" if kernel else "spectral"))
+    assert np.abs(b.reshape(ref.shape) - ref).max() <= 1e-13 * np.abs(ref).max()
+
+
 def test_admission_by_memory_queues_evicts_and_refuses():
     import torch
     U, P = F.UNB, F.PER
