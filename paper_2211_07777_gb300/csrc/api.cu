@@ -1114,6 +1114,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     L.p.ctypes = pack3(s->tf[0][o[1]], s->tf[1][o[1]], s->tf[2][o[1]]);
     if (s->fxp) fx_geom(L, s->dir[o[1]], o[1], real);
     else if (use_f2(s, L, s->dir[o[1]], o[1])) f2_geom(L, s->dir[o[1]], o[1], real);
+    if (s->fxp && !s->fx && prec == FLUPS_F64E) L.p.fx_df = 2;  // the curl's double-float array
     L.p.in = s->W1;
     L.p.out = s->W2;
     L.in_buf = 1;
@@ -1137,7 +1138,6 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     else if (use_f2(s, L, dp, o[2])) f2_geom(L, dp, o[2], real);
     L.p.in = s->W2;
     L.p.out = s->W2;
-    L.p.in_f64 = L.p.out_f64 = prec == FLUPS_F64E && s->fxp;  // between passes on FP64 arrays
     L.in_buf = 2;
     L.out_buf = 2;
     FusedGreen& g = L.p.g;
@@ -1211,6 +1211,7 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     L.p.ctypes = pack3(s->tu[0][o[1]], s->tu[1][o[1]], s->tu[2][o[1]]);
     if (s->fxp) fx_geom(L, s->dir[o[1]], o[1], real);
     else if (use_f2(s, L, s->dir[o[1]], o[1])) f2_geom(L, s->dir[o[1]], o[1], real);
+    if (s->fxp && !s->fx && prec == FLUPS_F64E) L.p.fx_df = 1;
     L.p.in = s->W2;
     L.p.out = s->W1;
     L.in_buf = 2;

@@ -299,6 +299,22 @@ FXD long long fx_decode(unsigned long long bits, int E, int up = kFxUp) {
   return ((t ^ sg) + 1) >> 1;
 }
 
+// The same for a double-float value hi + lo (hi in the lower word): both floats aligned and rounded to nearest.
+FXD long long fx_decode_float(unsigned w, int E, int up) {
+  const int e = (int)(w >> 23) & 255, sg = (int)w >> 31, s = E - e - 896;
+  const unsigned long long m = (unsigned long long)(e ? (w & 0x7fffffu) | 0x800000u : 0) << (30 + up);
+  const long long t = (long long)(m >> (s > 63 ? 63 : s));
+  return ((t ^ sg) + 1) >> 1;
+}
+FXD long long fx_decode_df(unsigned long long bits, int E, int up = kFxUp) {
+  return fx_decode_float((unsigned)bits, E, up) + fx_decode_float((unsigned)(bits >> 32), E, up);
+}
+// FP64's biased exponent of the larger float of a double-float value, from its bits without the sign
+FXD int fx_float_exp(unsigned w) {
+  const int e = (int)(w >> 23);
+  return e == 0 ? 0 : (e == 255 ? 2047 : e + 896);
+}
+
 // Green factors keep FP64's 53 bits and an exponent each: a pencil's factors fall by many orders of magnitude (1/k^2,
 // Gaussians), and modes under large factors decide the solution.  Word: the factor at 2^61 <= |g| < 2^62 in signed
 // halves, and in the low half's 9 zero bits the binary orders below the spectrum's largest exponent (`ref`); a

@@ -53,6 +53,10 @@ __device__ __forceinline__ unsigned abs_hi(double d) { return (unsigned)__double
 __device__ __forceinline__ long long dec(double d, int E, int up = kFxUp) {
   return fx_decode((unsigned long long)__double_as_longlong(d), E, up);
 }
+// a double-float value's bits; out of line, so that the passes' code stays short
+__device__ __noinline__ long long dec_df(double d, int E, int up) {
+  return fx_decode_df((unsigned long long)__double_as_longlong(d), E, up);
+}
 // FP64 value of x 2^q rounded to nearest, for results in FP64's normal range.  The conversion runs on the FP64
 // pipe (measured 1.9 per SM and clock), which is otherwise idle, and the scale joins the exponent field;
 // normalising in integers took 3 times the instructions.
@@ -65,11 +69,31 @@ __device__ __forceinline__ double enc(long long x, int q) {
 __device__ __noinline__ double enc_slow(long long x, int q, int kind) {
   return kind == 1 ? scalbn(__ll2double_rn(x), q) : __longlong_as_double(0x7ff8000000000000ll);
 }
+// the same as a double-float value (kind 3: the array of the double-float curl), hi in the lower word.  Conversions
+// between 32-bit integers and floats: the value is shifted up to 62 bits, hi takes the upper word's 24 leading bits, lo
+// the rest, at most 2^38, in steps of 2^8 (conversions of 64-bit integers run at 4.5 per SM and clock: forward pass
+// beside the curl, open 128^3, 161 us)
+__device__ __forceinline__ double enc_df(long long x, int q) {
+  const int h0 = (int)(x >> 32), z = max(__clz(h0 ^ (h0 >> 31)) - 2, 0);
+  x <<= z;
+  const int xh = fx_hi(x), xl = fx_lo(x);
+  const float a = __int2float_rn(xh);
+  const long long r = (((long long)(xh - __float2int_rz(a)) << 32) + xl + 128) >> 8;
+  const int s = min(max(q - z, -250), 190), s1 = s >> 1, s2 = s - s1;
+  const float sa = __int_as_float((s1 + 127) << 23), sb = __int_as_float((s2 + 127) << 23);
+  return __hiloint2double(__float_as_int(__int2float_rn((int)r) * sa * 256.f * sb), __float_as_int(a * sa * 4294967296.f * sb));
+}
 __device__ __forceinline__ double enc_any(long long x, int q, int kind) {
-  return __builtin_expect(kind == 0, 1) ? enc(x, q) : enc_slow(x, q, kind);
+  if (__builtin_expect(kind == 0, 1)) return enc(x, q);
+  return kind == 3 ? enc_df(x, q) : enc_slow(x, q, kind);
 }
 // 0: every |x| < 2^63 scales to a normal number (or 0); 1: not so; 2: NaN lane
 __device__ __forceinline__ int fx_out_kind(int E, int q) { return E >= 2047 ? 2 : (q > -1020 && q < 950 ? 0 : 1); }
+
+__device__ __forceinline__ int fx_store_kind(const PassParams& p, int E, int q) {
+  const int kind = fx_out_kind(E, q);
+  return (p.fx_df & 2) && kind != 2 ? 3 : kind;
+}
 
 // Largest magnitude (upper words) of the lane's inputs over the CTA, as a biased exponent; a thread's
 // inputs belong to lane `lane` = tid mod W.
@@ -94,6 +118,7 @@ struct FxTile {
   cfx* S;
   int W, lw, tid, nt;
   const fxw* tw;
+  bool df;  // FX_RAW_DF: the input array holds double-float values
 };
 // Rows of the tile are a compile-time number of values apart (FxRows), so that a butterfly's accesses are offsets
 // from one address; narrower tiles of small grids keep the stride.
@@ -127,11 +152,14 @@ template <class RW> struct FxToS {
 // again: the stage before ORs the magnitudes of its outputs' upper words per lane, the next one shifts by
 // the free bits, eight integer operations per value.  (The Green products are aligned one by one, fx_align.)  (Relative error against a 64-bit solution, mixed 256^3: 1e-13
 // to 1.7e-12 with the fixed factors alone, 4e-16 to 5e-15 with the shift from the third stage on.)
-enum FxSrc : int { FX_TILE = 0, FX_RAW = 1, FX_GAIN = 2 };
+enum FxSrc : int { FX_TILE = 0, FX_RAW = 1, FX_GAIN = 2, FX_RAW_DF = 3 };
 __device__ __forceinline__ int fx_free_tw(unsigned w) { return max(__clz(w) - 3, 0); }    // parts below 2^61
 __device__ __forceinline__ unsigned fx_mag(long long x) {
   const int h = (int)(x >> 32);
   return (unsigned)(h ^ (h >> 31));
+}
+__device__ __forceinline__ unsigned fx_mag_df(long long bits) {
+  return max((unsigned)bits & 0x7fffffffu, (unsigned)((unsigned long long)bits >> 32) & 0x7fffffffu);
 }
 __device__ __forceinline__ void lane_or(unsigned* word, unsigned m, int W, int lane, int tid) {
   for (int o = W; o < 32; o <<= 1) m |= __shfl_xor_sync(0xffffffffu, m, o);
@@ -156,7 +184,7 @@ __device__ __forceinline__ int fx_shifted(const unsigned* words, int W, int l, b
 }
 
 // One stage of radix R after a product Ns of earlier radices.  SRC: FX_RAW, In gives FP64 bits, aligned to the
-// lane's exponent (maxima in `lanes`) here; FX_GAIN, In gives Green products (FxGained) and aligns them to the lane's
+// lane's exponent (maxima in `lanes`) here, FX_RAW_DF the same or double-float values; FX_GAIN, In gives Green products (FxGained) and aligns them to the lane's
 // largest (`lanes`).  words: the transform's slots; every stage but the first is renormalised.  In and Out move whole butterflies: values
 // at positions j + r P/R, outputs at o + r Ns.
 template <int P, int R, int Ns, bool INV, int SRC, bool TO_S, int s, bool SCAN_LAST = false, class In, class Out>
@@ -179,20 +207,37 @@ __device__ __forceinline__ void fx_stage(const FxTile& t, unsigned* lanes, unsig
       for (int r = 0; r < R; ++r) v[b][r] = fx_make(0, 0);
     }
   }
-  if constexpr (SRC == FX_RAW) {
+  if constexpr (SRC == FX_RAW || SRC == FX_RAW_DF) {
+    const bool df = SRC == FX_RAW_DF && t.df;
     unsigned m = 0;
+    if (df) {
 #pragma unroll
-    for (int b = 0; b < NB; ++b)
+      for (int b = 0; b < NB; ++b)
 #pragma unroll
-      for (int r = 0; r < R; ++r)
-        m = max(m, max((unsigned)(v[b][r].x >> 32) & 0x7fffffffu, (unsigned)(v[b][r].y >> 32) & 0x7fffffffu));
+        for (int r = 0; r < R; ++r)
+          m = max(m, max(fx_mag_df(v[b][r].x), fx_mag_df(v[b][r].y)));
+      m = (unsigned)fx_float_exp(m) << 20;
+    } else {
+#pragma unroll
+      for (int b = 0; b < NB; ++b)
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          m = max(m, max((unsigned)(v[b][r].x >> 32) & 0x7fffffffu, (unsigned)(v[b][r].y >> 32) & 0x7fffffffu));
+    }
     lane_max(reinterpret_cast<int*>(lanes), m, t.W, lane, t.tid);
     __syncthreads();
     const int E = max((int)lanes[lane], kFxMinE);
+    if (df) {
 #pragma unroll
-    for (int b = 0; b < NB; ++b)
+      for (int b = 0; b < NB; ++b)
 #pragma unroll
-      for (int r = 0; r < R; ++r) v[b][r] = fx_make(fx_decode(v[b][r].x, E), fx_decode(v[b][r].y, E));
+        for (int r = 0; r < R; ++r) v[b][r] = fx_make(fx_decode_df(v[b][r].x, E), fx_decode_df(v[b][r].y, E));
+    } else {
+#pragma unroll
+      for (int b = 0; b < NB; ++b)
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[b][r] = fx_make(fx_decode(v[b][r].x, E), fx_decode(v[b][r].y, E));
+    }
   } else if constexpr (SRC == FX_GAIN) {
     lane_top(lanes, top, t.W, lane, t.tid);
     __syncthreads();
@@ -482,6 +527,7 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
   t.tid = tid;
   t.nt = nt;
   t.tw = (const fxw*)p.tw;
+  t.df = p.fx_df & 1;
   constexpr FxPlan pl = fx_plan(P);
   constexpr int ns = pl.n, half = P / 2, R0 = pl.r[0], RL = pl.r[ns - 1];
   const int W = p.W;
@@ -535,7 +581,7 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
     const int E = max(m.emax[l], kFxMinE);
     // the split leaves twice the modes; a phase costs 2^4, a quarter-wave type halves
     const int q = E + shift - fx_shifted<P>(m.words, W, l, true, false, false) - 1 + (cplx || !cell ? 0 : kFxTwShift) - (quarter ? 1 : 0);
-    const int kind = fx_out_kind(E, q);
+    const int kind = fx_store_kind(p, E, q);
     if (qa < p.npen) {
       const bool two = qa + 1 < p.npen;
       for (int k = tid >> p.lw; k < nm; k += nt >> p.lw) {
@@ -595,7 +641,14 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
           if (rb) bx[u] = in[off + p.ai.ls];
         }
       }
-      mx = max(max(mx, max(abs_hi(ax[u]), abs_hi(ay[u]))), max(abs_hi(bx[u]), abs_hi(by[u])));
+      if (!t.df) mx = max(max(mx, max(abs_hi(ax[u]), abs_hi(ay[u]))), max(abs_hi(bx[u]), abs_hi(by[u])));
+    }
+    if (t.df) {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        mx = max(max(mx, max(fx_mag_df(__double_as_longlong(ax[u])), fx_mag_df(__double_as_longlong(ay[u])))),
+                 max(fx_mag_df(__double_as_longlong(bx[u])), fx_mag_df(__double_as_longlong(by[u]))));
+      mx = (unsigned)fx_float_exp(mx) << 20;
     }
     lane_max(m.emax, mx, W, l, tid);
     if (quarter)  // even modes of the quarter-wave types are zero
@@ -609,7 +662,14 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
       const int k = (tid + u * nt) >> p.lw;
       if (k >= nm) continue;
       const int kk = quarter ? 2 * k + 1 : k;
-      cfx A = fx_make(dec(ax[u], E, up), dec(ay[u], E, up)), B = fx_make(dec(bx[u], E, up), dec(by[u], E, up));
+      cfx A, B;
+      if (t.df) {
+        A = fx_make(dec_df(ax[u], E, up), dec_df(ay[u], E, up));
+        B = fx_make(dec_df(bx[u], E, up), dec_df(by[u], E, up));
+      } else {
+        A = fx_make(dec(ax[u], E, up), dec(ay[u], E, up));
+        B = fx_make(dec(bx[u], E, up), dec(by[u], E, up));
+      }
       if (!cplx) {
         if (oddo) {
           A = fx_make(0, -A.x);
@@ -727,6 +787,10 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
 #pragma unroll
         for (int r = 0; r < R.value; ++r, d += step)
           if (r * Ns.value < lim) *d = make_double2(enc(v[r].x, q), enc(v[r].y, q));
+      } else if (KIND == K_FWD_C2C && kind == 3) {
+#pragma unroll
+        for (int r = 0; r < R.value; ++r, d += step)
+          if (r * Ns.value < lim) *d = make_double2(enc_df(v[r].x, q), enc_df(v[r].y, q));
       } else {
 #pragma unroll
         for (int r = 0; r < R.value; ++r, d += step)
@@ -754,11 +818,11 @@ __global__ void __launch_bounds__(512, 1) k_fx(const __grid_constant__ PassParam
       fx_stage<P, R0, P / R0, true, FX_TILE, false, ns - 1>(t, nullptr, wi, from_s, store);
     } else {
       constexpr bool INV = KIND == K_INV_C2C;
-      fx_stage<P, R0, 1, INV, FX_RAW, true, 0>(t, emax, wf, load, to_s);
+      fx_stage<P, R0, 1, INV, INV ? FX_RAW_DF : FX_RAW, true, 0>(t, emax, wf, load, to_s);
       fx_mid_stages<P, RW, INV, false, 1, ns - 1>(t, wf);
       const int E = max(m.emax[l0], kFxMinE);
       q = E + shift - fx_shifted<P>(m.words, W, l0, true, false, false);
-      kind = fx_out_kind(E, q);
+      kind = INV ? fx_out_kind(E, q) : fx_store_kind(p, E, q);
       fx_stage<P, RL, P / RL, INV, FX_TILE, false, ns - 1>(t, nullptr, wf, from_s, store);
     }
   }

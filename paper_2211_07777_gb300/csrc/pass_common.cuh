@@ -20,22 +20,6 @@ template <> __device__ __forceinline__ void st_real<dfloat>(dfloat* a, long long
   else reinterpret_cast<float2*>(a)[off] = make_float2(v.hi, v.lo);
 }
 
-// The same for complex values (a double-float pass between fixed-point ones reads and writes FP64 arrays).  Loads take
-// the element's 16 bytes as they are and convert where it is used: a branch between the loads of a batch would wait
-// for each before the next.
-template <typename T> __device__ __forceinline__ cpx<T> from_array(cpx<T> v, int f64) { return v; }
-template <> __device__ __forceinline__ cdfloat from_array<dfloat>(cdfloat v, int f64) {
-  if (!f64) return v;
-  return mk<dfloat>(
-      df_from_double(__hiloint2double(__float_as_int(v.x.lo), __float_as_int(v.x.hi))),
-      df_from_double(__hiloint2double(__float_as_int(v.y.lo), __float_as_int(v.y.hi))));
-}
-template <typename T> __device__ __forceinline__ void st_cplx(cpx<T>* a, long long off, cpx<T> v, int f64) { a[off] = v; }
-template <> __device__ __forceinline__ void st_cplx<dfloat>(cdfloat* a, long long off, cdfloat v, int f64) {
-  if (f64) reinterpret_cast<double2*>(a)[off] = make_double2(df_to_double(v.x), df_to_double(v.y));
-  else a[off] = v;
-}
-
 // Index of element (row i, lane l) of a tile: the compile-time engine's layout (WC > 0) or rows of
 // LS elements (runtime engine).
 // log2 of a power of two, at compile time
@@ -322,12 +306,11 @@ __device__ __forceinline__ void load_cplx(const PassParams& p, const cpx<T>* __r
       ll[u] = lane;
       ii[u] = i;
       const int q = q0 + lane;
-      v[u] = (i >= 0 && q < p.npen) ? in[(long long)q * p.ai.ls + (long long)i * p.ai.js]
-                                    : mk<T>((T)0, (T)0);
+      v[u] = (i >= 0 && q < p.npen) ? in[(long long)q * p.ai.ls + (long long)i * p.ai.js] : mk<T>((T)0, (T)0);
     }
 #pragma unroll
     for (int u = 0; u < LOADB; ++u)
-      if (ii[u] >= 0) S[tix<T, WC>(ii[u], ll[u], LS)] = from_array<T>(v[u], p.in_f64);
+      if (ii[u] >= 0) S[tix<T, WC>(ii[u], ll[u], LS)] = v[u];
   }
 }
 
@@ -344,7 +327,7 @@ __device__ __forceinline__ void store_cplx_data(const PassParams& p, cpx<T>* __r
     const int q = q0 + lane;
     if (q >= p.npen) continue;
     const int pos = (p.type == T_PER && p.center == C_NODE && i == p.N) ? 0 : i;
-    st_cplx<T>(out, (long long)q * p.ao.ls + (long long)i * p.ao.js, S[tix<T, WC>(pos, lane, LS)], p.out_f64);
+    out[(long long)q * p.ao.ls + (long long)i * p.ao.js] = S[tix<T, WC>(pos, lane, LS)];
   }
 }
 

@@ -82,6 +82,7 @@ struct PassParams {
   int rows_off;
   int fx;                 // FP64-class pass in 64-bit fixed point (fx_passes.cu)
   int fx_host;            // such an x pass reads or writes pinned host memory: whole row pieces per warp
+  int fx_df;              // double-float arrays around the FP64E curl: bit 0 this pass reads, bit 1 writes one
   int f2;                 // FP32 pass on pairs of lanes in packed arithmetic (f2_passes.cu)
   int f2_vec;             // its 16-byte accesses: bit 0 the input, bit 1 the output array
   int pdl;                // launched as a programmatic dependent of the stream's previous kernel: each CTA

@@ -88,6 +88,21 @@ int main() {
       else worst = std::fmax(worst, std::fabs(sum) / n - (d > up ? ldexpl(0.5L, up - d) : 0));
     }
   std::printf("decode_all %.4Lg\ndecode_mean %.3Lg\ndecode_binade %.3Lg\n", wd, all, worst);
+  // double-float values below the lane's largest (2^20): both floats rounded
+  ld wdf = 0;
+  for (int t = 0; t < 100000; ++t) {
+    const double v = std::ldexp((double)uni(), 20 - (t % 60));
+    const float hi = (float)v, lo = (float)(v - (double)hi);
+    unsigned wh, wl;
+    std::memcpy(&wh, &hi, 4);
+    std::memcpy(&wl, &lo, 4);
+    const int E = 1023 + 19;
+    const unsigned long long b = ((unsigned long long)wl << 32) | wh;
+    wdf = std::fmax(wdf, std::fabs(ldexpl((ld)hi + lo, kFxBias - E) - (ld)fx_decode_df(b, E)));
+    if (fx_float_exp(wh & 0x7fffffffu) > E) return 13;
+  }
+  if (fx_decode_df(0, kFxMinE) != 0 || fx_float_exp(0) != 0 || fx_float_exp(0x7f800000u) != 2047) return 14;
+  std::printf("decode_df %.3Lg\n", wdf);
   // Green products: factors over 60 binary orders with modes over 60, the larger product of a pair aligned to 57 bits
   ld wg = 0, wa = 0;
   for (int t = 0; t < 100000; ++t) {

@@ -40,6 +40,7 @@ def test_products_and_decoding(errors):
     assert errors["cmul"] < 1.5      # two parts of at most 0.5 + 0.25 + 0.25 units
     assert errors["mul"] < 1.0
     assert errors["decode"] <= 0.5 and errors["decode_all"] <= 0.5   # rounded to nearest
+    assert errors["decode_df"] <= 1.0   # two floats, half a unit each
     assert errors["zero"] == 0 and errors["subnormal"] == 0
     assert errors["shr_even"] == 207
 

@@ -6,6 +6,7 @@ import pytest
 import oracle
 from oracle import CELL, NODE, EVEN as E, ODD as O, PER, UNB as U
 from paper_2211_07777_gb300 import flups as F
+from paper_2211_07777_gb300 import serve
 from tests.gpu_util import cuda_solve, rel_linf
 
 pytestmark = pytest.mark.gpu
@@ -158,3 +159,23 @@ def test_sizes_around_the_line_match_the_oracle(n, prec):
     ref = oracle.solve(f, oracle.Problem(bc=((PER, PER),) * 3, h=h, center=CELL, kernel="spectral"))
     # double-float passes (at most 15 butterfly levels of 2u, u = 2^-48, per direction and way) bound the pair
     assert np.linalg.norm(got - ref) < 6 * 15 * 2.0 ** -47 * np.linalg.norm(ref)
+
+
+# FP64E Biot-Savart: the passes beside the curl write and read its double-float array (second direction complex, real
+# with complex modes, real with real modes; a quarter-wave and a semi-open one)
+@pytest.mark.parametrize("center", [CELL, NODE], ids=["cell", "node"])
+@pytest.mark.parametrize("bcs", [((U, U), (U, U), (U, U)), ((E, E), (PER, PER), (U, U)), ((O, O), (E, O), (U, U)),
+                                 ((E, U), (U, O), (E, E)), ((PER, PER), (PER, PER), (PER, PER))],
+                         ids=["open", "wall-periodic", "walls", "semi", "periodic"])
+def test_double_float_curl_between_fixed_point_passes(bcs, center):
+    n = (36, 32, 48)
+    data = [v + (1 if center == NODE else 0) for v in n]
+    f = np.random.default_rng(12).standard_normal((3, data[2], data[1], data[0]))
+    bc, h = serve.vector_bc(bcs), (1 / 48,) * 3
+    L = tuple(v / 48 for v in n)
+    kernel = "hej2" if any(U in b for b in bcs) else "spectral"
+    got = {p: cuda_solve(f, bc, center, p, kernel, h=h, L=L, op=F.BIOT_SAVART)[0] for p in (F.F64, F.F64E)}
+    # 15 butterfly levels of 2u, u = 2^-48, in the curl's two transforms
+    assert np.linalg.norm(got[F.F64E] - got[F.F64]) < 2 * 15 * 2.0 ** -47 * np.linalg.norm(got[F.F64])
+    f[1, 3, 4, 5] = np.nan
+    assert np.isnan(cuda_solve(f, bc, center, F.F64E, kernel, h=h, L=L, op=F.BIOT_SAVART)[0]).any()
