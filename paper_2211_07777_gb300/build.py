@@ -20,7 +20,13 @@ LIB = os.path.join(PKG, "libflups_gpu.so")
 INCLUDE = os.path.join(ROOT, "include")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2", "-I", INCLUDE, "-I", CSRC]
+FLAGS = ["-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2", "-I", INCLUDE, "-I", CSRC]
+
+
+def flags_of(src: str) -> list:
+    """Source lines for profiles in every unit but the fixed-point lengths: their line tables (deeply inlined code) made the
+    first plan of a unit's lengths wait 20 ms for its load, 1.4 ms without.  extra_flags=["-lineinfo"] brings them back."""
+    return FLAGS if os.path.basename(src).startswith("fx_len_") else [*FLAGS, "-lineinfo"]
 
 
 def nvcc() -> str:
@@ -46,7 +52,6 @@ def _stale(obj: str, src: str) -> bool:
 def build(verbose: bool = False, force: bool = False, extra_flags=None) -> str:
     os.makedirs(BUILD, exist_ok=True)
     cc = nvcc()
-    flags = FLAGS + list(extra_flags or [])
     srcs = sources()
     objs = [os.path.join(BUILD, os.path.basename(s)[:-3] + ".o") for s in srcs]
 
@@ -54,7 +59,7 @@ def build(verbose: bool = False, force: bool = False, extra_flags=None) -> str:
         src, obj = so
         if not force and not _stale(obj, src):
             return ""
-        cmd = [cc, *ARCH, *flags, "-c", src, "-o", obj]
+        cmd = [cc, *ARCH, *flags_of(src), *(extra_flags or []), "-c", src, "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed on {os.path.basename(src)}:\n{r.stderr}")

@@ -179,3 +179,30 @@ def test_double_float_curl_between_fixed_point_passes(bcs, center):
     assert np.linalg.norm(got[F.F64E] - got[F.F64]) < 2 * 15 * 2.0 ** -47 * np.linalg.norm(got[F.F64])
     f[1, 3, 4, 5] = np.nan
     assert np.isnan(cuda_solve(f, bc, center, F.F64E, kernel, h=h, L=L, op=F.BIOT_SAVART)[0]).any()
+
+
+FIRST_PLANS = """
+import sys, time
+sys.path.insert(0, sys.argv[1])
+import torch
+from paper_2211_07777_gb300 import flups as F
+def plan(n):
+    t = time.perf_counter()
+    F.Solver((n,) * 3, ((F.UNB, F.UNB),) * 3, prec=F.F64, green="hej2").close()
+    return time.perf_counter() - t
+torch.ones(1, device="cuda")
+plan(32)
+print(min(plan(n) for n in (64, 36, 48)))
+"""
+
+
+def test_the_first_plan_of_a_length_loads_its_kernels_quickly():
+    """In a new process, after its first plan: the lengths' kernels load in 1 to 3 ms (20 ms and more with their line
+    tables)."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", FIRST_PLANS, root], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert float(r.stdout) < 0.010, r.stdout
