@@ -1062,9 +1062,8 @@ void set_rows_bulk(Launch& L, int prec) {
 bool use_f2(const flups_solver_s* s, const Launch& L, const DirPlan& dp, int axis) {
   if (s->topo.prec != FLUPS_F32) return false;
   const int P = dp.P;
-  if (L.kind >= K_CURL_REAL)  // three times the threads of a tile, within the kernel's 512
-    return 3 * (((P * fx_width(FX_CURL, P) + f2_ept(FX_CURL, P) - 1) / f2_ept(FX_CURL, P) + 31) / 32 * 32) <= 512;
-  if (P & (P - 1)) return true;
+  if (L.kind >= K_CURL_REAL) return f2_curl(P);
+  if (f2_complex(P)) return true;
   if (L.kind == K_FUSED_REAL) return true;
   if (L.kind != K_FWD_REAL && L.kind != K_INV_REAL) return false;
   const bool modes = dp.type == T_PER || dp.type == T_UNB;

@@ -746,26 +746,38 @@ __global__ void __launch_bounds__(512, 1) k_f2_curl(const __grid_constant__ Pass
 
 }  // namespace
 
+template <int KIND, int P> constexpr bool f2_has() {
+  if (KIND == K_FWD_C2C || KIND == K_INV_C2C || KIND == K_FUSED_C2C) return f2_complex(P);
+  return KIND >= K_CURL_REAL ? f2_curl(P) : true;
+}
+// The kernel of a kind and length (nullptr: the planner sends no such pass here).
+template <int KIND, int P> constexpr auto f2_kernel() {
+  using Kernel = void (*)(PassParams);
+  if constexpr (!f2_has<KIND, P>()) return Kernel(nullptr);
+  else if constexpr (KIND >= K_CURL_REAL) return Kernel(k_f2_curl<KIND == K_CURL_REAL, P>);
+  else return Kernel(k_f2<KIND, P>);
+}
 template <int KIND, int P>
 cudaError_t f2_launch(const PassParams& p, dim3 grid, int nthr, size_t smem, cudaStream_t st) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3((unsigned)nthr);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = p.pdl ? 1 : 0;
-  if constexpr (KIND >= K_CURL_REAL) return cudaLaunchKernelEx(&cfg, k_f2_curl<KIND == K_CURL_REAL, P>, p);
-  else return cudaLaunchKernelEx(&cfg, k_f2<KIND, P>, p);
+  if constexpr (!f2_has<KIND, P>()) {
+    return cudaErrorInvalidValue;
+  } else {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)nthr);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = p.pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, f2_kernel<KIND, P>(), p);
+  }
 }
 template <int KIND, int P> cudaError_t f2_limit() {
-  const int lim = 227 * 1024;
-  if constexpr (KIND >= K_CURL_REAL)
-    return cudaFuncSetAttribute(k_f2_curl<KIND == K_CURL_REAL, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  else return cudaFuncSetAttribute(k_f2<KIND, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if constexpr (!f2_has<KIND, P>()) return cudaErrorInvalidValue;
+  else return cudaFuncSetAttribute(f2_kernel<KIND, P>(), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
 }
 #define F2_KINDS(DO)                   \
   switch (kind) {                      \

@@ -230,6 +230,13 @@ __host__ __device__ constexpr int f2_ept(int cls, int P) {
   }
   return e;
 }
+// threads of a full tile of the Biot-Savart pass; within a CTA's 512, else the length runs on the kernels of curl.cu
+__host__ __device__ constexpr int f2_curl_threads(int P) {
+  return 3 * (((P * fx_width(FX_CURL, P) + f2_ept(FX_CURL, P) - 1) / f2_ept(FX_CURL, P) + 31) / 32 * 32);
+}
+// What the lane pairs take: complex passes of powers of two stay on the column kernels (use_f2).
+__host__ __device__ constexpr bool f2_complex(int P) { return (P & (P - 1)) != 0; }
+__host__ __device__ constexpr bool f2_curl(int P) { return f2_curl_threads(P) <= 512; }
 template <int P, int CLS> struct F2Rows {
   static constexpr int W = fx_width(CLS, P);
   static constexpr F2Plan plan = f2_plan_of(CLS, P);

@@ -1091,6 +1091,10 @@ cudaError_t pass_launch(K kernel, const PassParams& p, dim3 grid, int nthr, size
   return cudaLaunchKernelEx(&cfg, kernel, p);
 }
 
+// FP64 tiles of 128 points and more serve flups_solve_periodic_noalloc alone (larger problems run in fixed point, and
+// below that no grid fills the device): x passes of real data and column passes, periodic.
+template <typename T, int PC> constexpr bool periodic_only() { return std::is_same<T, double>::value && PC >= 128; }
+
 template <typename T, int PC, int WC, bool HZ>
 cudaError_t launch_kind_hz(int kind, const PassParams& p, dim3 grid, int nthr, size_t smem, cudaStream_t st) {
   if constexpr (PC > 0 && std::is_same<T, float>::value) {
@@ -1131,6 +1135,10 @@ cudaError_t launch_kind_hz(int kind, const PassParams& p, dim3 grid, int nthr, s
   switch (kind) {
     case K_FWD_REAL: return pass_launch(k_fwd_real<T, PC, WC, HZ>, p, grid, nthr, smem, st);
     case K_INV_REAL: return pass_launch(k_inv_real<T, PC, WC, HZ>, p, grid, nthr, smem, st);
+    default: break;
+  }
+  if constexpr (periodic_only<T, PC>()) return cudaErrorInvalidValue;
+  else switch (kind) {
     case K_FWD_C2C: return pass_launch(k_fwd_c2c<T, PC, WC, HZ>, p, grid, nthr, smem, st);
     case K_INV_C2C: return pass_launch(k_inv_c2c<T, PC, WC, HZ>, p, grid, nthr, smem, st);
     case K_FUSED_REAL: return pass_launch(k_fused_real<T, PC, WC, HZ>, p, grid, nthr, smem, st);
@@ -1143,7 +1151,9 @@ cudaError_t launch_kind_hz(int kind, const PassParams& p, dim3 grid, int nthr, s
 // input is zero padding and half of its output is discarded (compile-time engine only)
 template <typename T, int PC, int WC>
 cudaError_t launch_kind(int kind, const PassParams& p, dim3 grid, int nthr, size_t smem, cudaStream_t st) {
-  if constexpr (PC > 0) {
+  if constexpr (periodic_only<T, PC>()) {
+    if (p.hz) return cudaErrorInvalidValue;
+  } else if constexpr (PC > 0) {
     if (p.hz) return launch_kind_hz<T, PC, WC, true>(kind, p, grid, nthr, smem, st);
   }
   return launch_kind_hz<T, PC, WC, false>(kind, p, grid, nthr, smem, st);
@@ -1155,9 +1165,6 @@ cudaError_t set_limits_hz() {
   cudaError_t e;
   if ((e = cudaFuncSetAttribute(k_fwd_real<T, PC, WC, HZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
   if ((e = cudaFuncSetAttribute(k_inv_real<T, PC, WC, HZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
-  if ((e = cudaFuncSetAttribute(k_fwd_c2c<T, PC, WC, HZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
-  if ((e = cudaFuncSetAttribute(k_inv_c2c<T, PC, WC, HZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
-  if ((e = cudaFuncSetAttribute(k_fused_real<T, PC, WC, HZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
   if constexpr (PC > 0) {
     if ((e = cudaFuncSetAttribute(k_fwd_c2c_col<T, PC, WC, HZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
     if ((e = cudaFuncSetAttribute(k_inv_c2c_col<T, PC, WC, HZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
@@ -1176,13 +1183,19 @@ cudaError_t set_limits_hz() {
       if ((e = cudaFuncSetAttribute(k_fused_c2c_col<T, PC, WC, HZ, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
     }
   }
-  return cudaFuncSetAttribute(k_fused_c2c<T, PC, WC, HZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if constexpr (!periodic_only<T, PC>()) {
+    if ((e = cudaFuncSetAttribute(k_fwd_c2c<T, PC, WC, HZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
+    if ((e = cudaFuncSetAttribute(k_inv_c2c<T, PC, WC, HZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
+    if ((e = cudaFuncSetAttribute(k_fused_real<T, PC, WC, HZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
+    if ((e = cudaFuncSetAttribute(k_fused_c2c<T, PC, WC, HZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
+  }
+  return cudaSuccess;
 }
 
 template <typename T, int PC, int WC>
 cudaError_t set_limits_kind() {
   cudaError_t e = set_limits_hz<T, PC, WC, false>();
-  if constexpr (PC > 0) {
+  if constexpr (PC > 0 && !periodic_only<T, PC>()) {
     if (!e) e = set_limits_hz<T, PC, WC, true>();
   }
   return e;

@@ -161,6 +161,23 @@ def test_sizes_around_the_line_match_the_oracle(n, prec):
     assert np.linalg.norm(got - ref) < 6 * 15 * 2.0 ** -47 * np.linalg.norm(ref)
 
 
+# Below the line, three components fill the device in short FP64 tiles along y (64 points between walls: runtime tiles)
+@pytest.mark.parametrize("bcs", [((PER, PER),) * 3, ((PER, PER), (U, U), (PER, PER)), ((E, E), (O, O), (PER, PER))],
+                         ids=["periodic", "open", "walls"])
+@pytest.mark.parametrize("P", [32, 64])
+def test_thin_vector_boxes_in_fp64_tiles(bcs, P):
+    m = 2 if bcs[1][0] in (U, O) else 1
+    n = (4, P // m, (4096 if bcs[0] == (E, E) else 8192) // P)  # 32768 points of the extension
+    f = np.random.default_rng(P).standard_normal((3, *n[::-1]))
+    h = (1.0 / max(n),) * 3
+    L = tuple(v * h[0] for v in n)
+    kernel = "hej2" if (U, U) in bcs else "spectral"
+    got = cuda_solve(f, (bcs,) * 3, CELL, F.F64, kernel, h=h, L=L)[0]
+    for c in range(3):
+        ref = oracle.solve(f[c], oracle.Problem(bc=bcs, h=h, center=CELL, kernel=kernel))
+        assert rel_linf(got[c], ref) < 1e-13
+
+
 # FP64E Biot-Savart: the passes beside the curl write and read its double-float array (second direction complex, real
 # with complex modes, real with real modes; a quarter-wave and a semi-open one)
 @pytest.mark.parametrize("center", [CELL, NODE], ids=["cell", "node"])

@@ -44,6 +44,23 @@ def test_noalloc_matches_regular_solve_on_two_calls_in_a_row():
         assert np.abs(out - ref).max() / np.abs(ref).max() < 1e-12
 
 
+# Every length of the FP64 tiles (128 points and more; grids that fill the device, within the fixed array)
+@pytest.mark.parametrize("n", [(128, 96, 108), (96, 128, 96), (96, 96, 128), (256, 64, 81), (64, 256, 64), (64, 64, 256),
+                               (512, 64, 81), (64, 512, 64), (64, 64, 512), (1024, 48, 54), (32, 1024, 64),
+                               (32, 64, 1024), (2048, 36, 36), (32, 2048, 36), (32, 36, 2048)])
+def test_noalloc_matches_regular_solve_at_every_tile_length(n):
+    import torch
+    from paper_2211_07777_gb300 import flups as F
+    f = np.random.default_rng(n[0]).standard_normal(n[::-1])
+    L = tuple(v / max(n) for v in n)
+    ref = _regular(f, L)
+    rhs = torch.from_numpy(f).cuda()
+    phi = torch.full_like(rhs, float("nan"))
+    F.flups_solve_periodic_noalloc(phi, rhs, n, L)
+    torch.cuda.synchronize()
+    assert np.linalg.norm(phi.cpu().numpy() - ref) < 1e-14 * np.linalg.norm(ref)
+
+
 def test_noalloc_rejects_sizes_beyond_its_array():
     import torch
     from paper_2211_07777_gb300 import flups as F
