@@ -165,8 +165,8 @@ int flups_pass_info(flups_solver s, int i, int* kind, int* axis, int* fft_len, d
 /* How pass i runs (bit flags): 1 compile-time tile engine, 2 Green slice staged in shared memory
  * ahead of the multiply, 4 that slice copied by TMA (tensor map + mbarrier), 8 doubled transform
  * pruned to its nonzero half, 16 input tile copied by TMA (tensor map + mbarrier), 32 x pass on the
- * column kernels' register-chained stages, 64 input rows staged by one bulk copy.  Introspection
- * only; no counterpart in the paper. */
+ * column kernels' register-chained stages, 64 input rows staged by one bulk copy, 128 64-bit fixed
+ * point, 256 FP32 on pairs of lanes.  Introspection only; no counterpart in the paper. */
 int flups_pass_features(flups_solver s, int i, int* flags);
 
 /* Allocation-free fully periodic solve (the paper has no counterpart; this is

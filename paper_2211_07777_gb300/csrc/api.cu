@@ -457,7 +457,7 @@ void fill_geom(Launch& L, const DirPlan& dp, int axis, const int* din, const int
 
 // Tile of a fixed-point pass (after fill_geom): the full width of fx_width, narrower when the grid would leave SMs
 // idle (rows keep their stride).
-void fx_geom(Launch& L, const DirPlan& dp, int axis, bool packed) {
+void fx_geom(Launch& L, const DirPlan& dp, bool packed) {
   PassParams& p = L.p;
   p.tw = dp.twx;
   const int P = p.P;
@@ -483,12 +483,10 @@ void fx_geom(Launch& L, const DirPlan& dp, int axis, bool packed) {
   L.nthr = nt;
   // alignment, mbarrier block, tile, Green offsets, lane exponents, renormalisation words
   L.smem = 128 + 128 + (size_t)fx_tile_values(cls, P) * 16 + (size_t)W * (2 * 8 + 4 + kFxSlots * 4);
-  p.rowx = (axis == 0 && p.center == C_CELL && (p.type == T_PER || p.type == T_UNB) &&
-            (L.kind == K_FWD_REAL || L.kind == K_INV_REAL)) ? 1 : 0;
 }
 
 // Tile of an FP32 lane-pair pass (after fill_geom): as fx_geom, a lane holding two complex or four real pencils.
-void f2_geom(Launch& L, const DirPlan& dp, int axis, bool packed) {
+void f2_geom(Launch& L, const DirPlan& dp, bool packed) {
   PassParams& p = L.p;
   const bool curl = L.kind >= K_CURL_REAL;
   const int P = p.P, per = packed ? 4 : 2, cls = curl ? FX_CURL : FX_PLAIN;
@@ -504,8 +502,6 @@ void f2_geom(Launch& L, const DirPlan& dp, int axis, bool packed) {
   p.W = W;
   p.lw = ilog2(W);
   p.f2 = 1;
-  p.rowx = (axis == 0 && p.center == C_CELL && (p.type == T_PER || p.type == T_UNB) &&
-            (L.kind == K_FWD_REAL || L.kind == K_INV_REAL)) ? 1 : 0;
   p.ct = 0;
   p.hz = 0;
   p.ept = 0;
@@ -713,7 +709,7 @@ int setup_green_compute(flups_solver_s* s, cudaStream_t st) {
     Launch L{};
     L.kind = K_FWD_REAL;
     fill_geom(L, gp, d, q.gext, q.gext, FLUPS_F64, true, FLUPS_NODE, 1);
-    fx_geom(L, gp, d, true);
+    fx_geom(L, gp, true);
     L.p.in = g64;
     L.p.out = g64;
     e = limit_fx(L.kind, gp.P);
@@ -1093,8 +1089,8 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     L.kind = K_FWD_REAL;
     fill_geom(L, s->dir[o[0]], o[0], s->dims[0], s->dims[1], prec, true, center, nc, 1, s->pitch[0], s->pitch[1]);
     L.p.ctypes = pack3(s->tf[0][o[0]], s->tf[1][o[0]], s->tf[2][o[0]]);
-    if (s->fxp) fx_geom(L, s->dir[o[0]], o[0], true);
-    else if (use_f2(s, L, s->dir[o[0]], o[0])) f2_geom(L, s->dir[o[0]], o[0], true);
+    if (s->fxp) fx_geom(L, s->dir[o[0]], true);
+    else if (use_f2(s, L, s->dir[o[0]], o[0])) f2_geom(L, s->dir[o[0]], true);
     L.p.out = s->W1;
     L.out_buf = 1;
     L.user_in = 1;
@@ -1111,8 +1107,8 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     L.kind = real ? K_FWD_REAL : K_FWD_C2C;
     fill_geom(L, s->dir[o[1]], o[1], s->dims[1], s->dims[2], prec, real, center, nc, 1, s->pitch[1], s->pitch[2]);
     L.p.ctypes = pack3(s->tf[0][o[1]], s->tf[1][o[1]], s->tf[2][o[1]]);
-    if (s->fxp) fx_geom(L, s->dir[o[1]], o[1], real);
-    else if (use_f2(s, L, s->dir[o[1]], o[1])) f2_geom(L, s->dir[o[1]], o[1], real);
+    if (s->fxp) fx_geom(L, s->dir[o[1]], real);
+    else if (use_f2(s, L, s->dir[o[1]], o[1])) f2_geom(L, s->dir[o[1]], real);
     if (s->fxp && !s->fx && prec == FLUPS_F64E) L.p.fx_df = 2;  // the curl's double-float array
     L.p.in = s->W1;
     L.p.out = s->W2;
@@ -1133,8 +1129,8 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     fill_geom(L, dp, o[2], s->dims[2], s->dims[2], prec, real, center, curl ? 1 : nc, curl ? 3 : 1, s->pitch[2],
               s->pitch[2]);
     L.p.ctypes = pack3(s->tf[0][o[2]], s->tf[1][o[2]], s->tf[2][o[2]]);
-    if (s->fx) fx_geom(L, dp, o[2], real);
-    else if (use_f2(s, L, dp, o[2])) f2_geom(L, dp, o[2], real);
+    if (s->fx) fx_geom(L, dp, real);
+    else if (use_f2(s, L, dp, o[2])) f2_geom(L, dp, real);
     L.p.in = s->W2;
     L.p.out = s->W2;
     L.in_buf = 2;
@@ -1208,8 +1204,8 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     L.kind = real ? K_INV_REAL : K_INV_C2C;
     fill_geom(L, s->dir[o[1]], o[1], s->dims[2], s->dims[1], prec, real, center, nc, 1, s->pitch[2], s->pitch[1]);
     L.p.ctypes = pack3(s->tu[0][o[1]], s->tu[1][o[1]], s->tu[2][o[1]]);
-    if (s->fxp) fx_geom(L, s->dir[o[1]], o[1], real);
-    else if (use_f2(s, L, s->dir[o[1]], o[1])) f2_geom(L, s->dir[o[1]], o[1], real);
+    if (s->fxp) fx_geom(L, s->dir[o[1]], real);
+    else if (use_f2(s, L, s->dir[o[1]], o[1])) f2_geom(L, s->dir[o[1]], real);
     if (s->fxp && !s->fx && prec == FLUPS_F64E) L.p.fx_df = 1;
     L.p.in = s->W2;
     L.p.out = s->W1;
@@ -1226,8 +1222,8 @@ int build_passes(flups_solver_s* s, cudaStream_t st) {
     L.kind = K_INV_REAL;
     fill_geom(L, s->dir[o[0]], o[0], s->dims[1], s->dims[0], prec, true, center, nc, 1, s->pitch[1], s->pitch[0]);
     L.p.ctypes = pack3(s->tu[0][o[0]], s->tu[1][o[0]], s->tu[2][o[0]]);
-    if (s->fxp) fx_geom(L, s->dir[o[0]], o[0], true);
-    else if (use_f2(s, L, s->dir[o[0]], o[0])) f2_geom(L, s->dir[o[0]], o[0], true);
+    if (s->fxp) fx_geom(L, s->dir[o[0]], true);
+    else if (use_f2(s, L, s->dir[o[0]], o[0])) f2_geom(L, s->dir[o[0]], true);
     L.p.in = s->W1;
     L.in_buf = 1;
     L.user_out = 1;
@@ -1689,7 +1685,7 @@ int flups_pass_features(flups_solver s, int i, int* flags) {
   if (i < 0 || i >= (int)s->passes.size()) return FLUPS_EINVAL;
   const PassParams& p = s->passes[i].p;
   *flags = (p.ct ? 1 : 0) | (p.gpre ? 2 : 0) | (p.gmap ? 4 : 0) | (p.hz ? 8 : 0) | (p.tin_rows ? 16 : 0) |
-           (p.rowx ? 32 : 0) | (p.rows_bulk ? 64 : 0);
+           (p.rowx ? 32 : 0) | (p.rows_bulk ? 64 : 0) | (p.fx ? 128 : 0) | (p.f2 ? 256 : 0);
   return FLUPS_OK;
 }
 

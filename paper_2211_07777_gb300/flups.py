@@ -444,14 +444,15 @@ class Solver:
         flups_solve_host(self._s, phi_host, rhs_host, stream)
 
     def features(self):
-        """Per pass: dict(ct, staged_green, tma_green, pruned) (flups_pass_features)."""
+        """Per pass: dict of the kernels' features (flups_pass_features)."""
         out = []
         for i in range(self.info["launches"]):
             f = ctypes.c_int(0)
             _check(lib().flups_pass_features(self._s, i, ctypes.byref(f)), "flups_pass_features")
             v = f.value
             out.append({"ct": bool(v & 1), "staged_green": bool(v & 2), "tma_green": bool(v & 4), "pruned": bool(v & 8),
-                        "tma_input": bool(v & 16), "row_stages": bool(v & 32), "bulk_rows": bool(v & 64)})
+                        "tma_input": bool(v & 16), "row_stages": bool(v & 32), "bulk_rows": bool(v & 64),
+                        "fixed_point": bool(v & 128), "lane_pairs": bool(v & 256)})
         return out
 
     def debug_wait_limit(self, mask: int):

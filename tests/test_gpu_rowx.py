@@ -1,6 +1,6 @@
-"""The x passes on the register-chained stages (periodic and doubled unbounded x, FP32 and
-double-float, 1024-point transforms) against the FP64 oracle, and the generic row kernels the same solve uses when its
-arrays are pinned host memory.  The grids have few y-z rows but enough for the compile-time
+"""The x passes on the register-chained stages (periodic and doubled unbounded x, FP32, 1024-point
+transforms) and in fixed point (FP64E) against the FP64 oracle, and the same solve on pinned host memory, where FP32 uses
+the generic row kernels.  The grids have few y-z rows but enough for the compile-time
 engine: 1024 (periodic) or 512 doubled (unbounded) points along x."""
 import numpy as np
 import pytest
@@ -49,7 +49,9 @@ def test_row_stages_match_the_oracle(n, bc, kernel, prec):
     dt = torch.float32 if prec == F.F32 else torch.float64
     with F.Solver(n, bc, L=L, center=F.CELL, prec=prec, green=kernel) as s:
         feats = s.features()
-        assert feats[0]["row_stages"] and feats[-1]["row_stages"], feats
+        engine = "row_stages" if prec == F.F32 else "fixed_point"
+        for key in ("row_stages", "fixed_point", "lane_pairs"):
+            assert feats[0][key] == feats[-1][key] == (key == engine), (key, feats)
         rhs = torch.from_numpy(f).to("cuda", dt)
         phi = torch.empty_like(rhs)
         s.solve(phi, rhs)
