@@ -363,7 +363,8 @@ def kernel_source_sha():
     return h.hexdigest()[:16]
 
 
-KIND_NAMES = {0: "k_fwd_real", 1: "k_inv_real", 2: "k_fwd_c2c", 3: "k_inv_c2c", 4: "k_fused_real", 5: "k_fused_c2c"}
+KIND_NAMES = {0: "k_fwd_real", 1: "k_inv_real", 2: "k_fwd_c2c", 3: "k_inv_c2c", 4: "k_fused_real", 5: "k_fused_c2c",
+              6: "k_curl_real", 7: "k_curl_c2c"}
 
 
 def measured_peaks():
@@ -411,27 +412,32 @@ def device_rhs(torch, wl, dev, f_host=None):
     return torch.from_numpy(f_host if f_host is not None else wl["rhs"]()).to(dev, dt)
 
 
+def pass_infos(solver, npass):
+    """Per pass: flups_pass_info and whether it runs in fixed point."""
+    return [dict(solver.pass_info(i), fixed_point=f["fixed_point"]) for i, f in zip(range(npass), solver.features())]
+
+
 def roofline(pinfo, mean_pass, prec, peaks, workload_name):
-    """Roofline of the dominant pass: HBM, and the FP64 FMA rate for the FP64 passes of small problems (larger ones
-    run in fixed point on the integer units)."""
-    axes = {i["axis"]: i["P"] for i in pinfo if "axis" in i and "P" in i}
-    if prec == 1 and len(axes) == 3 and int(np.prod(list(axes.values()))) > 32768:
-        prec = 2
+    """Roofline of the dominant pass by the engine that runs it (pass_infos): the FP64 FMA rate for FP64 kernels (the
+    small problems' and the Biot-Savart curl); HBM for the others, where fixed-point passes are bound by the integer
+    pipes and report the share of HBM beside that."""
     dom = int(np.argmax(mean_pass))
     kname = KIND_NAMES[pinfo[dom]["kind"]]
     hbm, hbm_src = measured_peaks()
     ach_gbs = pinfo[dom]["bytes"] / (mean_pass[dom] * 1e-3) / 1e9
     ach_tf = pinfo[dom]["flops"] / (mean_pass[dom] * 1e-3) / 1e12
     fp64 = peaks.get("fp64_tflops") if peaks else None
-    if prec == 1 and fp64:
+    fixed = bool(pinfo[dom].get("fixed_point"))
+    if prec == 1 and not fixed and fp64:
         roof = {"bound": "alu", "achieved": ach_tf, "peak": fp64, "unit": "TFLOP/s", "frac": ach_tf / fp64,
                 "peak_source": "measured FP64 FMA rate (flups_measure_fma_peak) on this device",
                 "hbm_achieved_gbs": ach_gbs, "hbm_frac": ach_gbs / hbm, "hbm_peak_gbs": hbm}
     else:
-        roof = {"bound": "hbm", "achieved": ach_gbs, "peak": hbm, "unit": "GB/s", "frac": ach_gbs / hbm,
+        roof = {"bound": "integer" if fixed else "hbm", "achieved": ach_gbs, "peak": hbm, "unit": "GB/s",
+                "frac": ach_gbs / hbm,
                 "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if hbm_src == "measured"
                 else "fallback 6.8 TB/s"}
-        if prec == 2 and fp64:
+        if prec in (1, 2) and fp64:
             roof["fp64_equiv_tflops"] = ach_tf
             roof["fp64_equiv_over_measured_fp64_peak"] = ach_tf / fp64
     roof["kernel"] = kname
@@ -487,7 +493,7 @@ def measure_variant(F, torch, name, f_host, ref, flush, stream, K, warmup, peaks
             rec["rel_err_vs_closed_form"] = rel_linf(phi[zidx].double().cpu().numpy(), cf)
             rec["closed_form_planes"] = zidx
         npass = s.info["launches"]
-        pinfo = [s.pass_info(i) for i in range(npass)]
+        pinfo = pass_infos(s, npass)
         step_ms, pass_ms = timed_solves(torch, s, phi, rhs, stream, flush, K, warmup, npass)
         ms = float(np.mean(step_ms))
         mean_pass = pass_ms.mean(axis=0)
@@ -629,7 +635,7 @@ def run_ours(args):
     phi = torch.empty_like(rhs)
     stream = torch.cuda.current_stream(dev)
     npass = solver.info["launches"]
-    pinfo = [solver.pass_info(i) for i in range(npass)]
+    pinfo = pass_infos(solver, npass)
     flush = L2Flush(torch, dev)
 
     # the timed region: K solves, barrier + synchronize on both sides, clocks sampled throughout

@@ -48,6 +48,22 @@ def test_roofline_of_the_dominant_pass(monkeypatch):
     assert roof64["bound"] == "alu" and roof64["frac"] == pytest.approx(8e9 / 2e-3 / 1e12 / 1.25)
 
 
+def test_roofline_follows_the_engine_of_the_dominant_pass(monkeypatch):
+    """FP64-class solves above the fixed-point line: integer pipes; the Biot-Savart curl among them: the FP64 units."""
+    monkeypatch.setattr(bench, "measured_peaks", lambda: (6790.0, "measured"))
+    monkeypatch.setattr(bench, "traffic_record", lambda k, w: None)
+    x = {"kind": 0, "axis": 0, "P": 256, "bytes": 1e9, "flops": 1e9, "fixed_point": True}
+    y, fused = dict(x, kind=2, axis=1), dict(x, kind=5, axis=2, bytes=4e9, flops=8e9)
+    ms, peaks = np.array([0.5, 0.4, 2.0]), {"fp64_tflops": 1.25}
+    for prec in (1, 2):
+        roof = bench.roofline([x, y, fused], ms, prec, peaks, "per1024_f64")
+        assert roof["bound"] == "integer" and roof["unit"] == "GB/s"
+        assert roof["fp64_equiv_over_measured_fp64_peak"] == pytest.approx(8e9 / 2e-3 / 1e12 / 1.25)
+    curl = dict(fused, kind=7, fixed_point=False)
+    roof = bench.roofline([x, y, curl], ms, 1, peaks, "tube_f64")
+    assert roof["bound"] == "alu" and roof["unit"] == "TFLOP/s" and roof["peak"] == 1.25
+
+
 def test_traffic_record_needs_the_current_kernel_sources(tmp_path, monkeypatch):
     prof = tmp_path / "profiles"
     prof.mkdir()
