@@ -84,6 +84,26 @@ FXD long long fx_shr(long long x, int s) {
   return (x + (((1LL << s) >> 1) - one) + ((x >> s) & one)) >> s;
 }
 
+// Shifts by any count: 64 and more leave 0 or the sign (what PTX's shifts do; a clamp would cost an instruction).
+FXD unsigned long long fx_lsr(unsigned long long x, int s) {
+#ifdef __CUDA_ARCH__
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(s));
+  return r;
+#else
+  return s > 63 ? 0 : x >> s;
+#endif
+}
+FXD long long fx_asr(long long x, int s) {
+#ifdef __CUDA_ARCH__
+  long long r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(s));
+  return r;
+#else
+  return x >> (s > 63 ? 63 : s);
+#endif
+}
+
 // round(x w 2^-64), w = wh 2^32 + wl
 FXD long long fx_mul(long long x, int wh, int wl) {
   const int xh = fx_hi(x), xl = fx_lo(x);
@@ -288,14 +308,14 @@ constexpr int kFxTwShift = 64 - kFxTwBits;  // every twiddled stage divides by 2
 // up: bits below the FP64 unit of the largest value (at most 8).  The word is aligned one bit higher and rounded to
 // nearest by that bit.  Ties go away from zero: that adds at most half a unit of the value's own FP64 precision, and only where
 // one bit of it is dropped (2^-54 of the value), so one-sign inputs gain no error that FP64 would not have; a
-// truncation has half a unit of the lane's largest value instead.  (Rounding costs 2-4% of a solve, open 128^3 294 ->
-// 301 us, periodic 1024^3 41.1 -> 42.7 ms; to nearest even, from the dropped bits' carry, it costs 7-10%.)
+// truncation has half a unit of the lane's largest value instead.  (Rounding costs about 2% of a solve; to nearest even,
+// from the dropped bits' carry, 7-10%: open 128^3 326 us, periodic 1024^3 44.5 ms, truncated 294 and 41.1.)
 FXD long long fx_decode(unsigned long long bits, int E, int up = kFxUp) {
   const int hi = (int)(unsigned)(bits >> 32);
   const int e = (hi >> 20) & 0x7ff;
   const unsigned long long m = ((bits & 0xfffffffffffffull) | 0x10000000000000ull) << (up + 1);
   const int s = E - e, sg = hi >> 31;
-  const long long t = (long long)(m >> (s > 63 ? 63 : s));
+  const long long t = (long long)fx_lsr(m, s);
   return ((t ^ sg) + 1) >> 1;
 }
 
@@ -303,7 +323,7 @@ FXD long long fx_decode(unsigned long long bits, int E, int up = kFxUp) {
 FXD long long fx_decode_float(unsigned w, int E, int up) {
   const int e = (int)(w >> 23) & 255, sg = (int)w >> 31, s = E - e - 896;
   const unsigned long long m = (unsigned long long)(e ? (w & 0x7fffffu) | 0x800000u : 0) << (30 + up);
-  const long long t = (long long)(m >> (s > 63 ? 63 : s));
+  const long long t = (long long)fx_lsr(m, s);
   return ((t ^ sg) + 1) >> 1;
 }
 FXD long long fx_decode_df(unsigned long long bits, int E, int up = kFxUp) {
@@ -354,10 +374,10 @@ FXD int fx_top_bit(cfx p, int d) {
 // The product at the lane's scale, where the largest one (top bit T) has 57 bits; rounded to nearest (a tie goes up,
 // which happens to values whose own last bit is the dropped one).
 constexpr int kFxAligned = 57;
-FXD long long fx_align1(long long p, int l, int r) { return (((p << l) >> r) + 1) >> 1; }
+FXD long long fx_align1(long long p, int l, int r) { return (fx_asr(p << l, r) + 1) >> 1; }
 FXD cfx fx_align(cfx p, int d, int T) {
   const int n = kFxAligned + kFxGreenRange - T - d;
-  const int l = n < 0 ? 1 : n + 1, r = n < 0 ? (n < -62 ? 62 : -n) : 0;
+  const int l = n < 0 ? 1 : n + 1, r = n < 0 ? -n : 0;
   return fx_make(fx_align1(p.x, l, r), fx_align1(p.y, l, r));
 }
 // x g = aligned value times 2 to this
