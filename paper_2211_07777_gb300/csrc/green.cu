@@ -554,8 +554,13 @@ __global__ void __launch_bounds__(256) k_green_top(const double* __restrict__ g,
   int m = 0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     m = max(m, (__double2hiint(g[i] * scale) >> 20) & 0x7ff);
+  __shared__ int top;
+  if (threadIdx.x == 0) top = 0;
+  __syncthreads();
   m = __reduce_max_sync(0xffffffffu, m);
-  if ((threadIdx.x & 31) == 0) atomicMax(ref, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(&top, m);
+  __syncthreads();
+  if (threadIdx.x == 0) atomicMax(ref, top);  // one per block: all of them meet at one address
 }
 __global__ void k_green_finalize_fx(const double* __restrict__ g, unsigned long long* __restrict__ out,
                                     const int* __restrict__ ref, long long n, int gx, int gp, double scale) {
@@ -658,7 +663,7 @@ cudaError_t launch_green_finalize_fx(const double* g, void* out, int* ref, long 
   const long long blocks = std::min<long long>((n + 255) / 256, 152 * 16);
   const cudaError_t e = cudaMemsetAsync(ref, 0, sizeof(int), st);
   if (e) return e;
-  k_green_top<<<(unsigned)blocks, 256, 0, st>>>(g, ref, n, scale);
+  k_green_top<<<(unsigned)std::min<long long>(blocks, 152 * 4), 256, 0, st>>>(g, ref, n, scale);
   k_green_finalize_fx<<<(unsigned)blocks, 256, 0, st>>>(g, (unsigned long long*)out, ref, n, gx, gp, scale);
   return cudaGetLastError();
 }

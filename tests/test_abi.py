@@ -146,6 +146,9 @@ def test_closing_a_solver_waits_for_the_streams_of_its_solves(lib, monkeypatch):
         def __init__(self, handle):
             self.cuda_stream = handle
 
+        def query(self):
+            return False
+
         def synchronize(self):
             log.append(("wait", self.cuda_stream))
 
