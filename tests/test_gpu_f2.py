@@ -63,14 +63,30 @@ def test_unaligned_arrays_give_the_same_bits(bcs, off):
         assert torch.equal(b, want)
 
 
-def test_non_finite_pencils_stay_apart_from_the_padding():
-    """Odd x extents: the rows' padding in the workspace takes no part in the last pencil's packing."""
-    n = (9, 16, 12)
-    f = np.random.default_rng(4).standard_normal((12, 16, 9))
-    bcs = ((E, E), (PER, PER), (PER, PER))
-    h = (1 / 16,) * 3
-    L = tuple(v / 16 for v in n)
-    ref = oracle.solve(f, oracle.Problem(bc=bcs, h=h, center=CELL, kernel="spectral"))
-    for _ in range(3):
-        out, _ = cuda_solve(f, bcs, CELL, F.F32, "spectral", L=L, h=h)
-        assert rel_linf(out, ref) < TOL
+@pytest.mark.parametrize("bcs", [((E, E), (PER, PER), (PER, PER)), ((U, U), (O, O), (E, E)), ((PER, PER), (E, O), (U, U))],
+                         ids=["x-first", "open-x", "y-first"])
+@pytest.mark.parametrize("nx", [9, 18, 27])
+def test_the_last_group_takes_nothing_from_the_padding(nx, bcs):
+    """Odd row lengths in the workspace: their padding, NaN before the solve, lies beside the last packed pencils."""
+    import torch
+    n = (nx, 16, 12)
+    f = np.random.default_rng(4).standard_normal(n[::-1])
+    h = (1 / 27,) * 3
+    L = tuple(v / 27 for v in n)
+    kernel = "hej2" if any(U in b for b in bcs) else "spectral"
+    ref = oracle.solve(f, oracle.Problem(bc=bcs, h=h, center=CELL, kernel=kernel))
+    t = F.flups_init_topo(n, CELL, 1, F.F32)
+    s = F.flups_init_solver(t, bcs, h, L, kernel)
+    try:
+        F.flups_setup_shared(s)
+        ws = torch.full((F.flups_workspace_size(s) // 4,), float("nan"), device="cuda")
+        rhs = torch.from_numpy(f).float().cuda()
+        phi = torch.empty_like(rhs)
+        F.flups_solve_ws(s, phi, rhs, ws)
+        torch.cuda.synchronize()
+        got = phi.double().cpu().numpy()
+    finally:
+        torch.cuda.synchronize()
+        F.flups_cleanup(s)
+        F.flups_topo_free(t)
+    assert np.isfinite(got).all() and rel_linf(got, ref) < TOL, rel_linf(got, ref)

@@ -155,10 +155,16 @@ def test_both_fp64_precisions_run_the_same_passes():
 def test_sizes_around_the_line_match_the_oracle(n, prec):
     f = np.random.default_rng(sum(n)).standard_normal(n[::-1])
     h = (1.0 / max(n),) * 3
-    got = cuda_solve(f, ((PER, PER),) * 3, CELL, prec, "spectral", h=h, L=tuple(v * h[0] for v in n))[0]
-    ref = oracle.solve(f, oracle.Problem(bc=((PER, PER),) * 3, h=h, center=CELL, kernel="spectral"))
-    # double-float passes (at most 15 butterfly levels of 2u, u = 2^-48, per direction and way) bound the pair
-    assert np.linalg.norm(got - ref) < 6 * 15 * 2.0 ** -47 * np.linalg.norm(ref)
+    bcs, L = ((PER, PER),) * 3, tuple(v * h[0] for v in n)
+    got = cuda_solve(f, bcs, CELL, prec, "spectral", h=h, L=L)[0]
+    ref = oracle.solve(f, oracle.Problem(bc=bcs, h=h, center=CELL, kernel="spectral"))
+    with F.Solver(n, bcs, L=L, h=h, prec=prec) as s:
+        fixed = [x["fixed_point"] for x in s.features()]
+    assert all(fixed) or not any(fixed)
+    # FP64 and fixed point: six transforms' rounding, 1e-14; double-float passes: at most 15 butterfly levels of 2u,
+    # u = 2^-48, per direction and way
+    bound = 1e-14 if prec == F.F64 or fixed[0] else 6 * 15 * 2.0 ** -47
+    assert np.linalg.norm(got - ref) < bound * np.linalg.norm(ref)
 
 
 # Below the line, three components fill the device in short FP64 tiles along y (64 points between walls: runtime tiles)
