@@ -145,12 +145,18 @@ def _stream(s) -> int:
     return s.cuda_stream
 
 
+_DEFAULT_STREAMS = {}  # the legacy default stream of each device (a stream object costs 20 us to make)
+
+
 def _held(stream):
     """The stream as an object that can be waited for later (None: the current device's legacy default stream)."""
-    if stream is None:
-        import torch
-        return torch.cuda.default_stream()
-    return stream
+    if stream is not None:
+        return stream
+    import torch
+    device = torch.cuda.current_device()
+    if device not in _DEFAULT_STREAMS:
+        _DEFAULT_STREAMS[device] = torch.cuda.default_stream(device)
+    return _DEFAULT_STREAMS[device]
 
 
 def _wait(stream):
