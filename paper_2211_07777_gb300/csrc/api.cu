@@ -1046,15 +1046,20 @@ void set_rows_bulk(Launch& L, int prec) {
 
 // FP32 passes on pairs of lanes in packed arithmetic (f2_passes.cu) or on the kernels of pass_kernels.cuh, by
 // measurement on GB300 (us per pass, old / lane pairs):
-// - lengths with a factor 3, which had only the runtime-shaped tiles: always (192^3: 473 / 238 fused, 104 / 59
-//   complex, 150-200 / 60-75 symmetric; 48^3 fused 16 / 14);
-// - the Biot-Savart pass: always (128^3: 191 / 102 with an open axis, 59 / 50 periodic, 148 / 76 symmetric);
-// - powers of two: real passes along y or z (256-point periodic 78 / 64 and 76 / 53) and symmetric ones along
-//   x (512 points: 90 / 86 and 123 / 82); x passes of periodic and unbounded data where the grid is too small for the
-//   compile-time tiles (128^3 periodic 20 / 12 and 23 / 16; with those tiles 27 / 37 and 21 / 42 on three
-//   components), the forward one also at 512 points (366 / 342);
-// - complex passes of powers of two: never (256 points 14 / 16, fused 31 / 47; 1024 points fused 1912 / 3077): the
-//   column kernels prefetch their tiles by TMA and hold twice the warps.
+// - lengths with a factor 3, which had only the runtime-shaped tiles: always (open 192^3: real 98 / 34 and 123 / 61,
+//   complex 105 / 63 and 125 / 59, fused 473 / 174; walls 192^3 86-188 / 33-66; open 48^3 fused 16 / 10, its inverse
+//   real pass 8 / 10);
+// - the Biot-Savart pass where its tiles fit a CTA (128^3: open 346 / 209, over a wall 184 / 100, periodic 55 / 49,
+//   walls 141 / 78);
+// - powers of two: real passes along y or z (256 cells, periodic: 62 / 40 and 61 / 45 of the caller's data, 60 / 39 and
+//   61 / 45 after a walled direction), symmetric ones (along x 86 / 75 and 119 / 78, fused 176 / 145);
+// - x passes of periodic and unbounded data in powers of two: where the grid is too small for the compile-time tiles;
+//   with those, on 256 x 256 rows of periodic data (open domains have the same order per length), forward 27 / 44,
+//   49 / 54, 101 / 90, 157 / 185 and inverse 25 / 43, 45 / 78, 125 / 141, 139 / 293 at 128, 256, 512 and 1024 points:
+//   only the forward pass of 512 points gains, whose old tile has 512 threads behind one barrier (half of that at 256
+//   points; from 1024 points on 4-lane tiles in registers), on every number of rows (64 x 64 to 512 x 256: 1.02-1.20);
+// - complex passes of powers of two: never (256 points 14 / 17, fused 28 / 51; 1024 points 699 / 1234, fused
+//   1844 / 4399): the column kernels prefetch their tiles by TMA and hold twice the warps.
 bool use_f2(const flups_solver_s* s, const Launch& L, const DirPlan& dp, int axis) {
   if (s->topo.prec != FLUPS_F32) return false;
   const int P = dp.P;

@@ -3,8 +3,9 @@
 //
 // A CTA holds W lanes x P values of 16 bytes in shared memory, a value being one position of two complex
 // sequences: two neighbouring pencils of a complex pass, or four real pencils q .. q + 3 packed as
-// q + i (q + 2) and (q + 1) + i (q + 3).  The tile is transformed in place, whole butterflies of up to 9 values in
-// registers between two barriers; complex passes and the real passes of periodic and unbounded directions
+// q + i (q + 2) and (q + 1) + i (q + 3).  The tile is transformed in place, whole butterflies in registers between two
+// barriers (one of up to 9 values a thread where three such stages make the length, else, and in the Biot-Savart pass,
+// up to 18 values: fx_plan.cuh); complex passes and the real passes of periodic and unbounded directions
 // read the first stage's inputs from memory and store the last stage's outputs from registers.
 #pragma once
 #include <cuda_runtime.h>

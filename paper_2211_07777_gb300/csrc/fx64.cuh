@@ -13,7 +13,9 @@
 // so no value passes 2^62.5, and none 2^61.5 where two values are added before the next scaling.  The unit in
 // the last place is 2^-57 of the lane's largest input: 16 times finer than the FP64 spacing at that value;
 // lanes whose values do not grow are shifted up between stages (fx_kernels.cuh), so the coarsest rounding is
-// the final one to FP64.  Infinite or NaN inputs make every value of their lane NaN.
+// the final one to FP64.  Values below 2^-4 of the lane's largest input hold less than FP64's 53 bits, and what lies below
+// 2^-58 of it is lost: an error of each pass against its lane's largest value, where FP64's sums may also cancel
+// exactly.  Infinite or NaN inputs make every value of their lane NaN.
 //
 // Products.  x = xh 2^32 + xl with both halves signed (|xl| <= 2^31), w likewise; (x w) >> 64 takes
 // xh wh and the upper part of xh wl + xl wh and drops xl wl, which is below one unit.  |xh wl| <= 2^30.5 2^31
@@ -72,7 +74,7 @@ FXD cfx fx_sub(cfx a, cfx b) { return fx_make(a.x - b.x, a.y - b.y); }
 // times -i (forward) or +i (inverse)
 template <bool INV> FXD cfx fx_mi(cfx a) { return INV ? fx_make(-a.y, a.x) : fx_make(a.y, -a.x); }
 
-// Every shift rounds to nearest: a truncation's mean error of half a unit is the same at every position, and
+// Every shift rounds to nearest, decoding too: a truncation's mean error of half a unit is the same at every position, and
 // a constant over the modes is a peak P times higher at the first point after the inverse transform (measured
 // with truncation at 256^3: 1.3e-12 relative instead of 4e-16).  The half unit starts the multiply-add chain.
 constexpr long long kFxHalf32 = 1LL << 31;

@@ -1,5 +1,6 @@
-// Passes of the FP64-class Poisson solves (FP64 arrays in and out) in 64-bit block fixed point
-// (fx64.cuh): one kernel per pass kind and length P = 2^a 3^b, for every axis and tile width.
+// FP64-class passes (FP64 arrays in and out) in 64-bit block fixed point (fx64.cuh): all five of a Poisson solve, the
+// four around the curl of a Biot-Savart solve (whose own array is double-float on FP64E), and the DCT-I of every
+// precision's Green spectrum.  One kernel per pass kind and length P = 2^a 3^b, for every axis and tile width.
 //
 // A CTA holds W lanes (pencils; two packed real pencils per lane for real data) x P complex values
 // in shared memory and transforms them in place: a thread takes whole butterflies of up to 18 values in

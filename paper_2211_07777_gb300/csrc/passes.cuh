@@ -116,7 +116,7 @@ cudaError_t launch_ct_f32(int P, int kind, const PassParams& p, dim3 grid, int n
 cudaError_t launch_ct_f64(int P, int kind, const PassParams& p, dim3 grid, int nthr, size_t smem, cudaStream_t st);
 cudaError_t set_limits_ct_f32();
 cudaError_t set_limits_ct_f64();
-// FP64-class Poisson passes in 64-bit block fixed point
+// FP64-class passes in 64-bit block fixed point
 cudaError_t launch_fx(int kind, const PassParams& p, dim3 grid, int nthr, size_t smem, cudaStream_t st);
 // shared-memory limit of the kernel of that kind and length (per device, set when a plan is made)
 cudaError_t limit_fx(int kind, int P);
