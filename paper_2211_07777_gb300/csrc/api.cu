@@ -1391,11 +1391,12 @@ int flups_init_solver(flups_topo t, const int* bc, const double h[3], const doub
   if (rc == FLUPS_OK) rc = build_plan(s);
   // FP64-class solves run in 64-bit fixed point, except the smallest, where a pass is one warp's chain of
   // instructions and the short columns of the warp engine are as fast or faster.  Measured, us per solve without / with
-  // fixed point, by points of the extension: FP64 periodic 16^3 22.4 / 24.0, 27^3 34.4 / 35.3, 32^3 25.8 / 25.7, 32 x 32
-  // x 36 31.4 / 25.1, open 18^3 (46656) 36.9 / 22.8, walls and open 16^3 (65536) 39.0 / 34.3, Biot-Savart periodic 36^3
-  // 73.8 / 51.2.  The double-float passes are faster than the FP64 ones: 32 x 32 x 36 (36864) 24.6 / 25.0, periodic 36^3
-  // 32.0 / 24.1, open 18^3 29.4 / 22.8, but in powers of two, whose columns stay in registers, walls and open 16^3
-  // 30.6 / 34.3; around their curl Biot-Savart at 8 x 8 x 972 127 / 148.
+  // fixed point, by points of the extension: FP64 periodic 16^3 22.4 / 24.2, 27^3 34.4 / 36.6, 32^3 (32768) 25.8 / 26.7,
+  // 32 x 32 x 36 31.4 / 25.9, open 18^3 (46656) 36.9 / 23.7, Biot-Savart periodic 36^3 73.8 / 51.3.  The double-float
+  // passes are faster than the FP64 ones: 12 x 12 x 243 (34992) 31.0 / 37.7, 32 x 32 x 36 (36864) 24.3 / 25.9, open 18^3
+  // 29.2 / 23.6, periodic 36^3 31.9 / 24.8, and in powers of two, whose columns stay in registers, open 16^3 (32768)
+  // 19.9 / 26.1, walls and open 16^3 (65536) 30.6 / 34.3.  Biot-Savart keeps its line at 65536 since the curl converted
+  // FP64 arrays itself; around double-float arrays fixed point would gain earlier (36^3 51.2 / 43.0, 8 x 8 x 972 129 / 121).
   {
     bool pow2 = true;
     for (int d = 0; d < 3; ++d) pow2 &= (s->dir[d].P & (s->dir[d].P - 1)) == 0;
