@@ -323,8 +323,8 @@ FXD long long fx_decode(unsigned long long bits, int E, int up = kFxUp) {
 
 // The same for a double-float value hi + lo (hi in the lower word): both floats aligned and rounded to nearest.
 FXD long long fx_decode_float(unsigned w, int E, int up) {
-  const int e = (int)(w >> 23) & 255, sg = (int)w >> 31, s = E - e - 896;
-  const unsigned long long m = (unsigned long long)(e ? (w & 0x7fffffu) | 0x800000u : 0) << (30 + up);
+  const int e = (int)(w >> 23) & 255, sg = (int)w >> 31, s = E - (e ? e : 1) - 896;
+  const unsigned long long m = (unsigned long long)((w & 0x7fffffu) | (e ? 0x800000u : 0)) << (30 + up);
   const long long t = (long long)fx_lsr(m, s);
   return ((t ^ sg) + 1) >> 1;
 }
@@ -334,7 +334,7 @@ FXD long long fx_decode_df(unsigned long long bits, int E, int up = kFxUp) {
 // FP64's biased exponent of the larger float of a double-float value, from its bits without the sign
 FXD int fx_float_exp(unsigned w) {
   const int e = (int)(w >> 23);
-  return e == 0 ? 0 : (e == 255 ? 2047 : e + 896);
+  return w == 0 ? 0 : (e == 255 ? 2047 : (e ? e : 1) + 896);
 }
 
 // Green factors keep FP64's 53 bits and an exponent each: a pencil's factors fall by many orders of magnitude (1/k^2,

@@ -101,6 +101,10 @@ int main() {
     wdf = std::fmax(wdf, std::fabs(ldexpl((ld)hi + lo, kFxBias - E) - (ld)fx_decode_df(b, E)));
     if (fx_float_exp(wh & 0x7fffffffu) > E) return 13;
   }
+  // subnormal floats: 2^-126 as the lane's largest beside 2^-140 and 2^-149
+  if (fx_float_exp(0x00400000u) != 897 || fx_decode_df(0x00000001u, 897) != 1LL << (kFxUp + 29) ||
+      fx_decode_df(0x8000020000800000ull, 897) != (1LL << (kFxUp + 52)) - (1LL << (kFxUp + 38)))
+    return 17;
   if (fx_decode_df(0, kFxMinE) != 0 || fx_float_exp(0) != 0 || fx_float_exp(0x7f800000u) != 2047) return 14;
   std::printf("decode_df %.3Lg\n", wdf);
   // Green products: factors over 60 binary orders with modes over 60, the larger product of a pair aligned to 57 bits

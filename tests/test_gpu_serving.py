@@ -129,7 +129,10 @@ def test_double_float_engine_in_the_mix_matches_native_fp64():
     ((64, 32, 27), ((F.PER, F.PER),) * 3, F.HEJ4),
     ((32, 48, 36), ((F.EVEN, F.ODD), (F.ODD, F.ODD), (F.EVEN, F.EVEN)), F.SPECTRAL),
     ((32, 24, 27), ((F.EVEN, F.EVEN), (F.ODD, F.ODD), (F.ODD, F.EVEN)), F.HEJ2),
-], ids=["complex", "complex-hej4", "real", "quarter-hej2"])
+    ((48, 36, 32), ((F.PER, F.PER), (F.EVEN, F.EVEN), (F.ODD, F.ODD)), F.SPECTRAL),
+    ((32, 48, 36), ((F.ODD, F.ODD), (F.PER, F.PER), (F.EVEN, F.ODD)), F.SPECTRAL),
+    ((48, 64, 24), ((F.PER, F.PER), (F.PER, F.PER), (F.EVEN, F.EVEN)), F.SPECTRAL),
+], ids=["complex", "complex-hej4", "real", "quarter-hej2", "real-x", "real-y", "complex-y"])
 def test_a_fully_spectral_plan_runs_in_the_memory_without_its_spectrum(n, bc, kernel):
     """A budget for the workspace, the arrays and the tables alone: the request is taken, its factors are evaluated in
     the pass, and the solution is the one with the stored spectrum to the factors' rounding."""
